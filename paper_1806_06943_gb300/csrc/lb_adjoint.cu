@@ -278,7 +278,7 @@ __global__ void k_adj_density(const Lat<double> L, const double *__restrict__ f,
     for (int k = 0; k < 2; ++k) {
         double v[9];
         for (int i = 0; i < 9; ++i) v[i] = f[(size_t)(k * 9 + i) * L.plane + c];
-        rho[(size_t)k * L.plane + c] = zeroth_moment<double>(v);
+        rho[(size_t)k * L.plane + c] = zeroth_moment<double>(v, L.one);
     }
 }
 

@@ -107,6 +107,12 @@ void fill_lat(lbk::Lat<real> &L, const lb_params &p)
     L.G1 = (real)p.G1;
     L.G2 = (real)p.G2;
     L.GAB = (real)p.G_AB;
+    L.one = (real)1;
+    const double factors[] = {p.G1, p.G2, p.G_AB, p.g[0], p.g[1], 1.0 / p.tau[0], 1.0 / p.tau[1],
+                              1.0 - 0.5 / p.tau[0], 1.0 - 0.5 / p.tau[1]};
+    L.products = 1;
+    for (double v : factors)
+        if (v != 0.0 && (std::fabs(v) < 0x1p-58 || std::fabs(v) >= 0x1p64)) L.products = 0;
     // the combined psi-sum weights of Eq. (8) on the inner ring,
     // c(|e|^2) = G1 w(|e|^2) + G2 p(|e|^2) for |e|^2 = 1, 2, and G2 for the
     // outer ring, negated
@@ -1202,6 +1208,8 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
     }
     // time-step tiles for every supported tile height, and the persistent
     // launch's control block and error word
+    if ((ce = e->precision == LB_FP64 ? lbk::Launch<double>::prepare() : lbk::Launch<float>::prepare()) != cudaSuccess)
+        return bail(cuda_fail(ce, "shared memory of the step kernels"));
     for (int ti = 0; ti < 3; ++ti) {
         const int tyv = kTileHeights[ti];
         std::vector<int> counts(n, 0);

@@ -1,0 +1,119 @@
+// lb_f64.cuh -- FP64 arithmetic of the plain step, arranged for a chip whose
+// FP64 pipe is its narrowest part.
+//
+// A GB300 SM starts one FP64 warp instruction every 16 to 19 clocks (2 lanes)
+// against 4 instructions of every other kind per clock, so the plain FP64 step
+// is bound by the number of its FP64 instructions and nothing else.  What is
+// measured on the device (clocks an SM spends per warp instruction):
+//   fma with three register operands                       16.0
+//   add, multiply, fma with a constant operand              19.0
+//   product by the integer routine below, alone             16.1
+//   add + multiply 40.1, add + integer product              22.8
+// The step therefore keeps only sums on the FP64 pipe, each written as an fma
+// with the factor 1 in a register (exact: one rounding, as the add), and forms
+// its products in integer instructions, which run beside them.  Every result
+// has the bits of the IEEE operation it stands for, so the step still rounds
+// as a plain evaluation of the equations, operation by operation.  With the
+// products shared between neighbours (Stage64) a node of the one-pass step
+// costs 380 FP64 instructions instead of 641; a 1024^2 step 0.78 ms instead
+// of 1.30, its FP64 pipe busy throughout.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace lbk {
+
+// A factor of an integer product: sign and exponent bits, the 53-bit mantissa
+// as (21, 32) bits, and whether it is zero.
+struct Factor {
+    uint32_t se, m1, m0;
+    bool zero;
+};
+
+__device__ __forceinline__ Factor factor(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    Factor f;
+    f.zero = ((hi & 0x7fffffffu) | lo) == 0u;
+    f.se = hi & 0xfff00000u;
+    f.m1 = (hi & 0x000fffffu) | 0x00100000u;
+    f.m0 = lo;
+    return f;
+}
+
+// The IEEE product (round to nearest even) of two factors that are zero or
+// normal, where the product is zero or normal too.  The second mantissa is
+// aligned to the top of 64 bits, so the upper half H of the 117-bit product
+// has 52 or 53 bits; one conditional shift normalises it, the lower half
+// decides the rounding, and a carry out of the mantissa runs into the
+// exponent by itself.  Signs add up in the top bit.
+__device__ __forceinline__ double factor_mul(const Factor &a, const Factor &b)
+{
+    const uint32_t b1 = (b.m1 << 11) | (b.m0 >> 21), b0 = b.m0 << 11;
+    const uint64_t p00 = (uint64_t)a.m0 * b0;
+    const uint64_t t = (uint64_t)a.m0 * b1 + (p00 >> 32);
+    const uint64_t v = (uint64_t)a.m1 * b0 + (uint32_t)t;
+    const uint64_t H = (uint64_t)a.m1 * b1 + (t >> 32) + (v >> 32);
+    uint32_t hh = (uint32_t)(H >> 32), hl = (uint32_t)H, lh = (uint32_t)v;
+    const uint32_t lost = (uint32_t)p00;
+    const uint32_t short_bit = ~hh & 0x00100000u, n = short_bit >> 20;   // 1: H has 52 bits
+    hh = __funnelshift_l(hl, hh, n);
+    hl = __funnelshift_l(lh, hl, n);
+    lh = __funnelshift_l(lost, lh, n);
+    const uint32_t top = hh + (a.se + b.se - 0x3ff00000u - short_bit);
+    uint32_t rl, rh;
+    // up where the discarded part lh:lost is above one half, or one half and
+    // H odd: the carry of lh + 0x7fffffff + (1 if H is odd or lost is not 0)
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %2, 0xffffffff;\n\t"
+        "addc.cc.u32 t, %3, 0x7fffffff;\n\t"
+        "addc.cc.u32 %0, %4, 0;\n\t"
+        "addc.u32 %1, %5, 0;\n\t}"
+        : "=r"(rl), "=r"(rh)
+        : "r"(lost | (hl & 1u)), "r"(lh), "r"(hl), "r"(top));
+    const bool z = a.zero || b.zero;
+    return __hiloint2double((int)(z ? (a.se ^ b.se) & 0x80000000u : rh), (int)(z ? 0u : rl));
+}
+
+// Where the node's products are formed, every factor and every product is
+// zero or normal, provided that
+//   the populations, densities and psi it reads are zero or in
+//     [2^-179, 2^77) (base_outside() is 0),
+//   the couplings, relaxation rates and body forces are zero or in
+//     [2^-64, 2^64) (checked on the host: Lat::products), and
+//   the velocity's components are zero or in [2^-255, 2^256)
+//     (velocity_outside() is 0).
+// A nonzero sum is at least 2^-53 times its smallest term, so stencil sums
+// are above 2^-250, forces above 2^-550, the Guo vectors above 2^-310, their
+// products with the force above 2^-920 and with (1 - omega/2) w above
+// 2^-980; the largest magnitudes stay below 2^700.
+__device__ __forceinline__ uint32_t base_outside(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    // exponent fields 0x34c .. 0x44b, moved down, leave the top three bits clear
+    return (((hi & 0x7fffffffu) | lo) == 0u) ? 0u : (hi - 0x34c00000u) & 0x70000000u;
+}
+__device__ __forceinline__ uint32_t velocity_outside(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    // exponent fields 0x300 .. 0x4ff, moved up by 0x100, have top bits 10
+    return (((hi & 0x7fffffffu) | lo) == 0u) ? 0u : ((hi + 0x10000000u) ^ 0x40000000u) & 0x60000000u;
+}
+
+// Arithmetic of a node: sums as register fmas, products by factor_mul (kInt)
+// or the FP64 pipe (the same bits).
+template <bool kInt>
+struct Arith64 {
+    double one;   // 1.0, in a register the compiler knows nothing about
+    __device__ __forceinline__ explicit Arith64(double one_) : one(one_) {}
+    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(-b, one, a); }
+    __device__ __forceinline__ double mul(double a, double b) const
+    {
+        if constexpr (kInt) return factor_mul(factor(a), factor(b));
+        else return __dmul_rn(a, b);
+    }
+};
+
+}  // namespace lbk

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "lb_f64.cuh"
 #include "lb_types.h"
 #include "lb_vops.cuh"
 
@@ -50,7 +51,9 @@ constexpr bool kOffset = sizeof(real) == 4;
 
 // Resident blocks per SM the fused kernel is compiled for: the FP32 kernel is
 // bound by HBM and needs the warps to keep enough loads in flight; the FP64
-// kernel is bound by the FP64 pipe and keeps its registers.
+// kernel is bound by the FP64 pipe, which 16 warps fill (8 warps without a
+// spill and 24 with 540 bytes of it measured 5 % and 1 % slower on a 1024^2
+// lattice).
 template <typename real, int TYv>
 constexpr int kCollideMinBlocks = (kOffset<real> ? 32 : 16) / TYv;
 
@@ -208,19 +211,12 @@ __device__ __forceinline__ void force_at(const Lat<real> &L, const real (*srho)[
 }
 
 // The staged density and psi tiles of the species as one [row][col] plane
-// per species and field, as collide_site reads them: species k's density
-// and force at a staged node, and rho_k(x) - rho_k(x + e), the difference a
-// push re-references with.  collide_site asks for species 0, then 1.
-template <typename real, int SHv>
+// per species and field, as the FP32 collide_site reads them: both species'
+// forces and densities at a staged node as (A, B) pairs.
+template <int SHv>
 struct SplitStage {
-    const real (*srho)[SHv][SW];
-    const real (*spsi)[SHv][SW];
-    __device__ __forceinline__ real density(int k, int cy, int cx) const { return srho[k][cy][cx]; }
-    __device__ __forceinline__ void force(const Lat<real> &L, int k, int cx, int cy, real &Fx, real &Fy) const
-    {
-        force_at<real, SHv>(L, srho, spsi, k, cx, cy, Fx, Fy);
-    }
-    // FP32: both species' forces and densities as (A, B) pairs
+    const float (*srho)[SHv][SW];
+    const float (*spsi)[SHv][SW];
     __device__ __forceinline__ void force2(const Lat<float> &L, int cx, int cy, float2 &Fx, float2 &Fy) const
     {
         force_at<float, SHv>(L, srho, spsi, 0, cx, cy, Fx.x, Fy.x);
@@ -230,12 +226,7 @@ struct SplitStage {
     {
         return make_float2(srho[0][cy][cx], srho[1][cy][cx]);
     }
-    template <int EX, int EY>
-    __device__ __forceinline__ real density_step(int k, int cx, int cy) const
-    {
-        return srho[k][cy][cx] - srho[k][cy + EY][cx + EX];
-    }
-    // FP32: both species' densities at the staged node (cx + EX, cy + EY)
+    // both species' densities at the staged node (cx + EX, cy + EY)
     template <int EX, int EY>
     __device__ __forceinline__ float2 dest(int cx, int cy) const
     {
@@ -253,83 +244,30 @@ __device__ __forceinline__ real edot(real ux, real uy)
     else return (EX > 0 ? ux : -ux) + (EY > 0 ? uy : -uy);
 }
 
-// (e_a - u_a)/cs^2 + (e.u) e_a / cs^4 for one component a.
-template <typename real, int E>
-__device__ __forceinline__ real guo_comp(real u, real eu)
-{
-    if constexpr (E == 0) return -((real)3 * u);
-    else if constexpr (E > 0) return (real)3 * ((real)1 - u) + (real)9 * eu;
-    else return (real)3 * ((real)-1 - u) - (real)9 * eu;
-}
-
-// BGK relaxation with Guo forcing for direction I of one species
-// (Eqs. 1, 2, 5).  FP64: f -> f*.  FP32: the offset from the node's own
-// density, f - w rho -> f* - w rho (its equilibrium is w rho (e.u terms)).
-template <typename real, int I>
-__device__ __forceinline__ real collide_dir(real f, real rho, real ux, real uy, real uu, real Fx, real Fy, real om,
-                                            real aw)
-{
-    constexpr int EX = ex9(I), EY = ey9(I);
-    const real w = (real)w9(I);
-    const real eu = edot<real, EX, EY>(ux, uy);
-    const real C = aw * (guo_comp<real, EX>(ux, eu) * Fx + guo_comp<real, EY>(uy, eu) * Fy);
-    const real feq = w * rho * ((real)1 + (real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu);
-    return f - om * (f - feq) + C;
-}
-
 // Store the post-collision value of direction I of species k at x + e_i
-// (half-way bounce-back: back to x, reversed).  FP32: re-reference the offset
-// from rho(x) to rho(x + e_i), the reference the next step reads there
-// (unless kReref is false: the caller did).
-template <typename real, int I, bool kInner, class Stage, bool kReref = true>
-__device__ __forceinline__ void push_dir(const Lat<real> &L, real *__restrict__ fn, const Stage &sg, int k, int x,
-                                         int y, int cx, int cy, real v)
+// (half-way bounce-back: back to x, reversed) near an edge of the lattice.
+template <int I>
+__device__ __forceinline__ void push_edge(const Lat<float> &L, float *__restrict__ fn, int k, int x, int y, float v)
 {
     constexpr int EX = ex9(I), EY = ey9(I);
-    if constexpr (kOffset<real> && kReref && I != 0) {
-        // the next step's reference at the destination is its density now
-        if (kInner || !(EY != 0 && L.walls && (y + EY < 0 || y + EY >= L.ny)))
-            v = cfma((float)w9(I), sg.template density_step<EX, EY>(k, cx, cy), v);
+    int xd = x + EX, yd = y + EY;
+    if constexpr (EX != 0) {
+        if (xd >= L.nx) xd -= L.nx;
+        if (xd < 0) xd += L.nx;
     }
-    if constexpr (kInner) {
-        // node and destination inside the lattice: a constant offset
-        fn[(size_t)(k * 9 + I) * L.plane + ((size_t)y * L.pitch + x) + (EY * L.pitch + EX)] = v;
-        return;
-    } else {
-        int xd = x + EX, yd = y + EY;
-        if constexpr (EX != 0) {
-            if (xd >= L.nx) xd -= L.nx;
-            if (xd < 0) xd += L.nx;
-        }
-        int dir = I;
-        if constexpr (EY != 0) {
-            if (yd < 0 || yd >= L.ny) {
-                if (L.walls) {       // half-way bounce-back: back to this node, reversed
-                    dir = opp9(I);
-                    xd = x;
-                    yd = y;
-                } else {
-                    yd = yd < 0 ? yd + L.ny : yd - L.ny;
-                }
+    int dir = I;
+    if constexpr (EY != 0) {
+        if (yd < 0 || yd >= L.ny) {
+            if (L.walls) {       // half-way bounce-back: back to this node, reversed
+                dir = opp9(I);
+                xd = x;
+                yd = y;
+            } else {
+                yd = yd < 0 ? yd + L.ny : yd - L.ny;
             }
         }
-        fn[(size_t)(k * 9 + dir) * L.plane + (size_t)yd * L.pitch + xd] = v;
     }
-}
-
-// Collision and push of direction I of both species (FP64), fk the node's
-// populations; sg the staged densities.
-template <typename real, int I, bool kInner, class Stage>
-__device__ __forceinline__ void collide_push_dir(const Lat<real> &L, real *__restrict__ fn, const Stage &sg,
-                                                 const real (&fk)[2][9], const real (&rho)[2], real ux, real uy,
-                                                 real uu, const real (&F)[2][2], int x, int y, int cx, int cy)
-{
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const real v = collide_dir<real, I>(fk[k][I], rho[k], ux, uy, uu, F[k][0], F[k][1], L.omega[k],
-                                            L.aw[k][cls9(I)]);
-        push_dir<real, I, kInner>(L, fn, sg, k, x, y, cx, cy, v);
-    }
+    fn[(size_t)(k * 9 + dir) * L.plane + (size_t)yd * L.pitch + xd] = v;
 }
 
 // Species momentum sum_i f e_i.  FP64: direction order, zero products
@@ -345,12 +283,19 @@ __device__ __forceinline__ void first_moment(const real (&f)[9], real &jx, real 
     }
 }
 
+// sum_i f_i.  FP64: direction order, as fmas with the factor `one` = 1
+// (lb_f64.cuh).
 template <typename real>
-__device__ __forceinline__ real zeroth_moment(const real (&f)[9])
+__device__ __forceinline__ real zeroth_moment(const real (&f)[9], real one)
 {
     if constexpr (!kOffset<real>) {
-        return (((((((f[0] + f[1]) + f[2]) + f[3]) + f[4]) + f[5]) + f[6]) + f[7]) + f[8];
+        const Arith64<false> A(one);
+        double r = f[0];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) r = A.add(r, f[i]);
+        return r;
     } else {
+        (void)one;
         return vzeroth<float>(f);
     }
 }
@@ -381,9 +326,12 @@ __device__ __forceinline__ void density_tile(const Lat<real> *__restrict__ lats,
         real v[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) v[i] = ldg_state<kCG>(&f[(size_t)(k * 9 + i) * L.plane + c]);
-        real r = zeroth_moment<real>(v);
+        real r = zeroth_moment<real>(v, L.one);
         if constexpr (kOffset<real>) r = ldg_state<kCG>(&L.rho[parity][(size_t)k * L.plane + c]) + r;
         L.rho[parity ^ 1][(size_t)k * L.plane + c] = r;
+        // FP64 keeps no reference densities: copy parity holds psi, so that
+        // exp() runs once per node instead of once per staged slot
+        if constexpr (!kOffset<real>) L.rho[parity][(size_t)k * L.plane + c] = psi_of<real>(r);
     }
 }
 
@@ -394,12 +342,12 @@ __global__ void __launch_bounds__(TX *TYv) k_density(const Lat<real> *__restrict
     density_tile<real, TYv, false>(lats, tiles[tile_offset + blockIdx.x], parity);
 }
 
-// Shared memory of the fused kernel for a tile of height TYv.
-template <typename real, int TYv>
+// Shared memory of the FP32 step kernels for a tile of height TYv.
+template <int TYv>
 struct CollideSmem {
-    real srho[2][TYv + 2 * HALO][SW];
-    real spsi[2][TYv + 2 * HALO][SW];
-    Lat<real> L;   // descriptor copy: stores to the populations cannot alias it
+    float srho[2][TYv + 2 * HALO][SW];
+    float spsi[2][TYv + 2 * HALO][SW];
+    Lat<float> L;   // descriptor copy: stores to the populations cannot alias it
 };
 
 // Moments of a node's FP32 offset populations that need no force, as
@@ -411,96 +359,6 @@ struct NodeMoments {
     float2 delta;
     float2 dg;
 };
-
-template <typename real, bool kInner, bool kBox = false, class Stage>
-__device__ __forceinline__ void collide_site(const Lat<real> &L, real *__restrict__ fn, const Stage &sg,
-                                             real (&fk)[2][9], const real (&Rn)[2], int x, int y, int cx, int cy,
-                                             const real *__restrict__ box = nullptr, int box_plane = 0,
-                                             const NodeMoments *pre = nullptr);
-
-// Fused force + collision + push-streaming + bounce-back for one tile.  Every
-// thread of the block calls it and returns from it; it ends after the tile's
-// pushes are issued (the caller synchronises before reusing sm).
-template <typename real, int TYv, bool kCG>
-__device__ __forceinline__ void collide_tile(const Lat<real> *__restrict__ lats, int4 t, int parity,
-                                             CollideSmem<real, TYv> &sm)
-{
-    const Lat<real> &G = lats[t.x];
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    static_assert(sizeof(Lat<real>) % 4 == 0, "descriptor copied as 32-bit words");
-    for (int i = tid; i < (int)(sizeof(Lat<real>) / 4); i += TX * TYv)
-        reinterpret_cast<uint32_t *>(&sm.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
-    const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
-    const bool valid = x < G.nx && y < G.ny;
-    // issue the population loads first so their latency overlaps the staging
-    const real *__restrict__ fc = G.f[parity];
-    real *__restrict__ fn = G.f[parity ^ 1];
-    const size_t c = valid ? (size_t)y * G.pitch + x : 0;
-    real fk[2][9];
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (real)0;
-    if constexpr (kCG) {
-        // staging reads the density copy through L2 as well
-        constexpr int SHv = TYv + 2 * HALO;
-        const int nx = G.nx, ny = G.ny;
-        const real *__restrict__ rho = G.rho[parity ^ 1];
-        for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
-            const int sx = idx % SW, sy = idx / SW;
-            const int gx = wrap_index(t.y + sx - HALO, nx);
-            int gy = t.z + sy - HALO;
-            real rA, rB;
-            bool fixed = false;
-            if (gy < 0 || gy >= ny) {
-                if (G.walls) {
-                    if (G.wall_mode == 1) {
-                        rA = G.wall_rho[0];
-                        rB = G.wall_rho[1];
-                        fixed = true;
-                    } else {
-                        gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
-                        gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);
-                    }
-                } else {
-                    gy = wrap_index(gy, ny);
-                }
-            }
-            if (!fixed) {
-                const size_t cc = (size_t)gy * G.pitch + gx;
-                rA = __ldcg(&rho[cc]);
-                rB = __ldcg(&rho[G.plane + cc]);
-            }
-            sm.srho[0][sy][sx] = rA;
-            sm.srho[1][sy][sx] = rB;
-            sm.spsi[0][sy][sx] = psi_of<real>(rA);
-            sm.spsi[1][sy][sx] = psi_of<real>(rB);
-        }
-    } else {
-        stage_tile<real, TYv + 2 * HALO>(G, G.rho[parity ^ 1], t.y, t.z, sm.srho, sm.spsi, tid, TX * TYv);
-    }
-    __syncthreads();
-    if (!valid) return;
-    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
-    real Rn[2] = {(real)0, (real)0};
-    if constexpr (kOffset<real>) {
-        Rn[0] = ldg_state<kCG>(&G.rho[parity][c]);
-        Rn[1] = ldg_state<kCG>(&G.rho[parity][G.plane + c]);
-    }
-    // tiles whose pushes stay inside the lattice (no wrap, no wall) take constant offsets
-    const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
-    const SplitStage<real, TYv + 2 * HALO> sg{sm.srho, sm.spsi};
-    if (inner) collide_site<real, true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
-    else collide_site<real, false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
-}
-
-template <typename real, int TYv>
-__global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
-    k_collide(const Lat<real> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity)
-{
-    __shared__ CollideSmem<real, TYv> sm;
-    collide_tile<real, TYv, false>(lats, tiles[tile_offset + blockIdx.x], parity, sm);
-}
 
 // The NodeMoments of a node from its offset populations h (both species as
 // pairs), rho its densities and Rn its references: the same operations, in
@@ -529,60 +387,8 @@ __device__ __forceinline__ real feq_dir(real rho, real ux, real uy, real uu)
     return (real)w9(I) * rho * ((real)1 + (real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu);
 }
 
-// BGK relaxation to f^eq(rho, u^eq) plus the velocity-shift term of Eq. (4),
-// C = (1/tau) [f^eq(rho, u^eq + tau F / rho) - f^eq(rho, u^eq)], then the
-// push of direction I of species k.
-template <typename real, int I, bool kInner, class Stage>
-__device__ __forceinline__ void shift_push_dir(const Lat<real> &L, real *__restrict__ fn, const Stage &sg, int k,
-                                               real f, real rho, real ux, real uy, real uu, real sx, real sy, real ss,
-                                               int x, int y, int cx, int cy)
-{
-    const real om = L.omega[k];
-    const real feq = feq_dir<real, I>(rho, ux, uy, uu);
-    const real feqs = feq_dir<real, I>(rho, sx, sy, ss);
-    const real C = om * (feqs - feq);
-    push_dir<real, I, kInner>(L, fn, sg, k, x, y, cx, cy, f - om * (f - feq) + C);
-}
-
-// The node's collision and pushes in the original model: u^eq of Eq. (3)
-// from the momenta sum_i f e_i (no force), species k relaxed with the
-// velocity-shift term of Eq. (4).
-template <typename real, bool kInner, class Stage>
-__device__ __forceinline__ void shift_collide_site(const Lat<real> &L, real *__restrict__ fn, const Stage &sg,
-                                                   real (&fk)[2][9], int x, int y, int cx, int cy)
-{
-    real F[2][2], rho[2], m[2][2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        sg.force(L, k, cx, cy, F[k][0], F[k][1]);
-        rho[k] = sg.density(k, cy, cx);
-        first_moment<real>(fk[k], m[k][0], m[k][1]);
-    }
-    const real om0 = L.omega[0], om1 = L.omega[1];
-    const real den = om0 * rho[0] + om1 * rho[1];
-    const real ux = (om0 * m[0][0] + om1 * m[1][0]) / den;
-    const real uy = (om0 * m[0][1] + om1 * m[1][1]) / den;
-    const real uu = ux * ux + uy * uy;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const real sx = ux + L.tau[k] * F[k][0] / rho[k], sy = uy + L.tau[k] * F[k][1] / rho[k];
-        const real ss = sx * sx + sy * sy;
-        const real(&f)[9] = fk[k];
-        const real r = rho[k];
-        shift_push_dir<real, 0, kInner>(L, fn, sg, k, f[0], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 1, kInner>(L, fn, sg, k, f[1], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 2, kInner>(L, fn, sg, k, f[2], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 3, kInner>(L, fn, sg, k, f[3], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 4, kInner>(L, fn, sg, k, f[4], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 5, kInner>(L, fn, sg, k, f[5], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 6, kInner>(L, fn, sg, k, f[6], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 7, kInner>(L, fn, sg, k, f[7], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-        shift_push_dir<real, 8, kInner>(L, fn, sg, k, f[8], r, ux, uy, uu, sx, sy, ss, x, y, cx, cy);
-    }
-}
-
 // Force, moments, u^eq, collision and push of the node (x, y), staged at
-// (cx, cy).  Its populations are fk (updated in place), or with kBox (FP32)
+// (cx, cy).  Its populations are fk (updated in place), or with kBox
 // the shared-memory box: box[(k * 9 + i) * box_plane] is population i of
 // species k, read again where it is used with the same density offset
 // applied, which keeps 18 registers free; fk is then not used, and the
@@ -590,10 +396,11 @@ __device__ __forceinline__ void shift_collide_site(const Lat<real> &L, real *__r
 // The FP32 node collision: half-force momenta (Eq. 6), the offsets from the
 // node's current density, u^eq and the terms shared by the directions, then
 // the collision of each direction of both species and its push.
-template <bool kInner, bool kBox, class Stage>
-__device__ __forceinline__ void collide_site_off(const Lat<float> &L, float *__restrict__ fn, const Stage &sg,
-                                                 float (&fk)[2][9], const float (&Rn)[2], int x, int y, int cx, int cy,
-                                                 const float *__restrict__ box, int box_plane, const NodeMoments *pre)
+template <bool kInner, bool kBox = false, class Stage>
+__device__ __forceinline__ void collide_site(const Lat<float> &L, float *__restrict__ fn, const Stage &sg,
+                                             float (&fk)[2][9], const float (&Rn)[2], int x, int y, int cx, int cy,
+                                             const float *__restrict__ box = nullptr, int box_plane = 0,
+                                             const NodeMoments *pre = nullptr)
 {
     // both species at once, as (A, B) pairs
     float2 Fx, Fy, jx, jy, delta, dg;
@@ -654,8 +461,8 @@ __device__ __forceinline__ void collide_site_off(const Lat<float> &L, float *__r
             node[(size_t)I * plane + (EY * pitch + EX)] = v.x;
             node[(size_t)(9 + I) * plane + (EY * pitch + EX)] = v.y;
         } else {
-            push_dir<float, I, kInner, Stage, false>(L, fn, sg, 0, x, y, cx, cy, v.x);
-            push_dir<float, I, kInner, Stage, false>(L, fn, sg, 1, x, y, cx, cy, v.y);
+            push_edge<I>(L, fn, 0, x, y, v.x);
+            push_edge<I>(L, fn, 1, x, y, v.y);
         }
     };
     dir(std::integral_constant<int, 0>{});
@@ -669,55 +476,412 @@ __device__ __forceinline__ void collide_site_off(const Lat<float> &L, float *__r
     dir(std::integral_constant<int, 8>{});
 }
 
-// Force, moments, u^eq, collision and push of the node (x, y), staged at
-// (cx, cy).  Its populations are fk (updated in place), or with kBox (FP32)
-// the shared-memory box: box[(k * 9 + i) * box_plane] is population i of
-// species k, read again where it is used with the same density offset
-// applied, which keeps 18 registers free; fk is then not used, and the
-// force-free moments come precomputed in *pre (node_moments).
-template <typename real, bool kInner, bool kBox, class Stage>
-__device__ __forceinline__ void collide_site(const Lat<real> &L, real *__restrict__ fn, const Stage &sg,
-                                             real (&fk)[2][9], const real (&Rn)[2], int x, int y, int cx, int cy,
-                                             const real *__restrict__ box, int box_plane, const NodeMoments *pre)
+// Fused force + collision + push-streaming + bounce-back for one tile.  Every
+// thread of the block calls it and returns from it; it ends after the tile's
+// pushes are issued (the caller synchronises before reusing sm).
+template <int TYv, bool kCG>
+__device__ __forceinline__ void collide_tile(const Lat<float> *__restrict__ lats, int4 t, int parity,
+                                             CollideSmem<TYv> &sm)
 {
-    static_assert(!kBox || kOffset<real>, "the box form is FP32 only");
-    if constexpr (kOffset<real>) {
-        collide_site_off<kInner, kBox>(L, fn, sg, fk, Rn, x, y, cx, cy, box, box_plane, pre);
-    } else {
-        (void)Rn;
-        (void)box;
-        (void)box_plane;
-        (void)pre;
-        if (L.forcing == 1) {   // the original model (Eq. 4), a block-uniform branch
-            shift_collide_site<real, kInner>(L, fn, sg, fk, x, y, cx, cy);
-            return;
-        }
-        real F[2][2], rho[2], m[2][2];
+    const Lat<float> &G = lats[t.x];
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    static_assert(sizeof(Lat<float>) % 4 == 0, "descriptor copied as 32-bit words");
+    for (int i = tid; i < (int)(sizeof(Lat<float>) / 4); i += TX * TYv)
+        reinterpret_cast<uint32_t *>(&sm.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
+    const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
+    const bool valid = x < G.nx && y < G.ny;
+    // issue the population loads first so their latency overlaps the staging
+    const float *__restrict__ fc = G.f[parity];
+    float *__restrict__ fn = G.f[parity ^ 1];
+    const size_t c = valid ? (size_t)y * G.pitch + x : 0;
+    float fk[2][9];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            sg.force(L, k, cx, cy, F[k][0], F[k][1]);
-            rho[k] = sg.density(k, cy, cx);
-            real jx, jy;
-            first_moment<real>(fk[k], jx, jy);
-            m[k][0] = jx + (real)0.5 * F[k][0];   // Eq. (6), half force
-            m[k][1] = jy + (real)0.5 * F[k][1];
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (float)0;
+    if constexpr (kCG) {
+        // staging reads the density copy through L2 as well
+        constexpr int SHv = TYv + 2 * HALO;
+        const int nx = G.nx, ny = G.ny;
+        const float *__restrict__ rho = G.rho[parity ^ 1];
+        for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
+            const int sx = idx % SW, sy = idx / SW;
+            const int gx = wrap_index(t.y + sx - HALO, nx);
+            int gy = t.z + sy - HALO;
+            float rA, rB;
+            bool fixed = false;
+            if (gy < 0 || gy >= ny) {
+                if (G.walls) {
+                    if (G.wall_mode == 1) {
+                        rA = G.wall_rho[0];
+                        rB = G.wall_rho[1];
+                        fixed = true;
+                    } else {
+                        gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
+                        gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);
+                    }
+                } else {
+                    gy = wrap_index(gy, ny);
+                }
+            }
+            if (!fixed) {
+                const size_t cc = (size_t)gy * G.pitch + gx;
+                rA = __ldcg(&rho[cc]);
+                rB = __ldcg(&rho[G.plane + cc]);
+            }
+            sm.srho[0][sy][sx] = rA;
+            sm.srho[1][sy][sx] = rB;
+            sm.spsi[0][sy][sx] = psi_of<float>(rA);
+            sm.spsi[1][sy][sx] = psi_of<float>(rB);
         }
-        // common velocity, Eq. (3)
-        const real om0 = L.omega[0], om1 = L.omega[1];
-        const real den = om0 * rho[0] + om1 * rho[1];
-        const real ux = (om0 * m[0][0] + om1 * m[1][0]) / den;
-        const real uy = (om0 * m[0][1] + om1 * m[1][1]) / den;
-        const real uu = ux * ux + uy * uy;
-        collide_push_dir<real, 0, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 1, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 2, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 3, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 4, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 5, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 6, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 7, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
-        collide_push_dir<real, 8, kInner>(L, fn, sg, fk, rho, ux, uy, uu, F, x, y, cx, cy);
+    } else {
+        stage_tile<float, TYv + 2 * HALO>(G, G.rho[parity ^ 1], t.y, t.z, sm.srho, sm.spsi, tid, TX * TYv);
     }
+    __syncthreads();
+    if (!valid) return;
+    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
+    float Rn[2] = {(float)0, (float)0};
+    Rn[0] = ldg_state<kCG>(&G.rho[parity][c]);
+    Rn[1] = ldg_state<kCG>(&G.rho[parity][G.plane + c]);
+    // tiles whose pushes stay inside the lattice (no wrap, no wall) take constant offsets
+    const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
+    const SplitStage<TYv + 2 * HALO> sg{sm.srho, sm.spsi};
+    if (inner) collide_site<true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
+    else collide_site<false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
+}
+
+// ---- the FP64 node ----------------------------------------------------------
+
+// What the FP64 step stages per slot and species: density, psi, and every
+// product with a stencil weight that a neighbour's sums take from the slot.
+// The sums of Eqs. (8), (9) use 40 such products per node and species, of
+// which only these 9 per slot differ (2 p5 psi is p5 psi doubled, exactly).
+enum Plane64 { sRho = 0, sPsi, sW1Psi, sW2Psi, sP1, sP2, s2P4, sP5, s2P8, sW1Rho, sW2Rho, kPlanes64 };
+
+template <int TYv>
+struct Stage64 {
+    double v[2][kPlanes64][TYv + 2 * HALO][SW];
+    Lat<double> L;   // descriptor copy: stores to the populations cannot alias it
+
+    // density and psi of species k at a slot, and the slot's products;
+    // nonzero where one lies outside the range of the integer products
+    __device__ __forceinline__ uint32_t put(int k, int sy, int sx, double r, double p)
+    {
+        double(*q)[TYv + 2 * HALO][SW] = v[k];
+        q[sRho][sy][sx] = r;
+        q[sPsi][sy][sx] = p;
+        const uint32_t outside = base_outside(r) | base_outside(p);
+        if (outside) {
+            q[sW1Psi][sy][sx] = (1.0 / 9.0) * p;
+            q[sW2Psi][sy][sx] = (1.0 / 36.0) * p;
+            q[sP1][sy][sx] = p25(1) * p;
+            q[sP2][sy][sx] = p25(2) * p;
+            q[s2P4][sy][sx] = (2.0 * p25(4)) * p;
+            q[sP5][sy][sx] = p25(5) * p;
+            q[s2P8][sy][sx] = (2.0 * p25(8)) * p;
+            q[sW1Rho][sy][sx] = (1.0 / 9.0) * r;
+            q[sW2Rho][sy][sx] = (1.0 / 36.0) * r;
+            return outside;
+        }
+        const Factor fp = factor(p), fr = factor(r);
+        q[sW1Psi][sy][sx] = factor_mul(fp, factor(1.0 / 9.0));
+        q[sW2Psi][sy][sx] = factor_mul(fp, factor(1.0 / 36.0));
+        q[sP1][sy][sx] = factor_mul(fp, factor(p25(1)));
+        q[sP2][sy][sx] = factor_mul(fp, factor(p25(2)));
+        q[s2P4][sy][sx] = factor_mul(fp, factor(2.0 * p25(4)));
+        q[sP5][sy][sx] = factor_mul(fp, factor(p25(5)));
+        q[s2P8][sy][sx] = factor_mul(fp, factor(2.0 * p25(8)));
+        q[sW1Rho][sy][sx] = factor_mul(fr, factor(1.0 / 9.0));
+        q[sW2Rho][sy][sx] = factor_mul(fr, factor(1.0 / 36.0));
+        return 0;
+    }
+};
+
+// Total force on species k at the staged node, Eq. (8) + Eq. (9) + rho_k g:
+// the sums in direction order (D2Q9) and raster order (D2Q25), as q9_sum and
+// q25_sum form them, from the staged products.
+template <bool kInt, int TYv>
+__device__ __forceinline__ void force64(const Arith64<kInt> &A, const Stage64<TYv> &sm, int k, int cx, int cy, double &Fx,
+                                        double &Fy)
+{
+    const double(*q)[TYv + 2 * HALO][SW] = sm.v[k];
+    const double(*o)[TYv + 2 * HALO][SW] = sm.v[1 - k];
+    auto at = [&](int plane, int dy, int dx) { return q[plane][cy + dy][cx + dx]; };
+    auto ot = [&](int plane, int dy, int dx) { return o[plane][cy + dy][cx + dx]; };
+    auto q9 = [&](auto &&g, int w1, int w2, double &sx, double &sy) {
+        const double a5 = g(w2, 1, 1), a6 = g(w2, 1, -1), a7 = g(w2, -1, -1), a8 = g(w2, -1, 1);
+        sx = A.add(A.sub(A.sub(A.add(A.sub(g(w1, 0, 1), g(w1, 0, -1)), a5), a6), a7), a8);
+        sy = A.sub(A.sub(A.add(A.add(A.sub(g(w1, 1, 0), g(w1, -1, 0)), a5), a6), a7), a8);
+    };
+    double s1x, s1y, s2x, s2y, s3x, s3y;
+    q9(at, sW1Psi, sW2Psi, s1x, s1y);
+    q9(ot, sW1Rho, sW2Rho, s3x, s3y);
+    const double two = A.one + A.one;
+    {
+        // rows dy = -2 .. 2, columns dx = -2 .. 2 within a row; a term's
+        // component along an axis of reach 2 is twice p psi
+        double a, x, y;
+        a = at(s2P8, -2, -2);
+        x = -a;
+        y = -a;
+        a = at(sP5, -2, -1);
+        x = A.sub(x, a);
+        y = __fma_rn(-a, two, y);
+        y = A.sub(y, at(s2P4, -2, 0));
+        a = at(sP5, -2, 1);
+        x = A.add(x, a);
+        y = __fma_rn(-a, two, y);
+        a = at(s2P8, -2, 2);
+        x = A.add(x, a);
+        y = A.sub(y, a);
+
+        a = at(sP5, -1, -2);
+        x = __fma_rn(-a, two, x);
+        y = A.sub(y, a);
+        a = at(sP2, -1, -1);
+        x = A.sub(x, a);
+        y = A.sub(y, a);
+        y = A.sub(y, at(sP1, -1, 0));
+        a = at(sP2, -1, 1);
+        x = A.add(x, a);
+        y = A.sub(y, a);
+        a = at(sP5, -1, 2);
+        x = __fma_rn(a, two, x);
+        y = A.sub(y, a);
+
+        x = A.sub(x, at(s2P4, 0, -2));
+        x = A.sub(x, at(sP1, 0, -1));
+        x = A.add(x, at(sP1, 0, 1));
+        x = A.add(x, at(s2P4, 0, 2));
+
+        a = at(sP5, 1, -2);
+        x = __fma_rn(-a, two, x);
+        y = A.add(y, a);
+        a = at(sP2, 1, -1);
+        x = A.sub(x, a);
+        y = A.add(y, a);
+        y = A.add(y, at(sP1, 1, 0));
+        a = at(sP2, 1, 1);
+        x = A.add(x, a);
+        y = A.add(y, a);
+        a = at(sP5, 1, 2);
+        x = __fma_rn(a, two, x);
+        y = A.add(y, a);
+
+        a = at(s2P8, 2, -2);
+        x = A.sub(x, a);
+        y = A.add(y, a);
+        a = at(sP5, 2, -1);
+        x = A.sub(x, a);
+        y = __fma_rn(a, two, y);
+        y = A.add(y, at(s2P4, 2, 0));
+        a = at(sP5, 2, 1);
+        x = A.add(x, a);
+        y = __fma_rn(a, two, y);
+        a = at(s2P8, 2, 2);
+        s2x = A.add(x, a);
+        s2y = A.add(y, a);
+    }
+    const double psi = q[sPsi][cy][cx], rho = q[sRho][cy][cx];
+    const double c1 = A.mul(-sm.L.G1, psi), c2 = A.mul(sm.L.G2, psi), c3 = A.mul(sm.L.GAB, rho);
+    Fx = A.sub(A.sub(A.mul(c1, s1x), A.mul(c2, s2x)), A.mul(c3, s3x));
+    Fy = A.sub(A.sub(A.mul(c1, s1y), A.mul(c2, s2y)), A.mul(c3, s3y));
+    // + rho g; a zero component adds nothing to a finite force
+    if (!kInt || sm.L.g[0] != 0.0) Fx = A.add(Fx, A.mul(rho, sm.L.g[0]));
+    if (!kInt || sm.L.g[1] != 0.0) Fy = A.add(Fy, A.mul(rho, sm.L.g[1]));
+}
+
+// Where the node's pushes go: element offsets to its neighbours, and whether
+// a vertical push meets a wall.
+struct Push64 {
+    long long oE, oW, oN, oS;
+    bool wallN, wallS;
+    __device__ __forceinline__ Push64(const Lat<double> &L, int x, int y)
+    {
+        oE = x + 1 < L.nx ? 1 : 1 - L.nx;
+        oW = x > 0 ? -1 : L.nx - 1;
+        oN = y + 1 < L.ny ? (long long)L.pitch : -(long long)L.pitch * (L.ny - 1);
+        oS = y > 0 ? -(long long)L.pitch : (long long)L.pitch * (L.ny - 1);
+        wallN = L.walls && y + 1 >= L.ny;
+        wallS = L.walls && y <= 0;
+    }
+    // store v, the post-collision value of direction I of the species whose
+    // population planes at the node start at fk (half-way bounce-back at walls)
+    template <int I>
+    __device__ __forceinline__ void store(double *__restrict__ fk, size_t plane, double v) const
+    {
+        constexpr int EX = ex9(I), EY = ey9(I);
+        long long off = (EX > 0 ? oE : EX < 0 ? oW : 0) + (EY > 0 ? oN : EY < 0 ? oS : 0);
+        int dir = I;
+        if constexpr (EY != 0)
+            if (EY > 0 ? wallN : wallS) {
+                dir = opp9(I);
+                off = 0;
+            }
+        fk[(long long)((size_t)dir * plane) + off] = v;
+    }
+};
+
+// Force, half-force momenta, u^eq, collision with the Guo term and push of
+// both species at node (x, y), staged at (cx, cy): Eqs. (1)-(3), (5), (6),
+// (8), (9), operation by operation as collide_dir writes them.  j: the
+// species' momenta sum_i f e_i; fc, fn: the node's first population plane in
+// the current and the next copy.  Returns whether a value lay outside the
+// range the integer products cover (lb_f64.cuh; the caller then redoes the
+// node with kInt = false).
+template <bool kInt, int TYv, bool kCG>
+__device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const double *__restrict__ fc,
+                                       double *__restrict__ fn, const double (&j)[2][2], int x, int y, int cx, int cy)
+{
+    const Arith64<kInt> A(one);
+    const Lat<double> &L = sm.L;
+    const size_t plane = L.plane;
+    uint32_t outside = 0;
+    double F[2][2], m[2][2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        force64<kInt, TYv>(A, sm, k, cx, cy, F[k][0], F[k][1]);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) m[k][a] = __fma_rn(0.5, F[k][a], j[k][a]);   // Eq. (6): F/2 is exact
+    }
+    const double r0 = sm.v[0][sRho][cy][cx], r1 = sm.v[1][sRho][cy][cx];
+    const double om0 = L.omega[0], om1 = L.omega[1];
+    const double den = A.add(A.mul(om0, r0), A.mul(om1, r1));
+    const double ux = A.add(A.mul(om0, m[0][0]), A.mul(om1, m[1][0])) / den;
+    const double uy = A.add(A.mul(om0, m[0][1]), A.mul(om1, m[1][1])) / den;
+    if constexpr (kInt) {
+        outside = velocity_outside(ux) | velocity_outside(uy);
+    }
+    const double uu15 = A.mul(1.5, A.add(A.mul(ux, ux), A.mul(uy, uy)));
+    // e.u of the diagonals; opposite directions differ by an exact sign
+    const double s = A.add(ux, uy), d = A.sub(ux, uy);
+    // the Guo vectors (e - u)/cs^2 + (e.u) e/cs^4
+    const double gx0 = -A.mul(3.0, ux), gy0 = -A.mul(3.0, uy);
+    const double xp = A.mul(3.0, A.sub(1.0, ux)), xm = A.mul(3.0, A.sub(-1.0, ux));
+    const double yp = A.mul(3.0, A.sub(1.0, uy)), ym = A.mul(3.0, A.sub(-1.0, uy));
+    const double x9 = A.mul(9.0, ux), y9 = A.mul(9.0, uy), s9 = A.mul(9.0, s), d9 = A.mul(9.0, d);
+    const double gx[9] = {gx0, A.add(xp, x9), gx0, A.add(xm, x9), gx0, A.add(xp, s9), A.add(xm, d9), A.add(xm, s9),
+                          A.add(xp, d9)};
+    const double gy[9] = {gy0, gy0, A.add(yp, y9), gy0, A.add(ym, y9), A.add(yp, s9), A.sub(yp, d9), A.add(ym, s9),
+                          A.sub(ym, d9)};
+    // 1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u.u
+    double po[9];
+    po[0] = A.sub(1.0, uu15);
+    {
+        const double e[4] = {ux, uy, s, d};
+        constexpr int plus[4] = {1, 2, 5, 8}, minus[4] = {3, 4, 7, 6};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double e3 = A.mul(3.0, e[q]), ee = A.mul(A.mul(4.5, e[q]), e[q]);
+            po[plus[q]] = A.sub(A.add(A.add(1.0, e3), ee), uu15);
+            po[minus[q]] = A.sub(A.add(A.sub(1.0, e3), ee), uu15);
+        }
+    }
+    const Push64 push(L, x, y);
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        const double *__restrict__ fk = fc + (size_t)(k * 9) * plane;
+        double *__restrict__ nk = fn + (size_t)(k * 9) * plane;
+        const double r = k ? r1 : r0, om = k ? om1 : om0;
+        const double Fx = k ? F[1][0] : F[0][0], Fy = k ? F[1][1] : F[0][1];
+        double f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = ldg_state<kCG>(&fk[(size_t)i * plane]);
+        if constexpr (kInt) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) outside |= base_outside(f[i]);
+        }
+        const double p0x = A.mul(gx0, Fx), p0y = A.mul(gy0, Fy);
+        const double wr[3] = {A.mul(4.0 / 9.0, r), A.mul(1.0 / 9.0, r), A.mul(1.0 / 36.0, r)};
+        const double aw[3] = {L.aw[k][0], L.aw[k][1], L.aw[k][2]};
+        auto dir = [&](auto Ic) {
+            constexpr int I = decltype(Ic)::value, c = cls9(I);
+            const double gFx = ex9(I) == 0 ? p0x : A.mul(gx[I], Fx), gFy = ey9(I) == 0 ? p0y : A.mul(gy[I], Fy);
+            const double C = A.mul(aw[c], A.add(gFx, gFy));
+            const double feq = A.mul(wr[c], po[I]);
+            push.store<I>(nk, plane, A.add(A.sub(f[I], A.mul(om, A.sub(f[I], feq))), C));
+        };
+        dir(std::integral_constant<int, 0>{});
+        dir(std::integral_constant<int, 1>{});
+        dir(std::integral_constant<int, 2>{});
+        dir(std::integral_constant<int, 3>{});
+        dir(std::integral_constant<int, 4>{});
+        dir(std::integral_constant<int, 5>{});
+        dir(std::integral_constant<int, 6>{});
+        dir(std::integral_constant<int, 7>{});
+        dir(std::integral_constant<int, 8>{});
+    }
+    return outside != 0;
+}
+
+// The species' momenta sum_i f e_i of a node.
+struct Mom64 {
+    double j[2][2];
+};
+
+// The velocity-shift node (Eq. 4) on the staged planes.
+template <int TYv, bool kCG>
+__device__ __noinline__ void shift_node64(const Stage64<TYv> &sm, double one, const double *__restrict__ fc,
+                                          double *__restrict__ fn, Mom64 jj, int x, int y, int cx, int cy)
+{
+    const double(&j)[2][2] = jj.j;
+    const Lat<double> &L = sm.L;
+    const Arith64<false> A(one);
+    double F[2][2], rho[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        force64<false, TYv>(A, sm, k, cx, cy, F[k][0], F[k][1]);
+        rho[k] = sm.v[k][sRho][cy][cx];
+    }
+    const double om0 = L.omega[0], om1 = L.omega[1];
+    const double den = om0 * rho[0] + om1 * rho[1];
+    const double ux = (om0 * j[0][0] + om1 * j[1][0]) / den;
+    const double uy = (om0 * j[0][1] + om1 * j[1][1]) / den;
+    const double uu = ux * ux + uy * uy;
+    const Push64 push(L, x, y);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double sx = ux + L.tau[k] * F[k][0] / rho[k], sy = uy + L.tau[k] * F[k][1] / rho[k];
+        const double ss = sx * sx + sy * sy, om = L.omega[k];
+        // relaxation to f^eq(rho, u^eq) plus (1/tau) [f^eq(rho, u^eq + tau F / rho) - f^eq(rho, u^eq)]
+        auto dir = [&](auto Ic) {
+            constexpr int I = decltype(Ic)::value;
+            const double f = ldg_state<kCG>(&fc[(size_t)(k * 9 + I) * L.plane]);
+            const double feq = feq_dir<double, I>(rho[k], ux, uy, uu), feqs = feq_dir<double, I>(rho[k], sx, sy, ss);
+            push.store<I>(fn + (size_t)(k * 9) * L.plane, L.plane, f - om * (f - feq) + om * (feqs - feq));
+        };
+        dir(std::integral_constant<int, 0>{});
+        dir(std::integral_constant<int, 1>{});
+        dir(std::integral_constant<int, 2>{});
+        dir(std::integral_constant<int, 3>{});
+        dir(std::integral_constant<int, 4>{});
+        dir(std::integral_constant<int, 5>{});
+        dir(std::integral_constant<int, 6>{});
+        dir(std::integral_constant<int, 7>{});
+        dir(std::integral_constant<int, 8>{});
+    }
+}
+
+template <int TYv, bool kCG>
+__device__ __noinline__ void plain_node64(const Stage64<TYv> &sm, double one, const double *__restrict__ fc,
+                                          double *__restrict__ fn, Mom64 j, int x, int y, int cx, int cy)
+{
+    node64<false, TYv, kCG>(sm, one, fc, fn, j.j, x, y, cx, cy);
+}
+
+// The node's step after staging, in the lattice's forcing; plain: a staged
+// value of the block lies outside the range of the integer products.
+template <int TYv, bool kCG>
+__device__ __forceinline__ void finish64(const Stage64<TYv> &sm, const double *__restrict__ fc, double *__restrict__ fn,
+                                         const Mom64 &j, int x, int y, int cx, int cy, bool plain)
+{
+    const double one = sm.L.one;
+    if (sm.L.forcing == 1) {   // the original model (Eq. 4), a block-uniform branch
+        shift_node64<TYv, kCG>(sm, one, fc, fn, j, x, y, cx, cy);
+        return;
+    }
+    if (plain || !sm.L.products || node64<true, TYv, kCG>(sm, one, fc, fn, j.j, x, y, cx, cy))
+        plain_node64<TYv, kCG>(sm, one, fc, fn, j, x, y, cx, cy);
 }
 
 // ---- one-pass step ------------------------------------------------------------
@@ -732,7 +896,7 @@ __device__ __forceinline__ real node_density(const Lat<real> &L, int k, int gx, 
     real v[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) v[i] = ldg_state<kCG>(&f[(size_t)(k * 9 + i) * L.plane + c]);
-    real r = zeroth_moment<real>(v);
+    real r = zeroth_moment<real>(v, L.one);
     if constexpr (kOffset<real>) r = ldg_state<kCG>(&L.rho[parity][(size_t)k * L.plane + c]) + r;
     return r;
 }
@@ -765,17 +929,38 @@ __device__ __forceinline__ void slot_densities(const Lat<real> &G, int4 t, int p
     rB = node_density<real, kCG>(G, 1, gx, gy, parity);
 }
 
+// Staged slot (sx, sy) of the h-th position of a tile's halo ring, enumerated
+// compactly: two rows above, two below, then the two columns on each side of
+// the tile's rows.
+template <int TYv>
+constexpr int kRing = 4 * SW + 4 * TYv;
+template <int TYv>
+__device__ __forceinline__ void ring_slot(int h, int &sx, int &sy)
+{
+    if (h < 2 * SW) {
+        sy = h / SW;
+        sx = h % SW;
+    } else if (h < 4 * SW) {
+        sy = TYv + HALO + (h - 2 * SW) / SW;
+        sx = (h - 2 * SW) % SW;
+    } else {
+        const int q = h - 4 * SW;
+        sy = HALO + q / 4;
+        sx = (q % 4 < 2) ? q % 4 : TX + q % 4;
+    }
+}
+
 // The same, staged with psi into the tile's density and psi planes.
-template <typename real, int TYv, bool kCG>
-__device__ __forceinline__ void stage_slot(const Lat<real> &G, int4 t, int parity, CollideSmem<real, TYv> &sm, int sx,
+template <int TYv, bool kCG>
+__device__ __forceinline__ void stage_slot(const Lat<float> &G, int4 t, int parity, CollideSmem<TYv> &sm, int sx,
                                            int sy)
 {
-    real rA, rB;
-    slot_densities<real, kCG>(G, t, parity, sx, sy, rA, rB);
+    float rA, rB;
+    slot_densities<float, kCG>(G, t, parity, sx, sy, rA, rB);
     sm.srho[0][sy][sx] = rA;
     sm.srho[1][sy][sx] = rB;
-    sm.spsi[0][sy][sx] = psi_of<real>(rA);
-    sm.spsi[1][sy][sx] = psi_of<real>(rB);
+    sm.spsi[0][sy][sx] = psi_of<float>(rA);
+    sm.spsi[1][sy][sx] = psi_of<float>(rB);
 }
 
 // One time step of one tile in a single pass: each thread forms its node's
@@ -783,83 +968,219 @@ __device__ __forceinline__ void stage_slot(const Lat<real> &G, int4 t, int parit
 // slots of a ragged tile's missing nodes) is formed from the neighbours'
 // populations, mostly L2 hits.  The halo goes first, so that its loads and
 // the node's own 18 populations are not held in registers at the same time.
-// FP32 writes the node's density as the next step's reference.  Then the
+// It writes the node's density as the next step's reference.  Then the
 // fused force + collision + push of collide_site.
-template <typename real, int TYv, bool kCG>
-__device__ __forceinline__ void fused_tile(const Lat<real> *__restrict__ lats, int4 t, int parity,
-                                           CollideSmem<real, TYv> &sm)
+template <int TYv, bool kCG>
+__device__ __forceinline__ void fused_tile(const Lat<float> *__restrict__ lats, int4 t, int parity,
+                                           CollideSmem<TYv> &sm)
 {
     constexpr int SHv = TYv + 2 * HALO;
-    const Lat<real> &G = lats[t.x];
+    const Lat<float> &G = lats[t.x];
     const int tid = threadIdx.y * TX + threadIdx.x;
-    for (int i = tid; i < (int)(sizeof(Lat<real>) / 4); i += TX * TYv)
+    for (int i = tid; i < (int)(sizeof(Lat<float>) / 4); i += TX * TYv)
         reinterpret_cast<uint32_t *>(&sm.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
     const int nx = G.nx, ny = G.ny;
     const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
     const bool valid = x < nx && y < ny;
-    const real *__restrict__ fc = G.f[parity];
-    real *__restrict__ fn = G.f[parity ^ 1];
+    const float *__restrict__ fc = G.f[parity];
+    float *__restrict__ fn = G.f[parity ^ 1];
     const size_t c = valid ? (size_t)y * G.pitch + x : 0;
-    // the halo ring, enumerated compactly: two rows above, two below, then
-    // the two columns on each side of the tile's rows
-    constexpr int kRing = 4 * SW + 4 * TYv;
-    for (int h = tid; h < kRing; h += TX * TYv) {
+    for (int h = tid; h < kRing<TYv>; h += TX * TYv) {
         int sx, sy;
-        if (h < 2 * SW) {
-            sy = h / SW;
-            sx = h % SW;
-        } else if (h < 4 * SW) {
-            sy = TYv + HALO + (h - 2 * SW) / SW;
-            sx = (h - 2 * SW) % SW;
-        } else {
-            const int q = h - 4 * SW;
-            sy = HALO + q / 4;
-            sx = (q % 4 < 2) ? q % 4 : TX + q % 4;
-        }
-        stage_slot<real, TYv, kCG>(G, t, parity, sm, sx, sy);
+        ring_slot<TYv>(h, sx, sy);
+        stage_slot<TYv, kCG>(G, t, parity, sm, sx, sy);
     }
     // a ragged tile's slots without a node of their own hold wrapped copies
     if (t.y + TX > nx || t.z + TYv > ny) {
         for (int q = tid; q < TX * TYv; q += TX * TYv) {
             const int sx = HALO + q % TX, sy = HALO + q / TX;
-            if (t.y + sx - HALO >= nx || t.z + sy - HALO >= ny) stage_slot<real, TYv, kCG>(G, t, parity, sm, sx, sy);
+            if (t.y + sx - HALO >= nx || t.z + sy - HALO >= ny) stage_slot<TYv, kCG>(G, t, parity, sm, sx, sy);
         }
     }
     // then the node's own populations (kept in registers for the collision)
-    real fk[2][9];
+    float fk[2][9];
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (real)0;
+        for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (float)0;
     const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
-    real Rn[2] = {(real)0, (real)0};
+    float Rn[2] = {(float)0, (float)0};
     if (valid) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            real r = zeroth_moment<real>(fk[k]);
-            if constexpr (kOffset<real>) {
-                Rn[k] = ldg_state<kCG>(&G.rho[parity][(size_t)k * G.plane + c]);
-                r = Rn[k] + r;
-                G.rho[parity ^ 1][(size_t)k * G.plane + c] = r;
-            }
+            float r = zeroth_moment<float>(fk[k], 1.f);
+            Rn[k] = ldg_state<kCG>(&G.rho[parity][(size_t)k * G.plane + c]);
+            r = Rn[k] + r;
+            G.rho[parity ^ 1][(size_t)k * G.plane + c] = r;
             sm.srho[k][cy][cx] = r;
-            sm.spsi[k][cy][cx] = psi_of<real>(r);
+            sm.spsi[k][cy][cx] = psi_of<float>(r);
         }
     }
     __syncthreads();
     if (!valid) return;
     const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
-    const SplitStage<real, SHv> sg{sm.srho, sm.spsi};
-    if (inner) collide_site<real, true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
-    else collide_site<real, false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
+    const SplitStage<SHv> sg{sm.srho, sm.spsi};
+    if (inner) collide_site<true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
+    else collide_site<false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
+}
+
+// ---- the FP64 tiles -------------------------------------------------------------
+
+template <int TYv>
+__device__ __forceinline__ void copy_lat64(Stage64<TYv> &sm, const Lat<double> &G, int tid)
+{
+    for (int i = tid; i < (int)(sizeof(Lat<double>) / 4); i += TX * TYv)
+        reinterpret_cast<uint32_t *>(&sm.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
+}
+
+// First moments of the node's populations (direction order).
+template <bool kCG>
+__device__ __forceinline__ void node_moments64(const double *__restrict__ fc, size_t plane, double one, Mom64 &m,
+                                               double (*rho)[2])
+{
+    const Arith64<false> A(one);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        double f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * plane]);
+        m.j[k][0] = A.add(A.sub(A.sub(A.add(A.sub(f[1], f[3]), f[5]), f[6]), f[7]), f[8]);
+        m.j[k][1] = A.sub(A.sub(A.add(A.add(A.sub(f[2], f[4]), f[5]), f[6]), f[7]), f[8]);
+        if (rho) {
+            (*rho)[k] = zeroth_moment<double>(f, one);
+        }
+    }
+}
+
+// The fused kernel of the two-pass step in FP64: stages the densities and psi
+// the density pass wrote, then the node.
+template <int TYv, bool kCG>
+__device__ __forceinline__ void collide_tile64(const Lat<double> *__restrict__ lats, int4 t, int parity,
+                                               Stage64<TYv> &sm)
+{
+    constexpr int SHv = TYv + 2 * HALO;
+    const Lat<double> &G = lats[t.x];
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    copy_lat64<TYv>(sm, G, tid);
+    const int nx = G.nx, ny = G.ny;
+    const bool inner = t.y >= HALO && t.y + TX + HALO <= nx && t.z >= HALO && t.z + TYv + HALO <= ny;
+    const double *__restrict__ rho = G.rho[parity ^ 1], *__restrict__ psi = G.rho[parity];
+    uint32_t outside = 0;
+    for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
+        const int sx = idx % SW, sy = idx / SW;
+        int gx = t.y + sx - HALO, gy = t.z + sy - HALO;
+        bool fixed = false;
+        if (!inner) {
+            gx = wrap_index(gx, nx);
+            if (gy < 0 || gy >= ny) {
+                if (!G.walls) {
+                    gy = wrap_index(gy, ny);
+                } else if (G.wall_mode == 1) {
+                    fixed = true;
+                } else {
+                    gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
+                    gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);  // rows no valid node reads
+                }
+            }
+        }
+        const size_t c = (size_t)gy * G.pitch + gx;
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            const double r = fixed ? G.wall_rho[k] : ldg_state<kCG>(&rho[(size_t)k * G.plane + c]);
+            const double p = fixed ? psi_of<double>(r) : ldg_state<kCG>(&psi[(size_t)k * G.plane + c]);
+            outside |= sm.put(k, sy, sx, r, p);
+        }
+    }
+    const bool plain = __syncthreads_or(outside != 0);
+    const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
+    if (x >= nx || y >= ny) return;
+    const size_t c = (size_t)y * sm.L.pitch + x;
+    const double *__restrict__ fc = sm.L.f[parity] + c;
+    Mom64 m;
+    node_moments64<kCG>(fc, sm.L.plane, sm.L.one, m, nullptr);
+    finish64<TYv, kCG>(sm, fc, sm.L.f[parity ^ 1] + c, m, x, y, threadIdx.x + HALO, threadIdx.y + HALO, plain);
+}
+
+// One time step of one tile in a single pass in FP64: the densities of the
+// halo ring (and of a ragged tile's missing nodes) from the neighbours'
+// populations, the node's own from the populations its momenta need anyway.
+template <int TYv, bool kCG>
+__device__ __forceinline__ void fused_tile64(const Lat<double> *__restrict__ lats, int4 t, int parity,
+                                             Stage64<TYv> &sm)
+{
+    const Lat<double> &G = lats[t.x];
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    copy_lat64<TYv>(sm, G, tid);
+    const int nx = G.nx, ny = G.ny;
+    const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
+    const bool valid = x < nx && y < ny;
+    const size_t c = valid ? (size_t)y * G.pitch + x : 0;
+    const double *__restrict__ fc = G.f[parity] + c;
+    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
+    Mom64 m;
+    uint32_t outside = 0;
+    // own slot first (h < 0), then the thread's ring slots
+#pragma unroll 1
+    for (int h = tid - TX * TYv; h < kRing<TYv>; h += TX * TYv) {
+        double r[2];
+        int sx = cx, sy = cy;
+        if (h >= 0) ring_slot<TYv>(h, sx, sy);
+        if (h < 0 && valid) node_moments64<kCG>(fc, G.plane, G.one, m, &r);
+        else slot_densities<double, kCG>(G, t, parity, sx, sy, r[0], r[1]);
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            const double rk = k ? r[1] : r[0];
+            outside |= sm.put(k, sy, sx, rk, psi_of<double>(rk));
+        }
+    }
+    const bool plain = __syncthreads_or(outside != 0);
+    if (!valid) return;
+    finish64<TYv, kCG>(sm, fc, G.f[parity ^ 1] + c, m, x, y, cx, cy, plain);
+}
+
+// Shared memory of a step kernel: static in FP32; dynamic in FP64, whose
+// planes are above the 48 KB of static shared memory.
+template <typename real, int TYv>
+using StepSmem = std::conditional_t<kOffset<real>, CollideSmem<TYv>, Stage64<TYv>>;
+template <typename real, int TYv>
+constexpr size_t kStepSmem = kOffset<real> ? 0 : sizeof(Stage64<TYv>);
+
+extern __shared__ __align__(16) unsigned char lb_step_smem[];
+
+template <typename real, int TYv>
+__device__ __forceinline__ StepSmem<real, TYv> &step_smem()
+{
+    if constexpr (kOffset<real>) {
+        __shared__ CollideSmem<TYv> sm;
+        return sm;
+    } else {
+        return *reinterpret_cast<Stage64<TYv> *>(lb_step_smem);
+    }
+}
+
+template <typename real, int TYv, bool kCG>
+__device__ __forceinline__ void collide_any(const Lat<real> *__restrict__ lats, int4 t, int parity,
+                                            StepSmem<real, TYv> &sm)
+{
+    if constexpr (kOffset<real>) collide_tile<TYv, kCG>(lats, t, parity, sm);
+    else collide_tile64<TYv, kCG>(lats, t, parity, sm);
+}
+
+template <typename real, int TYv>
+__global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
+    k_collide(const Lat<real> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity)
+{
+    collide_any<real, TYv, false>(lats, tiles[tile_offset + blockIdx.x], parity, step_smem<real, TYv>());
 }
 
 template <typename real, int TYv>
 __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
     k_fused(const Lat<real> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity)
 {
-    __shared__ CollideSmem<real, TYv> sm;
-    fused_tile<real, TYv, false>(lats, tiles[tile_offset + blockIdx.x], parity, sm);
+    const int4 t = tiles[tile_offset + blockIdx.x];
+    auto &sm = step_smem<real, TYv>();
+    if constexpr (kOffset<real>) fused_tile<TYv, false>(lats, t, parity, sm);
+    else fused_tile64<TYv, false>(lats, t, parity, sm);
 }
 
 // ---- persistent launch over many time steps -----------------------------------
@@ -905,7 +1226,7 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
                  int n_tiles, int nsteps, int parity0, PersistCtl *ctl, unsigned *dens_done, unsigned *coll_done,
                  int *err, long long wait_cycles, int drop_tile)
 {
-    __shared__ CollideSmem<real, TYv> sm;
+    auto &sm = step_smem<real, TYv>();
     __shared__ long long s_item;
     __shared__ int s_ok;
     const int tid = threadIdx.y * TX + threadIdx.x;
@@ -930,7 +1251,7 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
         __syncthreads();
         if (!s_ok) break;
         if (phase == 0) density_tile<real, TYv, true>(lats, tl, parity);
-        else collide_tile<real, TYv, true>(lats, tl, parity, sm);
+        else collide_any<real, TYv, true>(lats, tl, parity, sm);
         __syncthreads();
         if (tid == 0 && tile != drop_tile) {
             __threadfence();

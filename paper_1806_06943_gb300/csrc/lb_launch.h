@@ -13,6 +13,9 @@ namespace lbk {
 
 template <typename real>
 struct Launch {
+    // shared-memory opt-in of the step kernels on the current device; call
+    // before the first launch, outside stream capture
+    static cudaError_t prepare();
     // one kernel launch over tiles [tile_offset, tile_offset + n_tiles) of
     // height ty (2, 4 or 8)
     static cudaError_t density(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,

@@ -7,6 +7,28 @@
 
 namespace lbk {
 
+template <typename real, int TYv>
+cudaError_t prepare_height()
+{
+    const int bytes = (int)kStepSmem<real, TYv>;
+    cudaError_t e = cudaFuncSetAttribute(k_collide<real, TYv>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_fused<real, TYv>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_persistent<real, TYv>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
+
+template <typename real>
+cudaError_t Launch<real>::prepare()
+{
+    if (kOffset<real>) return cudaSuccess;   // static shared memory
+    cudaError_t e = prepare_height<real, 2>();
+    if (e == cudaSuccess) e = prepare_height<real, 4>();
+    if (e == cudaSuccess) e = prepare_height<real, 8>();
+    return e;
+}
+
 template <typename real>
 cudaError_t Launch<real>::density(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                                   int ty, cudaStream_t s)
@@ -27,9 +49,9 @@ cudaError_t Launch<real>::collide(const Lat<real> *lats, const int4 *tiles, int 
 {
     if (n_tiles <= 0) return cudaSuccess;
     switch (ty) {
-    case 2: k_collide<real, 2><<<n_tiles, dim3(TX, 2), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 4: k_collide<real, 4><<<n_tiles, dim3(TX, 4), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 8: k_collide<real, 8><<<n_tiles, dim3(TX, 8), 0, s>>>(lats, tiles, tile_offset, parity); break;
+    case 2: k_collide<real, 2><<<n_tiles, dim3(TX, 2), kStepSmem<real, 2>, s>>>(lats, tiles, tile_offset, parity); break;
+    case 4: k_collide<real, 4><<<n_tiles, dim3(TX, 4), kStepSmem<real, 4>, s>>>(lats, tiles, tile_offset, parity); break;
+    case 8: k_collide<real, 8><<<n_tiles, dim3(TX, 8), kStepSmem<real, 8>, s>>>(lats, tiles, tile_offset, parity); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -41,9 +63,9 @@ cudaError_t Launch<real>::fused(const Lat<real> *lats, const int4 *tiles, int ti
 {
     if (n_tiles <= 0) return cudaSuccess;
     switch (ty) {
-    case 2: k_fused<real, 2><<<n_tiles, dim3(TX, 2), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 4: k_fused<real, 4><<<n_tiles, dim3(TX, 4), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 8: k_fused<real, 8><<<n_tiles, dim3(TX, 8), 0, s>>>(lats, tiles, tile_offset, parity); break;
+    case 2: k_fused<real, 2><<<n_tiles, dim3(TX, 2), kStepSmem<real, 2>, s>>>(lats, tiles, tile_offset, parity); break;
+    case 4: k_fused<real, 4><<<n_tiles, dim3(TX, 4), kStepSmem<real, 4>, s>>>(lats, tiles, tile_offset, parity); break;
+    case 8: k_fused<real, 8><<<n_tiles, dim3(TX, 8), kStepSmem<real, 8>, s>>>(lats, tiles, tile_offset, parity); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -59,15 +81,15 @@ cudaError_t Launch<real>::persistent(const Lat<real> *lats, const int4 *tiles, c
     PersistCtl *c = (PersistCtl *)ctl;
     switch (ty) {
     case 2:
-        k_persistent<real, 2><<<blocks, dim3(TX, 2), 0, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
+        k_persistent<real, 2><<<blocks, dim3(TX, 2), kStepSmem<real, 2>, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
                                                               coll_done, err, wait_cycles, drop_tile);
         break;
     case 4:
-        k_persistent<real, 4><<<blocks, dim3(TX, 4), 0, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
+        k_persistent<real, 4><<<blocks, dim3(TX, 4), kStepSmem<real, 4>, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
                                                               coll_done, err, wait_cycles, drop_tile);
         break;
     case 8:
-        k_persistent<real, 8><<<blocks, dim3(TX, 8), 0, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
+        k_persistent<real, 8><<<blocks, dim3(TX, 8), kStepSmem<real, 8>, s>>>(lats, tiles, lat_ntiles, n_tiles, nsteps, parity0, c, dens_done,
                                                               coll_done, err, wait_cycles, drop_tile);
         break;
     default: return cudaErrorInvalidValue;
@@ -80,9 +102,9 @@ int Launch<real>::persistent_blocks_per_sm(int ty)
 {
     int n = 0;
     cudaError_t e = cudaErrorInvalidValue;
-    if (ty == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 2>, TX * 2, 0);
-    if (ty == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 4>, TX * 4, 0);
-    if (ty == 8) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 8>, TX * 8, 0);
+    if (ty == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 2>, TX * 2, kStepSmem<real, 2>);
+    if (ty == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 4>, TX * 4, kStepSmem<real, 4>);
+    if (ty == 8) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_persistent<real, 8>, TX * 8, kStepSmem<real, 8>);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -62,7 +62,7 @@ __device__ __forceinline__ void stage_from_pops(const lbk::Lat<double> &L, const
             for (int k = 0; k < 2; ++k) {
                 double v[9];
                 for (int i = 0; i < 9; ++i) v[i] = f[(size_t)(k * 9 + i) * n + c];
-                r[k] = zeroth_moment<double>(v);
+                r[k] = zeroth_moment<double>(v, 1.0);
             }
         }
         for (int k = 0; k < 2; ++k) {

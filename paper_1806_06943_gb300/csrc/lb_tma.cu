@@ -125,24 +125,6 @@ struct PairStage {
     }
 };
 
-// Staged slot (sx, sy) of the h-th position of the halo ring: two rows above,
-// two below, then the two columns on each side of the tile's rows.
-template <int TYv>
-__device__ __forceinline__ void ring_slot(int h, int &sx, int &sy)
-{
-    if (h < 2 * SW) {
-        sy = h / SW;
-        sx = h % SW;
-    } else if (h < 4 * SW) {
-        sy = TYv + HALO + (h - 2 * SW) / SW;
-        sx = (h - 2 * SW) % SW;
-    } else {
-        const int q = h - 4 * SW;
-        sy = HALO + q / 4;
-        sx = (q % 4 < 2) ? q % 4 : TX + q % 4;
-    }
-}
-
 // The slot's node lies beyond the lattice (across a periodic edge, or a wall
 // ghost row): not in the box's lattice part.
 __device__ __forceinline__ bool slot_outside(const Lat<float> &G, int4 t, int sx, int sy)
@@ -196,8 +178,7 @@ __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ la
             v[i] = make_float2(pop[(i * H + sy) * W + sx + 2], pop[((9 + i) * H + sy) * W + sx + 2]);
         return vadd(make_float2(ref[sy * W + sx + 2], ref[(H + sy) * W + sx + 2]), vzeroth<float2>(v));
     };
-    constexpr int kRing = 4 * SW + 4 * TYv;
-    for (int h = tid; h < kRing; h += TX * TYv) {
+    for (int h = tid; h < kRing<TYv>; h += TX * TYv) {
         int sx, sy;
         ring_slot<TYv>(h, sx, sy);
         if (slot_outside(G, t, sx, sy)) continue;
@@ -208,8 +189,8 @@ __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ la
     __syncthreads();
     const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
     const PairStage<SHv> sg{sm.sr, sm.sp};
-    if (inner) collide_site<float, true, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
-    else collide_site<float, false, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
+    if (inner) collide_site<true, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
+    else collide_site<false, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
 }
 
 // One block per tile: thread 0 starts the two copies, every thread waits
@@ -263,8 +244,7 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     {
         const Lat<float> &G = lats[t.x];
         if (good && (t.y == 0 || t.y + TX + HALO > G.nx || t.z < HALO || t.z + TYv + HALO > G.ny)) {
-            constexpr int kRing = 4 * SW + 4 * TYv;
-            for (int h = tid; h < kRing; h += TX * TYv) {
+            for (int h = tid; h < kRing<TYv>; h += TX * TYv) {
                 int sx, sy;
                 ring_slot<TYv>(h, sx, sy);
                 if (slot_outside(G, t, sx, sy)) {

@@ -5,7 +5,8 @@
 //   populations  f[species][dir][y][pitch]   two ping-pong copies
 //   densities    rho[species][y][pitch]       two copies: the density pass of
 //                                              a step with parity p writes copy
-//                                              p^1, the fused kernel reads it
+//                                              p^1, the fused kernel reads it;
+//                                              FP64: psi in copy p
 // pitch = nx rounded up to 32 elements, so every row starts on a 128-byte
 // (FP32) or 256-byte (FP64) boundary and a warp's row segment is one or two
 // full cache lines.  A batch of lattices shares one allocation; each lattice
@@ -43,6 +44,7 @@ struct Lat {
     int32_t tile_begin, tile_end;
     int32_t has_probe;
     int32_t forcing;     // 0 Guo forcing (Eqs. 5, 6), 1 velocity shift (Eq. 4; FP64 only)
+    int32_t products;    // FP64: the lattice's constants lie where integer products may be used (lb_f64.cuh)
     // model parameters in the compute precision
     real omega[2];       // 1 / tau_k
     real tau[2];         // tau_k (the velocity shift tau_k F_k / rho_k of Eq. 4)
@@ -52,6 +54,7 @@ struct Lat {
     real G1, G2, GAB;
     real g[2];
     real wall_rho[2];
+    real one;            // 1: a register operand the FP64 sums are formed with (lb_f64.cuh)
     // observable settings, always FP64
     double probe[3];     // cx, cy, R
     double tau_B;        // for the closed-form flux Q0
