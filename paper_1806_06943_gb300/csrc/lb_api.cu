@@ -48,6 +48,8 @@ constexpr int kGraphSteps = 32;   // steps per captured graph (even: parity retu
 constexpr int kPersistSteps = 64; // time steps per persistent launch
 constexpr int kChains = 2;         // chains of time steps of a batch's step graph
 constexpr int kTileHeights[3] = {2, 4, 8};
+// rows of 32 nodes per SM up to which an FP64 step runs as k_small64
+constexpr int kSmallRowsPerSm = 3;
 
 int ty_index(int ty) { return ty == 2 ? 0 : (ty == 4 ? 1 : (ty == 8 ? 2 : -1)); }
 constexpr size_t kAlign = 256;
@@ -182,6 +184,11 @@ struct lb_engine {
     lbk::TmaMaps *d_tmaps = nullptr;
     int4 *d_btiles[3] = {nullptr, nullptr, nullptr};
     int n_box[3] = {0, 0, 0};
+    // FP64 lattices of few nodes: one-row tiles (chain by chain for a batch)
+    // of k_small64, which both LB_MODE_LAUNCH and LB_MODE_FUSED then step with
+    int4 *d_rows = nullptr;
+    int n_rows = 0;
+    int r_off[kChains] = {}, r_cnt[kChains] = {};
     bool tma_ok = false;
     std::string tma_why = "LB_MODE_TMA needs LB_FP32 populations";
     double *d_partials = nullptr;
@@ -216,6 +223,7 @@ struct lb_engine {
             cudaFree(d_sntiles[i]);
             cudaFree(d_btiles[i]);
         }
+        cudaFree(d_rows);
         cudaFree(d_ctl);
         cudaFree(d_err);
         cudaFree(d_pool);
@@ -277,6 +285,7 @@ struct lb_engine {
         cudaError_t e;
         if (precision == LB_FP64) {
             const lbk::Lat<double> *L = (const lbk::Lat<double> *)d_lats;
+            if (n_rows) return lbk::Launch<double>::small(L, d_rows, 0, n_rows, par, stream);
             if (mode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, d_stiles[ti], 0, nt, par, ty, stream);
             e = lbk::Launch<double>::density(L, d_stiles[ti], 0, nt, par, ty, stream);
             if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, d_stiles[ti], 0, nt, par, ty, stream);
@@ -326,6 +335,7 @@ struct lb_engine {
         cudaError_t e;
         if (precision == LB_FP64) {
             const lbk::Lat<double> *L = (const lbk::Lat<double> *)d_lats;
+            if (n_rows) return lbk::Launch<double>::small(L, d_rows, r_off[g], r_cnt[g], par, s);
             if (mode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, T, off, cnt, par, ty, s);
             e = lbk::Launch<double>::density(L, T, off, cnt, par, ty, s);
             if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, T, off, cnt, par, ty, s);
@@ -450,6 +460,37 @@ struct lb_engine {
             if (ce != cudaSuccess) return cuda_fail(ce, "TMA tile list upload");
         }
         tma_ok = true;
+        return LB_OK;
+    }
+
+    // Row tiles of k_small64 where the FP64 step of all lattices is short of
+    // nodes: up to kSmallRowsPerSm rows of 32 nodes per SM (a wave of one row
+    // per SM takes 15 k clocks, the tile kernels 40 k for their first wave of
+    // four).  The velocity-shift model stays on the tile kernels.
+    int build_rows(const std::vector<int> &chain)
+    {
+        if (precision != LB_FP64) return LB_OK;
+        int64_t rows = 0;
+        for (const lb_params &p : P) {
+            if (p.forcing != LB_FORCING_GUO) return LB_OK;
+            rows += (int64_t)((p.nx + lbk::TX - 1) / lbk::TX) * p.ny;
+        }
+        if (rows > (int64_t)kSmallRowsPerSm * sm_count) return LB_OK;
+        std::vector<int4> list;
+        for (int g = 0; g < nchains; ++g) {
+            r_off[g] = (int)list.size();
+            for (int l = 0; l < n; ++l)
+                for (int y = 0; chain[l] == g && y < P[l].ny; ++y)
+                    for (int x0 = 0; x0 < P[l].nx; x0 += lbk::TX) list.push_back(make_int4(l, x0, y, 0));
+            r_cnt[g] = (int)list.size() - r_off[g];
+        }
+        if (cudaMalloc((void **)&d_rows, list.size() * sizeof(int4)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(LB_ENOMEM, "cudaMalloc of the row list failed");
+        }
+        LB_CUDA(cudaMemcpyAsync(d_rows, list.data(), list.size() * sizeof(int4), cudaMemcpyHostToDevice, stream));
+        LB_CUDA(cudaStreamSynchronize(stream));
+        n_rows = (int)list.size();
         return LB_OK;
     }
 
@@ -1253,6 +1294,8 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
         const int rc = e->build_tma_maps();
         if (rc) return bail(rc);
     }
+    std::vector<int> chain_of(n, 0);
+    int rc = LB_OK;
     // the chains of a batch's step graph (as many as lattices, at most
     // kChains): lattices by node count, each to the group with the fewest
     // nodes so far
@@ -1300,7 +1343,9 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
                 (ce = cudaEventCreateWithFlags(&e->ev_join[g], cudaEventDisableTiming)) != cudaSuccess)
                 return bail(cuda_fail(ce, "auxiliary streams of the step graph"));
         e->nchains = nc;
+        chain_of = group;
     }
+    if ((rc = e->build_rows(chain_of))) return bail(rc);
     *out = e;
     return LB_OK;
 }

@@ -565,13 +565,14 @@ struct Stage64 {
 
     // density and psi of species k at a slot, and the slot's products;
     // nonzero where one lies outside the range of the integer products
+    template <bool kInt = true>
     __device__ __forceinline__ uint32_t put(int k, int sy, int sx, double r, double p)
     {
         double(*q)[TYv + 2 * HALO][SW] = v[k];
         q[sRho][sy][sx] = r;
         q[sPsi][sy][sx] = p;
-        const uint32_t outside = base_outside(r) | base_outside(p);
-        if (outside) {
+        const uint32_t outside = kInt ? base_outside(r) | base_outside(p) : 0u;
+        if (!kInt || outside) {
             q[sW1Psi][sy][sx] = (1.0 / 9.0) * p;
             q[sW2Psi][sy][sx] = (1.0 / 36.0) * p;
             q[sP1][sy][sx] = p25(1) * p;
@@ -597,98 +598,43 @@ struct Stage64 {
     }
 };
 
-// Total force on species k at the staged node, Eq. (8) + Eq. (9) + rho_k g:
-// the sums in direction order (D2Q9) and raster order (D2Q25), as q9_sum and
-// q25_sum form them, from the staged products.
-template <bool kInt, int TYv>
-__device__ __forceinline__ void force64(const Arith64<kInt> &A, const Stage64<TYv> &sm, int k, int cx, int cy, double &Fx,
-                                        double &Fy)
+// Component AX (0: x, 1: y) of the total force on species k at the staged
+// node, Eq. (8) + Eq. (9) + rho_k g: the sums in direction order (D2Q9) and
+// raster order (D2Q25), as q9_sum and q25_sum form them, from the staged
+// products.
+template <int AX, bool kInt, int TYv>
+__device__ __forceinline__ double force64(const Arith64<kInt> &A, const Stage64<TYv> &sm, int k, int cx, int cy)
 {
     const double(*q)[TYv + 2 * HALO][SW] = sm.v[k];
     const double(*o)[TYv + 2 * HALO][SW] = sm.v[1 - k];
-    auto at = [&](int plane, int dy, int dx) { return q[plane][cy + dy][cx + dx]; };
-    auto ot = [&](int plane, int dy, int dx) { return o[plane][cy + dy][cx + dx]; };
-    auto q9 = [&](auto &&g, int w1, int w2, double &sx, double &sy) {
-        const double a5 = g(w2, 1, 1), a6 = g(w2, 1, -1), a7 = g(w2, -1, -1), a8 = g(w2, -1, 1);
-        sx = A.add(A.sub(A.sub(A.add(A.sub(g(w1, 0, 1), g(w1, 0, -1)), a5), a6), a7), a8);
-        sy = A.sub(A.sub(A.add(A.add(A.sub(g(w1, 1, 0), g(w1, -1, 0)), a5), a6), a7), a8);
+    auto signed_add = [&](double s, double t, int e) { return e > 0 ? A.add(s, t) : A.sub(s, t); };
+    // D2Q9: the axis pair, then the diagonals in direction order
+    auto q9 = [&](const double(*f)[TYv + 2 * HALO][SW], int w1, int w2) {
+        double s = AX == 0 ? A.sub(f[w1][cy][cx + 1], f[w1][cy][cx - 1]) : A.sub(f[w1][cy + 1][cx], f[w1][cy - 1][cx]);
+#pragma unroll
+        for (int i = 5; i < 9; ++i) s = signed_add(s, f[w2][cy + ey9(i)][cx + ex9(i)], AX == 0 ? ex9(i) : ey9(i));
+        return s;
     };
-    double s1x, s1y, s2x, s2y, s3x, s3y;
-    q9(at, sW1Psi, sW2Psi, s1x, s1y);
-    q9(ot, sW1Rho, sW2Rho, s3x, s3y);
+    const double s1 = q9(q, sW1Psi, sW2Psi), s3 = q9(o, sW1Rho, sW2Rho);
+    // D2Q25: the planes of |e|^2 = 4, 8 hold 2 p psi, the component being +-2
     const double two = A.one + A.one;
-    {
-        // rows dy = -2 .. 2, columns dx = -2 .. 2 within a row; a term's
-        // component along an axis of reach 2 is twice p psi
-        double a, x, y;
-        a = at(s2P8, -2, -2);
-        x = -a;
-        y = -a;
-        a = at(sP5, -2, -1);
-        x = A.sub(x, a);
-        y = __fma_rn(-a, two, y);
-        y = A.sub(y, at(s2P4, -2, 0));
-        a = at(sP5, -2, 1);
-        x = A.add(x, a);
-        y = __fma_rn(-a, two, y);
-        a = at(s2P8, -2, 2);
-        x = A.add(x, a);
-        y = A.sub(y, a);
-
-        a = at(sP5, -1, -2);
-        x = __fma_rn(-a, two, x);
-        y = A.sub(y, a);
-        a = at(sP2, -1, -1);
-        x = A.sub(x, a);
-        y = A.sub(y, a);
-        y = A.sub(y, at(sP1, -1, 0));
-        a = at(sP2, -1, 1);
-        x = A.add(x, a);
-        y = A.sub(y, a);
-        a = at(sP5, -1, 2);
-        x = __fma_rn(a, two, x);
-        y = A.sub(y, a);
-
-        x = A.sub(x, at(s2P4, 0, -2));
-        x = A.sub(x, at(sP1, 0, -1));
-        x = A.add(x, at(sP1, 0, 1));
-        x = A.add(x, at(s2P4, 0, 2));
-
-        a = at(sP5, 1, -2);
-        x = __fma_rn(-a, two, x);
-        y = A.add(y, a);
-        a = at(sP2, 1, -1);
-        x = A.sub(x, a);
-        y = A.add(y, a);
-        y = A.add(y, at(sP1, 1, 0));
-        a = at(sP2, 1, 1);
-        x = A.add(x, a);
-        y = A.add(y, a);
-        a = at(sP5, 1, 2);
-        x = __fma_rn(a, two, x);
-        y = A.add(y, a);
-
-        a = at(s2P8, 2, -2);
-        x = A.sub(x, a);
-        y = A.add(y, a);
-        a = at(sP5, 2, -1);
-        x = A.sub(x, a);
-        y = __fma_rn(a, two, y);
-        y = A.add(y, at(s2P4, 2, 0));
-        a = at(sP5, 2, 1);
-        x = A.add(x, a);
-        y = __fma_rn(a, two, y);
-        a = at(s2P8, 2, 2);
-        s2x = A.add(x, a);
-        s2y = A.add(y, a);
+    double s2 = 0.0;
+#pragma unroll
+    for (int j = 0; j < 25; ++j) {
+        const int dx = j % 5 - 2, dy = j / 5 - 2, e2 = dx * dx + dy * dy, e = AX == 0 ? dx : dy;
+        if (e == 0) continue;
+        const int plane = e2 == 1 ? sP1 : e2 == 2 ? sP2 : e2 == 4 ? s2P4 : e2 == 5 ? sP5 : s2P8;
+        const double t = q[plane][cy + dy][cx + dx];
+        if (j == 0) s2 = -t;
+        else if (e2 == 5 && (e == 2 || e == -2)) s2 = __fma_rn(e > 0 ? t : -t, two, s2);
+        else s2 = signed_add(s2, t, e);
     }
     const double psi = q[sPsi][cy][cx], rho = q[sRho][cy][cx];
-    const double c1 = A.mul(-sm.L.G1, psi), c2 = A.mul(sm.L.G2, psi), c3 = A.mul(sm.L.GAB, rho);
-    Fx = A.sub(A.sub(A.mul(c1, s1x), A.mul(c2, s2x)), A.mul(c3, s3x));
-    Fy = A.sub(A.sub(A.mul(c1, s1y), A.mul(c2, s2y)), A.mul(c3, s3y));
+    double F = A.sub(A.sub(A.mul(A.mul(-sm.L.G1, psi), s1), A.mul(A.mul(sm.L.G2, psi), s2)),
+                     A.mul(A.mul(sm.L.GAB, rho), s3));
     // + rho g; a zero component adds nothing to a finite force
-    if (!kInt || sm.L.g[0] != 0.0) Fx = A.add(Fx, A.mul(rho, sm.L.g[0]));
-    if (!kInt || sm.L.g[1] != 0.0) Fy = A.add(Fy, A.mul(rho, sm.L.g[1]));
+    if (!kInt || sm.L.g[AX] != 0.0) F = A.add(F, A.mul(rho, sm.L.g[AX]));
+    return F;
 }
 
 // Where the node's pushes go: element offsets to its neighbours, and whether
@@ -722,6 +668,53 @@ struct Push64 {
     }
 };
 
+// What the directions of the collision share: the velocity's terms of the Guo
+// vectors (e - u)/cs^2 + (e.u) e/cs^4 and of the equilibrium polynomial.
+// Opposite directions' e.u differ by an exact sign.
+template <bool kInt>
+struct Dirs64 {
+    double e[4];            // e.u of directions 1, 2, 5, 8
+    double uu15;            // 1.5 u.u
+    double g0[2];           // -3 u
+    double gp[2], gm[2];    // 3 (1 - u), 3 (-1 - u)
+    __device__ __forceinline__ Dirs64(const Arith64<kInt> &A, double ux, double uy)
+        : e{ux, uy, A.add(ux, uy), A.sub(ux, uy)}, uu15(A.mul(1.5, A.add(A.mul(ux, ux), A.mul(uy, uy)))),
+          g0{-A.mul(3.0, ux), -A.mul(3.0, uy)}, gp{A.mul(3.0, A.sub(1.0, ux)), A.mul(3.0, A.sub(1.0, uy))},
+          gm{A.mul(3.0, A.sub(-1.0, ux)), A.mul(3.0, A.sub(-1.0, uy))}
+    {
+    }
+    // Guo vector and 1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u.u of direction I
+    template <int I>
+    __device__ __forceinline__ void terms(const Arith64<kInt> &A, double (&g)[2], double &po) const
+    {
+        if constexpr (I == 0) {
+            g[0] = g0[0];
+            g[1] = g0[1];
+            po = A.sub(1.0, uu15);
+        } else {
+            constexpr int B = vbase9(I), S = vsign9(I) > 0 ? 1 : -1, E[2] = {ex9(I), ey9(I)};   // e.u = S e[B]
+            const double e9 = A.mul(9.0, e[B]), e3 = A.mul(3.0, e[B]);
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                g[a] = E[a] == 0 ? g0[a]
+                                 : (E[a] * S > 0 ? A.add(E[a] > 0 ? gp[a] : gm[a], e9)
+                                                 : A.sub(E[a] > 0 ? gp[a] : gm[a], e9));
+            const double lin = S > 0 ? A.add(1.0, e3) : A.sub(1.0, e3);
+            po = A.sub(A.add(lin, A.mul(A.mul(4.5, e[B]), e[B])), uu15);
+        }
+    }
+};
+
+// Post-collision value of direction I of one species (Eqs. 1, 2, 5):
+// f - omega (f - feq) + C, feq = w rho po, C = (1 - omega/2) w (g . F).
+template <int I, bool kInt>
+__device__ __forceinline__ double relax64(const Arith64<kInt> &A, double f, double wrho, double om, double aw,
+                                          const double (&g)[2], double po, double Fx, double Fy)
+{
+    const double C = A.mul(aw, A.add(A.mul(g[0], Fx), A.mul(g[1], Fy)));
+    return A.add(A.sub(f, A.mul(om, A.sub(f, A.mul(wrho, po)))), C);
+}
+
 // Force, half-force momenta, u^eq, collision with the Guo term and push of
 // both species at node (x, y), staged at (cx, cy): Eqs. (1)-(3), (5), (6),
 // (8), (9), operation by operation as collide_dir writes them.  j: the
@@ -740,7 +733,8 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
     double F[2][2], m[2][2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        force64<kInt, TYv>(A, sm, k, cx, cy, F[k][0], F[k][1]);
+        F[k][0] = force64<0, kInt, TYv>(A, sm, k, cx, cy);
+        F[k][1] = force64<1, kInt, TYv>(A, sm, k, cx, cy);
 #pragma unroll
         for (int a = 0; a < 2; ++a) m[k][a] = __fma_rn(0.5, F[k][a], j[k][a]);   // Eq. (6): F/2 is exact
     }
@@ -752,31 +746,17 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
     if constexpr (kInt) {
         outside = velocity_outside(ux) | velocity_outside(uy);
     }
-    const double uu15 = A.mul(1.5, A.add(A.mul(ux, ux), A.mul(uy, uy)));
-    // e.u of the diagonals; opposite directions differ by an exact sign
-    const double s = A.add(ux, uy), d = A.sub(ux, uy);
-    // the Guo vectors (e - u)/cs^2 + (e.u) e/cs^4
-    const double gx0 = -A.mul(3.0, ux), gy0 = -A.mul(3.0, uy);
-    const double xp = A.mul(3.0, A.sub(1.0, ux)), xm = A.mul(3.0, A.sub(-1.0, ux));
-    const double yp = A.mul(3.0, A.sub(1.0, uy)), ym = A.mul(3.0, A.sub(-1.0, uy));
-    const double x9 = A.mul(9.0, ux), y9 = A.mul(9.0, uy), s9 = A.mul(9.0, s), d9 = A.mul(9.0, d);
-    const double gx[9] = {gx0, A.add(xp, x9), gx0, A.add(xm, x9), gx0, A.add(xp, s9), A.add(xm, d9), A.add(xm, s9),
-                          A.add(xp, d9)};
-    const double gy[9] = {gy0, gy0, A.add(yp, y9), gy0, A.add(ym, y9), A.add(yp, s9), A.sub(yp, d9), A.add(ym, s9),
-                          A.sub(ym, d9)};
-    // 1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u.u
-    double po[9];
-    po[0] = A.sub(1.0, uu15);
-    {
-        const double e[4] = {ux, uy, s, d};
-        constexpr int plus[4] = {1, 2, 5, 8}, minus[4] = {3, 4, 7, 6};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const double e3 = A.mul(3.0, e[q]), ee = A.mul(A.mul(4.5, e[q]), e[q]);
-            po[plus[q]] = A.sub(A.add(A.add(1.0, e3), ee), uu15);
-            po[minus[q]] = A.sub(A.add(A.sub(1.0, e3), ee), uu15);
-        }
-    }
+    const Dirs64<kInt> dirs(A, ux, uy);
+    double g[9][2], po[9];
+    dirs.template terms<0>(A, g[0], po[0]);
+    dirs.template terms<1>(A, g[1], po[1]);
+    dirs.template terms<2>(A, g[2], po[2]);
+    dirs.template terms<3>(A, g[3], po[3]);
+    dirs.template terms<4>(A, g[4], po[4]);
+    dirs.template terms<5>(A, g[5], po[5]);
+    dirs.template terms<6>(A, g[6], po[6]);
+    dirs.template terms<7>(A, g[7], po[7]);
+    dirs.template terms<8>(A, g[8], po[8]);
     const Push64 push(L, x, y);
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
@@ -791,15 +771,11 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
 #pragma unroll
             for (int i = 0; i < 9; ++i) outside |= base_outside(f[i]);
         }
-        const double p0x = A.mul(gx0, Fx), p0y = A.mul(gy0, Fy);
         const double wr[3] = {A.mul(4.0 / 9.0, r), A.mul(1.0 / 9.0, r), A.mul(1.0 / 36.0, r)};
         const double aw[3] = {L.aw[k][0], L.aw[k][1], L.aw[k][2]};
         auto dir = [&](auto Ic) {
             constexpr int I = decltype(Ic)::value, c = cls9(I);
-            const double gFx = ex9(I) == 0 ? p0x : A.mul(gx[I], Fx), gFy = ey9(I) == 0 ? p0y : A.mul(gy[I], Fy);
-            const double C = A.mul(aw[c], A.add(gFx, gFy));
-            const double feq = A.mul(wr[c], po[I]);
-            push.store<I>(nk, plane, A.add(A.sub(f[I], A.mul(om, A.sub(f[I], feq))), C));
+            push.store<I>(nk, plane, relax64<I>(A, f[I], wr[c], om, aw[c], g[I], po[I], Fx, Fy));
         };
         dir(std::integral_constant<int, 0>{});
         dir(std::integral_constant<int, 1>{});
@@ -830,7 +806,8 @@ __device__ __noinline__ void shift_node64(const Stage64<TYv> &sm, double one, co
     double F[2][2], rho[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        force64<false, TYv>(A, sm, k, cx, cy, F[k][0], F[k][1]);
+        F[k][0] = force64<0, false, TYv>(A, sm, k, cx, cy);
+        F[k][1] = force64<1, false, TYv>(A, sm, k, cx, cy);
         rho[k] = sm.v[k][sRho][cy][cx];
     }
     const double om0 = L.omega[0], om1 = L.omega[1];
@@ -901,32 +878,34 @@ __device__ __forceinline__ real node_density(const Lat<real> &L, int k, int gx, 
     return r;
 }
 
-// Densities of staged slot (sx, sy) of tile t (slot (HALO, HALO) is the
-// tile's first node) from the populations of its node: x wraps; beyond the
-// lattice in y, periodic wrap, or a wall ghost row (the mirrored fluid row,
-// or the fixed wall densities).
+// Density of species k at staged slot (sx, sy) of tile t (slot (HALO, HALO)
+// is the tile's first node) from the populations of its node: x wraps; beyond
+// the lattice in y, periodic wrap, or a wall ghost row (the mirrored fluid
+// row, or the fixed wall densities).
 template <typename real, bool kCG>
-__device__ __forceinline__ void slot_densities(const Lat<real> &G, int4 t, int parity, int sx, int sy, real &rA,
-                                               real &rB)
+__device__ __forceinline__ real slot_density(const Lat<real> &G, int4 t, int parity, int sx, int sy, int k)
 {
     const int nx = G.nx, ny = G.ny;
     const int gx = wrap_index(t.y + sx - HALO, nx);
     int gy = t.z + sy - HALO;
     if (gy < 0 || gy >= ny) {
         if (G.walls) {
-            if (G.wall_mode == 1) {
-                rA = G.wall_rho[0];
-                rB = G.wall_rho[1];
-                return;
-            }
+            if (G.wall_mode == 1) return G.wall_rho[k];
             gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
             gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);  // rows no valid node reads
         } else {
             gy = wrap_index(gy, ny);
         }
     }
-    rA = node_density<real, kCG>(G, 0, gx, gy, parity);
-    rB = node_density<real, kCG>(G, 1, gx, gy, parity);
+    return node_density<real, kCG>(G, k, gx, gy, parity);
+}
+
+template <typename real, bool kCG>
+__device__ __forceinline__ void slot_densities(const Lat<real> &G, int4 t, int parity, int sx, int sy, real &rA,
+                                               real &rB)
+{
+    rA = slot_density<real, kCG>(G, t, parity, sx, sy, 0);
+    rB = slot_density<real, kCG>(G, t, parity, sx, sy, 1);
 }
 
 // Staged slot (sx, sy) of the h-th position of a tile's halo ring, enumerated
@@ -1181,6 +1160,88 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
     auto &sm = step_smem<real, TYv>();
     if constexpr (kOffset<real>) fused_tile<TYv, false>(lats, t, parity, sm);
     else fused_tile64<TYv, false>(lats, t, parity, sm);
+}
+
+// ---- the FP64 step of small lattices ------------------------------------------
+//
+// One warp issues an FP64 instruction every 64 clocks, whatever its
+// neighbours do (each of an SM's four schedulers has a quarter of the pipe), so
+// a lattice of few nodes is bound by the FP64 instructions of one warp: 435 a
+// node with the products on the pipe, 20 us.  Here a row of 32 nodes is a
+// block of four warps, one per scheduler: warp (k, a) forms component a of
+// species k's force and momentum, then half a's directions of species k.  A
+// step is this one launch; the densities of the row's 36 x 5 slots are formed
+// by the block itself.  Every operation is that of node64<false>.
+constexpr int kSmallWarps = 4;
+
+struct Small64 {
+    Stage64<1> st;
+    double F[2][2][TX], m[2][2][TX], u[2][TX];
+};
+
+template <int kWarps>
+__global__ void __launch_bounds__(TX *kWarps, 2)
+    k_small64(const Lat<double> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity)
+{
+    static_assert(kWarps == 4, "two species, two components");
+    extern __shared__ __align__(16) unsigned char lb_step_smem[];
+    Small64 &sm = *reinterpret_cast<Small64 *>(lb_step_smem);
+    const int4 t = tiles[tile_offset + blockIdx.x];
+    const Lat<double> &G = lats[t.x];
+    const int lane = threadIdx.x, k = threadIdx.y & 1, a = threadIdx.y >> 1;
+    const int tid = threadIdx.y * TX + lane;
+    for (int i = tid; i < (int)(sizeof(Lat<double>) / 4); i += TX * kWarps)
+        reinterpret_cast<uint32_t *>(&sm.st.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
+    const int x = t.y + lane, y = t.z, cx = lane + HALO, cy = HALO;
+    const bool valid = x < G.nx;
+    const size_t plane = G.plane, c = valid ? (size_t)y * G.pitch + x : 0;
+    const double *__restrict__ fk = G.f[parity] + (size_t)(k * 9) * plane + c;
+    double f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = fk[(size_t)i * plane];
+    const Arith64<false> A(G.one);
+    for (int q = tid; q < 2 * SW * (1 + 2 * HALO); q += TX * kWarps) {
+        const int sp = q / (SW * (1 + 2 * HALO)), slot = q % (SW * (1 + 2 * HALO)), sx = slot % SW, sy = slot / SW;
+        const double r = slot_density<double, false>(G, t, parity, sx, sy, sp);
+        sm.st.put<false>(sp, sy, sx, r, psi_of<double>(r));
+    }
+    __syncthreads();
+    const Lat<double> &L = sm.st.L;
+    const double j = a == 0 ? A.add(A.sub(A.sub(A.add(A.sub(f[1], f[3]), f[5]), f[6]), f[7]), f[8])
+                            : A.sub(A.sub(A.add(A.add(A.sub(f[2], f[4]), f[5]), f[6]), f[7]), f[8]);
+    const double Fa = a == 0 ? force64<0, false, 1>(A, sm.st, k, cx, cy) : force64<1, false, 1>(A, sm.st, k, cx, cy);
+    sm.F[k][a][lane] = Fa;
+    sm.m[k][a][lane] = __fma_rn(0.5, Fa, j);   // Eq. (6)
+    __syncthreads();
+    if (k == 0) {   // component a of u^eq, Eq. (3)
+        const double om0 = L.omega[0], om1 = L.omega[1];
+        const double den = A.add(A.mul(om0, sm.st.v[0][sRho][cy][cx]), A.mul(om1, sm.st.v[1][sRho][cy][cx]));
+        sm.u[a][lane] = A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane])) / den;
+    }
+    __syncthreads();
+    if (!valid) return;
+    const Dirs64<false> dirs(A, sm.u[0][lane], sm.u[1][lane]);
+    const double r = sm.st.v[k][sRho][cy][cx], om = L.omega[k], Fx = sm.F[k][0][lane], Fy = sm.F[k][1][lane];
+    const Push64 push(L, x, y);
+    double *__restrict__ nk = L.f[parity ^ 1] + (size_t)(k * 9) * plane + c;
+    auto dir = [&](auto Ic) {
+        constexpr int I = decltype(Ic)::value;
+        double g[2], po;
+        dirs.template terms<I>(A, g, po);
+        push.store<I>(nk, plane, relax64<I>(A, f[I], A.mul(w9(I), r), om, L.aw[k][cls9(I)], g, po, Fx, Fy));
+    };
+    if (a == 0) {   // the directions along e[0] and e[2], and rest
+        dir(std::integral_constant<int, 0>{});
+        dir(std::integral_constant<int, 1>{});
+        dir(std::integral_constant<int, 3>{});
+        dir(std::integral_constant<int, 5>{});
+        dir(std::integral_constant<int, 7>{});
+    } else {
+        dir(std::integral_constant<int, 2>{});
+        dir(std::integral_constant<int, 4>{});
+        dir(std::integral_constant<int, 6>{});
+        dir(std::integral_constant<int, 8>{});
+    }
 }
 
 // ---- persistent launch over many time steps -----------------------------------

@@ -26,6 +26,9 @@ cudaError_t Launch<real>::prepare()
     cudaError_t e = prepare_height<real, 2>();
     if (e == cudaSuccess) e = prepare_height<real, 4>();
     if (e == cudaSuccess) e = prepare_height<real, 8>();
+    if constexpr (!kOffset<real>)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_small64<kSmallWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Small64));
     return e;
 }
 
@@ -69,6 +72,19 @@ cudaError_t Launch<real>::fused(const Lat<real> *lats, const int4 *tiles, int ti
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+template <typename real>
+cudaError_t Launch<real>::small(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
+                                cudaStream_t s)
+{
+    if (n_tiles <= 0) return cudaSuccess;
+    if constexpr (kOffset<real>) {
+        return cudaErrorInvalidValue;
+    } else {
+        k_small64<kSmallWarps><<<n_tiles, dim3(TX, kSmallWarps), sizeof(Small64), s>>>(lats, tiles, tile_offset, parity);
+        return cudaGetLastError();
+    }
 }
 
 template <typename real>
