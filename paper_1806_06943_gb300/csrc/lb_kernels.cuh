@@ -565,14 +565,13 @@ struct Stage64 {
 
     // density and psi of species k at a slot, and the slot's products;
     // nonzero where one lies outside the range of the integer products
-    template <bool kInt = true>
     __device__ __forceinline__ uint32_t put(int k, int sy, int sx, double r, double p)
     {
         double(*q)[TYv + 2 * HALO][SW] = v[k];
         q[sRho][sy][sx] = r;
         q[sPsi][sy][sx] = p;
-        const uint32_t outside = kInt ? base_outside(r) | base_outside(p) : 0u;
-        if (!kInt || outside) {
+        const uint32_t outside = base_outside(r) | base_outside(p);
+        if (outside) {
             q[sW1Psi][sy][sx] = (1.0 / 9.0) * p;
             q[sW2Psi][sy][sx] = (1.0 / 36.0) * p;
             q[sP1][sy][sx] = p25(1) * p;
@@ -1166,18 +1165,92 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
 //
 // One warp issues an FP64 instruction every 64 clocks, whatever its
 // neighbours do (each of an SM's four schedulers has a quarter of the pipe), so
-// a lattice of few nodes is bound by the FP64 instructions of one warp: 435 a
-// node with the products on the pipe, 20 us.  Here a row of 32 nodes is a
-// block of four warps, one per scheduler: warp (k, a) forms component a of
-// species k's force and momentum, then half a's directions of species k.  A
-// step is this one launch; the densities of the row's 36 x 5 slots are formed
-// by the block itself.  Every operation is that of node64<false>.
+// a lattice of few nodes is bound by the instructions of one warp: 13 us of
+// FP64 alone.  Here a row of 32 nodes is a block of four warps, one per
+// scheduler: warp (k, a) forms component a of species k's force and momentum,
+// then half a's directions of species k.  A step is this one launch; the
+// densities of the row's 36 x 5 slots are formed by the block itself.  Every
+// operation is that of node64.  64^2: 25.6 us a step as tiles of 32 x 4 nodes
+// in two launches, 13.4 here with the products on the FP64 pipe, 12.0 with
+// them in integers, which fill the 64 clocks between FP64 instructions
+// (unrolling the staging loop: 14.1, its code outgrows the instruction cache).
 constexpr int kSmallWarps = 4;
 
 struct Small64 {
     Stage64<1> st;
     double F[2][2][TX], m[2][2][TX], u[2][TX];
 };
+
+// The populations of one species at a node.
+struct Pops64 {
+    double f[9];
+};
+
+// Component a of species k's force and half-force momentum (Eqs. 6, 8, 9).
+template <bool kInt>
+__device__ __forceinline__ void small_force(Small64 &sm, const Pops64 &p, int k, int a)
+{
+    const Arith64<kInt> A(sm.st.L.one);
+    const int lane = threadIdx.x, cx = lane + HALO, cy = HALO;
+    const double(&f)[9] = p.f;
+    const double j = a == 0 ? A.add(A.sub(A.sub(A.add(A.sub(f[1], f[3]), f[5]), f[6]), f[7]), f[8])
+                            : A.sub(A.sub(A.add(A.add(A.sub(f[2], f[4]), f[5]), f[6]), f[7]), f[8]);
+    const double F = a == 0 ? force64<0, kInt, 1>(A, sm.st, k, cx, cy) : force64<1, kInt, 1>(A, sm.st, k, cx, cy);
+    sm.F[k][a][lane] = F;
+    sm.m[k][a][lane] = __fma_rn(0.5, F, j);
+}
+
+// Component a of u^eq (Eq. 3).
+template <bool kInt>
+__device__ __forceinline__ double small_velocity(const Small64 &sm, int a)
+{
+    const Arith64<kInt> A(sm.st.L.one);
+    const int lane = threadIdx.x, cx = lane + HALO, cy = HALO;
+    const double om0 = sm.st.L.omega[0], om1 = sm.st.L.omega[1];
+    const double den = A.add(A.mul(om0, sm.st.v[0][sRho][cy][cx]), A.mul(om1, sm.st.v[1][sRho][cy][cx]));
+    return A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane])) / den;
+}
+
+// Collision and push of half a's directions of species k at node (x, y):
+// those along e[0] and e[2] of Dirs64 and rest, or those along e[1] and e[3].
+template <bool kInt>
+__device__ __forceinline__ void small_push(const Small64 &sm, const Pops64 &p, double *__restrict__ nk, int k, int a,
+                                           int x, int y)
+{
+    const Lat<double> &L = sm.st.L;
+    const Arith64<kInt> A(L.one);
+    const int lane = threadIdx.x;
+    const Dirs64<kInt> dirs(A, sm.u[0][lane], sm.u[1][lane]);
+    const double r = sm.st.v[k][sRho][HALO][lane + HALO], om = L.omega[k], Fx = sm.F[k][0][lane], Fy = sm.F[k][1][lane];
+    const Push64 push(L, x, y);
+    auto dir = [&](auto Ic) {
+        constexpr int I = decltype(Ic)::value;
+        double g[2], po;
+        dirs.template terms<I>(A, g, po);
+        push.store<I>(nk, L.plane, relax64<I>(A, p.f[I], A.mul(w9(I), r), om, L.aw[k][cls9(I)], g, po, Fx, Fy));
+    };
+    if (a == 0) {
+        dir(std::integral_constant<int, 0>{});
+        dir(std::integral_constant<int, 1>{});
+        dir(std::integral_constant<int, 3>{});
+        dir(std::integral_constant<int, 5>{});
+        dir(std::integral_constant<int, 7>{});
+    } else {
+        dir(std::integral_constant<int, 2>{});
+        dir(std::integral_constant<int, 4>{});
+        dir(std::integral_constant<int, 6>{});
+        dir(std::integral_constant<int, 8>{});
+    }
+}
+
+// The same on the FP64 pipe, out of line: for blocks with a value outside the
+// range of the integer products.
+static __device__ __noinline__ void small_force_plain(Small64 &sm, Pops64 p, int k, int a) { small_force<false>(sm, p, k, a); }
+static __device__ __noinline__ double small_velocity_plain(const Small64 &sm, int a) { return small_velocity<false>(sm, a); }
+static __device__ __noinline__ void small_push_plain(const Small64 &sm, Pops64 p, double *nk, int k, int a, int x, int y)
+{
+    small_push<false>(sm, p, nk, k, a, x, y);
+}
 
 template <int kWarps>
 __global__ void __launch_bounds__(TX *kWarps, 2)
@@ -1192,56 +1265,37 @@ __global__ void __launch_bounds__(TX *kWarps, 2)
     const int tid = threadIdx.y * TX + lane;
     for (int i = tid; i < (int)(sizeof(Lat<double>) / 4); i += TX * kWarps)
         reinterpret_cast<uint32_t *>(&sm.st.L)[i] = reinterpret_cast<const uint32_t *>(&G)[i];
-    const int x = t.y + lane, y = t.z, cx = lane + HALO, cy = HALO;
+    const int x = t.y + lane, y = t.z;
     const bool valid = x < G.nx;
     const size_t plane = G.plane, c = valid ? (size_t)y * G.pitch + x : 0;
     const double *__restrict__ fk = G.f[parity] + (size_t)(k * 9) * plane + c;
-    double f[9];
+    Pops64 p;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) f[i] = fk[(size_t)i * plane];
-    const Arith64<false> A(G.one);
+    for (int i = 0; i < 9; ++i) p.f[i] = fk[(size_t)i * plane];
+    uint32_t outside = G.products ? 0u : 1u;
+#pragma unroll 1
     for (int q = tid; q < 2 * SW * (1 + 2 * HALO); q += TX * kWarps) {
         const int sp = q / (SW * (1 + 2 * HALO)), slot = q % (SW * (1 + 2 * HALO)), sx = slot % SW, sy = slot / SW;
         const double r = slot_density<double, false>(G, t, parity, sx, sy, sp);
-        sm.st.put<false>(sp, sy, sx, r, psi_of<double>(r));
+        outside |= sm.st.put(sp, sy, sx, r, psi_of<double>(r));
     }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) outside |= base_outside(p.f[i]);
+    const bool plain = __syncthreads_or(outside != 0);
+    if (plain) small_force_plain(sm, p, k, a);
+    else small_force<true>(sm, p, k, a);
     __syncthreads();
-    const Lat<double> &L = sm.st.L;
-    const double j = a == 0 ? A.add(A.sub(A.sub(A.add(A.sub(f[1], f[3]), f[5]), f[6]), f[7]), f[8])
-                            : A.sub(A.sub(A.add(A.add(A.sub(f[2], f[4]), f[5]), f[6]), f[7]), f[8]);
-    const double Fa = a == 0 ? force64<0, false, 1>(A, sm.st, k, cx, cy) : force64<1, false, 1>(A, sm.st, k, cx, cy);
-    sm.F[k][a][lane] = Fa;
-    sm.m[k][a][lane] = __fma_rn(0.5, Fa, j);   // Eq. (6)
-    __syncthreads();
-    if (k == 0) {   // component a of u^eq, Eq. (3)
-        const double om0 = L.omega[0], om1 = L.omega[1];
-        const double den = A.add(A.mul(om0, sm.st.v[0][sRho][cy][cx]), A.mul(om1, sm.st.v[1][sRho][cy][cx]));
-        sm.u[a][lane] = A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane])) / den;
+    outside = 0;
+    if (k == 0) {
+        const double u = plain ? small_velocity_plain(sm, a) : small_velocity<true>(sm, a);
+        sm.u[a][lane] = u;
+        outside = velocity_outside(u);
     }
-    __syncthreads();
+    const bool plain_push = __syncthreads_or(outside != 0) || plain;
     if (!valid) return;
-    const Dirs64<false> dirs(A, sm.u[0][lane], sm.u[1][lane]);
-    const double r = sm.st.v[k][sRho][cy][cx], om = L.omega[k], Fx = sm.F[k][0][lane], Fy = sm.F[k][1][lane];
-    const Push64 push(L, x, y);
-    double *__restrict__ nk = L.f[parity ^ 1] + (size_t)(k * 9) * plane + c;
-    auto dir = [&](auto Ic) {
-        constexpr int I = decltype(Ic)::value;
-        double g[2], po;
-        dirs.template terms<I>(A, g, po);
-        push.store<I>(nk, plane, relax64<I>(A, f[I], A.mul(w9(I), r), om, L.aw[k][cls9(I)], g, po, Fx, Fy));
-    };
-    if (a == 0) {   // the directions along e[0] and e[2], and rest
-        dir(std::integral_constant<int, 0>{});
-        dir(std::integral_constant<int, 1>{});
-        dir(std::integral_constant<int, 3>{});
-        dir(std::integral_constant<int, 5>{});
-        dir(std::integral_constant<int, 7>{});
-    } else {
-        dir(std::integral_constant<int, 2>{});
-        dir(std::integral_constant<int, 4>{});
-        dir(std::integral_constant<int, 6>{});
-        dir(std::integral_constant<int, 8>{});
-    }
+    double *nk = sm.st.L.f[parity ^ 1] + (size_t)(k * 9) * plane + c;
+    if (plain_push) small_push_plain(sm, p, nk, k, a, x, y);
+    else small_push<true>(sm, p, nk, k, a, x, y);
 }
 
 // ---- persistent launch over many time steps -----------------------------------

@@ -13,6 +13,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 C6 = dict(G_AB=3.0, G1=-7.4, G2=6.4)
+# a lattice stepped row by row (k_small64), and one stepped in tiles
+SIZES = [(70, 37), (230, 75)]
 
 
 @pytest.fixture(scope="module")
@@ -36,8 +38,8 @@ def populations(nx, ny, seed, kind="wide"):
 
 @pytest.mark.parametrize("mode,height", [(0, 2), (0, 4), (0, 8), (1, 8), (2, 2), (2, 4), (2, 8)])
 @pytest.mark.parametrize("kind,walls,wall_mode", [("wide", 0, 0), ("wide", 1, 0), ("ties", 1, 1), ("ties", 0, 0)])
-def test_integer_products_equal_the_fp64_pipe(lbmod, mode, height, kind, walls, wall_mode):
-    nx, ny = 70, 37
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_integer_products_equal_the_fp64_pipe(lbmod, mode, height, kind, walls, wall_mode, nx, ny):
     got = []
     for g in ((0.0, 0.0), (1e-70, 1e-70)):
         L = lbmod.Lattice(nx, ny, tau=(0.83, 2.7), g=g, walls=walls, wall_mode=wall_mode, wall_rho=(0.03, 1.0), **C6)
@@ -53,8 +55,8 @@ def test_integer_products_equal_the_fp64_pipe(lbmod, mode, height, kind, walls, 
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("scale", [1.0, 1e-40, 1e-62, 1e-306, 1e60, 1e140])
 @pytest.mark.parametrize("what", ["uniform", "one species", "random"])
-def test_values_at_and_beyond_the_covered_range(oracle_mod, lbmod, mode, scale, what):
-    nx, ny = 40, 21
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_values_at_and_beyond_the_covered_range(oracle_mod, lbmod, mode, scale, what, nx, ny):
     f = populations(nx, ny, 5)
     if what == "uniform":                     # forces and velocities exactly zero
         w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4).reshape(1, 9, 1, 1)
@@ -80,8 +82,8 @@ def test_values_at_and_beyond_the_covered_range(oracle_mod, lbmod, mode, scale, 
 
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("bad", [np.inf, np.nan, 1e300])
-def test_a_bad_node_spreads_as_in_the_oracle(oracle_mod, lbmod, mode, bad):
-    nx, ny = 70, 21
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_a_bad_node_spreads_as_in_the_oracle(oracle_mod, lbmod, mode, bad, nx, ny):
     f = populations(nx, ny, 7)
     f[0, 3, 9, 33] = bad
     kw = dict(tau=(1.0, 2.0), **C6)
