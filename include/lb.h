@@ -368,7 +368,7 @@ int lb_batch_set_wait_limit(lb_batch *b, double seconds, int32_t drop_tile);
  * order rest, (+-1,0,0), (0,+-1,0), (0,0,+-1), (1,1,0), (-1,-1,0), (1,-1,0),
  * (-1,1,0), (1,0,1), (-1,0,-1), (1,0,-1), (-1,0,1), (0,1,1), (0,-1,-1),
  * (0,1,-1), (0,-1,1).  One time step is two launches (density pass, fused
- * force / collision / push); LB_FP32 stores offsets from the node's previous
+ * force / collision / push), for LB_FP32 one; LB_FP32 stores offsets from the node's previous
  * density as the 2-D form does.  Same error conventions as above. */
 typedef struct lb3_params {
     int32_t nx, ny, nz;   /* each >= 5 */
@@ -412,7 +412,8 @@ int lb3_observables(lb3_handle *h, lb3_obs *o);
 int lb3_get_fields(lb3_handle *h, double *rho, double *ubar);
 /* Populations as FP64 host [2][19][nz][ny][nx] (LB_FP32: w_i R added back). */
 int lb3_get_populations(lb3_handle *h, double *f);
-/* As lb_profile: ms[0] density pass, ms[1] fused kernel, ms[2] whole step. */
+/* As lb_profile: ms[0] density pass (0 for LB_FP32, whose step is one launch),
+ * ms[1] fused kernel, ms[2] whole step. */
 int lb3_profile(lb3_handle *h, int32_t nsteps, void *flush_buf, size_t flush_bytes, double ms[3]);
 
 /* ---- device diagnostics ------------------------------------------------------ */

@@ -51,6 +51,9 @@ void fill3(lbk3::Lat3<real> &L, const lb3_params &p)
         L.omega[k] = (real)omega;
         for (int c = 0; c < 3; ++c) L.aw[k][c] = (real)((1.0 - 0.5 * omega) * wcls[c]);
     }
+    const double q[9] = {0.0, lbk3::q125(1), lbk3::q125(2), lbk3::q125(3), lbk3::q125(4), lbk3::q125(5), lbk3::q125(6), 0.0,
+                         lbk3::q125(8)};
+    for (int e = 1; e < 9; ++e) L.cw[e] = (real)(-((e == 1 ? p.G1 / 18.0 : e == 2 ? p.G1 / 36.0 : 0.0) + p.G2 * q[e]));
     L.G1 = (real)p.G1;
     L.G2 = (real)p.G2;
     L.GAB = (real)p.G_AB;
@@ -70,6 +73,7 @@ struct lb3_handle {
     double *partials = nullptr, *obs = nullptr, *tmp = nullptr;
     size_t tmp_elems = 0;
     int n_tiles = 0;
+    int sm_count = 0;
     int parity = 0;
     int64_t t = 0;
 
@@ -108,6 +112,11 @@ struct lb3_handle {
     {
         return f64() ? lbk3::Launch3<double>::collide(L64, par, stream) : lbk3::Launch3<float>::collide(L32, par, stream);
     }
+    cudaError_t step(int par)
+    {
+        return f64() ? lbk3::Launch3<double>::step(L64, par, sm_count, stream)
+                     : lbk3::Launch3<float>::step(L32, par, sm_count, stream);
+    }
     cudaError_t observe(double *part, double *rho, double *u)
     {
         return f64() ? lbk3::Launch3<double>::observe(L64, parity, part, rho, u, stream)
@@ -140,6 +149,10 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
     if (cudaGetDevice(&h->device) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail3(LB_ECUDA, "no CUDA device"));
+    }
+    if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) {
+        cudaGetLastError();
+        return bail(fail3(LB_ECUDA, "cudaDeviceGetAttribute failed"));
     }
     if (p->stream) {
         h->stream = (cudaStream_t)p->stream;
@@ -207,8 +220,7 @@ int lb3_step(lb3_handle *h, int64_t n)
     CHECK3(h);
     if (n < 0) return fail3(LB_EINVAL, "negative step count");
     for (int64_t s = 0; s < n; ++s) {
-        LB3_CUDA(h->density(h->parity));
-        LB3_CUDA(h->collide(h->parity));
+        LB3_CUDA(h->step(h->parity));
         h->parity ^= 1;
         h->t += 1;
     }
@@ -310,9 +322,10 @@ int lb3_profile(lb3_handle *h, int32_t nsteps, void *flush_buf, size_t flush_byt
     for (int s = 0; s < nsteps && ce == cudaSuccess; ++s) {
         if (flush_bytes) ce = cudaMemsetAsync(flush_buf, s & 0xff, flush_bytes, h->stream);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s], h->stream);
-        if (ce == cudaSuccess) ce = h->density(h->parity);
+        // FP32: the whole step is one kernel
+        if (ce == cudaSuccess && h->f64()) ce = h->density(h->parity);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], h->stream);
-        if (ce == cudaSuccess) ce = h->collide(h->parity);
+        if (ce == cudaSuccess) ce = h->f64() ? h->collide(h->parity) : h->step(h->parity);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 2], h->stream);
         if (ce == cudaSuccess) {
             h->parity ^= 1;

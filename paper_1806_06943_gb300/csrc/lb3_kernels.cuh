@@ -16,12 +16,14 @@
 // node's density at the previous step R, with the stencil and momentum sums
 // formed from differences of opposite neighbours.
 //
-// One time step is two launches over tiles of 32 x 4 x 2 nodes:
-//   k3_density : rho_k = sum_i f_k,i (FP32: R + sum_i h_i) into copy parity^1
+// One FP64 time step is two launches over tiles of 32 x 4 x 2 nodes:
+//   k3_density : rho_k = sum_i f_k,i (FP32: R + sum_i h_i, for the observables)
+//                into copy parity^1
 //   k3_collide : stages rho_k and psi_k of the tile plus a 2-node halo in
 //                shared memory, forms the forces, moments, u^eq, relaxes with
-//                the Guo term and pushes each population to x + e_i (FP32:
-//                re-referenced to rho(x + e_i), the destination's next R).
+//                the Guo term and pushes each population to x + e_i.
+// FP32 steps in one launch (k3_march), which also re-references each pushed
+// offset to rho(x + e_i), the destination's next R.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -29,7 +31,22 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <type_traits>
+
+#include "lb_vops.cuh"
+
 namespace lbk3 {
+
+using lbk::cfma;
+using lbk::cmul;
+using lbk::vadd;
+using lbk::vdiv;
+using lbk::vfma;
+using lbk::vmul;
+using lbk::vneg;
+using lbk::vsplat;
+using lbk::vsub;
+using lbk::vswap;
 
 constexpr int TX = 32, TY = 4, TZ = 2, HALO = 2;
 constexpr int SX = TX + 2 * HALO, SY = TY + 2 * HALO, SZ = TZ + 2 * HALO;
@@ -69,6 +86,7 @@ struct Lat3 {
     int32_t nx, ny, nz, pitch;
     int32_t tiles_x, tiles_y, tiles_z, has_probe;
     real omega[2], aw[2][3];   // 1 / tau_k; (1 - omega_k / 2) w(|e|^2) for |e|^2 = 0, 1, 2
+    real cw[9];          // -(G1 w + G2 q) for |e|^2 = 0 .. 8 (FP32: the two psi sums of Eq. 8 as one)
     real G1, G2, GAB;
     real g[3];
     double probe[4];     // cx, cy, cz, R
@@ -221,11 +239,11 @@ __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int p
 // 48 KB of static shared memory): the stage, then the observation partials.
 extern __shared__ __align__(16) unsigned char lb3_smem[];
 
-// FP32: three blocks per SM (80 registers; the spill of a few values costs
-// less than the latency a third block hides), FP64: as many as fit.
+// The FP64 step after its density pass.
 template <typename real>
-__global__ void __launch_bounds__(kThreads, kOffset3<real> ? 3 : 1) k3_collide(const Lat3<real> L, int parity)
+__global__ void __launch_bounds__(kThreads) k3_collide(const Lat3<real> L, int parity)
 {
+    static_assert(!kOffset3<real>, "FP32 steps in one pass (k3_march)");
     Stage3<real> &sm = *reinterpret_cast<Stage3<real> *>(lb3_smem);
     int x0, y0, z0;
     tile_origin(L.tiles_x, L.tiles_y, blockIdx.x, x0, y0, z0);
@@ -238,38 +256,18 @@ __global__ void __launch_bounds__(kThreads, kOffset3<real> ? 3 : 1) k3_collide(c
     const size_t c = ((size_t)z * L.ny + y) * L.pitch + x;
     const real *__restrict__ fc = L.f[parity];
     real *__restrict__ fn = L.f[parity ^ 1];
-    real F[2][3], rho[2], m[2][3], delta[2] = {(real)0, (real)0}, dg[2] = {(real)0, (real)0};
+    real F[2][3], rho[2], m[2][3];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         force3<real>(L, sm, k, cx, cy, cz, F[k]);
         rho[k] = sm.rho[k][cz][cy][cx];
-        real j[3] = {(real)0, (real)0, (real)0}, s = (real)0;
+        real j[3] = {(real)0, (real)0, (real)0};
 #pragma unroll
         for (int i = 0; i < 19; ++i) {
             const real fi = fc[(size_t)(k * 19 + i) * L.plane + c];
-            if constexpr (!kOffset3<real>) {
-                if (ex(i)) j[0] += ex(i) > 0 ? fi : -fi;
-                if (ey(i)) j[1] += ey(i) > 0 ? fi : -fi;
-                if (ez(i)) j[2] += ez(i) > 0 ? fi : -fi;
-            } else {
-                (void)s;
-            }
-        }
-        if constexpr (kOffset3<real>) {
-            // first moment from differences of opposite offsets; the offsets
-            // from the node's current density h - w (rho - R), their sum dg
-#pragma unroll
-            for (int i = 1; i < 19; i += 2) {
-                const real d = fc[(size_t)(k * 19 + i) * L.plane + c] - fc[(size_t)(k * 19 + i + 1) * L.plane + c];
-                if (ex(i)) j[0] += ex(i) > 0 ? d : -d;
-                if (ey(i)) j[1] += ey(i) > 0 ? d : -d;
-                if (ez(i)) j[2] += ez(i) > 0 ? d : -d;
-            }
-            delta[k] = rho[k] - L.rho[parity][(size_t)k * L.plane + c];
-            real sum = (real)0;
-#pragma unroll
-            for (int i = 0; i < 19; ++i) sum += fc[(size_t)(k * 19 + i) * L.plane + c] - (real)w19(i) * delta[k];
-            dg[k] = sum;
+            if (ex(i)) j[0] += ex(i) > 0 ? fi : -fi;
+            if (ey(i)) j[1] += ey(i) > 0 ? fi : -fi;
+            if (ez(i)) j[2] += ez(i) > 0 ? fi : -fi;
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a) m[k][a] = j[a] + (real)0.5 * F[k][a];   // Eq. (6), half force
@@ -284,36 +282,283 @@ __global__ void __launch_bounds__(kThreads, kOffset3<real> ? 3 : 1) k3_collide(c
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const real om = L.omega[k];
-        const real uF = u[0] * F[k][0] + u[1] * F[k][1] + u[2] * F[k][2];
 #pragma unroll
         for (int i = 0; i < 19; ++i) {
             const int EX = ex(i), EY = ey(i), EZ = ez(i), C = e2(i);
             const real w = (real)w19(i);
             const real eu = (real)EX * u[0] + (real)EY * u[1] + (real)EZ * u[2];
-            const real eF = (real)EX * F[k][0] + (real)EY * F[k][1] + (real)EZ * F[k][2];
             const real f = fc[(size_t)(k * 19 + i) * L.plane + c];
-            real v;
-            if constexpr (!kOffset3<real>) {
-                // Eqs. (1), (2), (5)
-                const real feq = w * rho[k] * ((real)1 + (real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu);
-                real Cg = (real)0;
-                const real e[3] = {(real)EX, (real)EY, (real)EZ};
+            // Eqs. (1), (2), (5)
+            const real feq = w * rho[k] * ((real)1 + (real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu);
+            real Cg = (real)0;
+            const real e[3] = {(real)EX, (real)EY, (real)EZ};
 #pragma unroll
-                for (int a = 0; a < 3; ++a) Cg += ((real)3 * (e[a] - u[a]) + (real)9 * eu * e[a]) * F[k][a];
-                Cg = L.aw[k][C] * Cg;
-                v = f - om * (f - feq) + Cg;
-            } else {
-                // offset form: Eq. (2) less w rho, Eq. (5) as 3 (1 - 1/2tau) w [(e.F)(1 + 3 e.u) - u.F]
-                const real h = f - w * delta[k];
-                const real geq = w * rho[k] * ((real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu) + w * dg[k];
-                const real Cg = (real)3 * L.aw[k][C] * (eF * ((real)1 + (real)3 * eu) - uF);
-                v = (h + om * (geq - h)) + Cg;
-                // re-referenced to the destination's density (its next R)
-                if (i != 0) v += w * (rho[k] - sm.rho[k][cz + EZ][cy + EY][cx + EX]);
-            }
+            for (int a = 0; a < 3; ++a) Cg += ((real)3 * (e[a] - u[a]) + (real)9 * eu * e[a]) * F[k][a];
+            Cg = L.aw[k][C] * Cg;
+            const real v = f - om * (f - feq) + Cg;
             const int xd = wrap1(x + EX, L.nx), yd = wrap1(y + EY, L.ny), zd = wrap1(z + EZ, L.nz);
             fn[(size_t)(k * 19 + i) * L.plane + ((size_t)zd * L.ny + yd) * L.pitch + xd] = v;
         }
+    }
+}
+
+// ---- the FP32 step in one pass ------------------------------------------------
+//
+// A block owns a column of 32 x 8 nodes in (x, y) and marches along z.  Per
+// plane it forms the densities and psi of the 36 x 12 slots two planes ahead
+// from their populations (into a ring of six planes in shared memory, both
+// species as a pair), then, one barrier later, the forces, the collision and
+// the pushes of its own plane, whose populations it reads a second time out
+// of L2.  A step is one launch; the density pass and collide kernel before it
+// moved 160 bytes a node more and formed the stencils once per species and as
+// two sums each, 3021 instructions a node against 1606 here.  160^3: 660 us a
+// step before, 421 now; 64^3: 50 and 37.  What bounds it is latency at 16 warps
+// per SM (39 % of the issue slots, 42 % of HBM): three blocks of 80 registers
+// spill (566 us); the populations by cp.async into shared memory a plane ahead
+// (436 us, 462 at three blocks), an L2 prefetch of the planes ahead (440 us) and
+// the density as a pass of its own before the same march (424 us) gained nothing.
+constexpr int RY = 8;                       // tile height in y
+constexpr int RW = TX + 2 * HALO, RH = RY + 2 * HALO;
+constexpr int kRing3 = 6;                   // planes z-2 .. z+2, and the one being written
+constexpr int kRingSlots = RW * RH - TX * RY;
+
+struct March3 {
+    float2 rho[kRing3][RH][RW];
+    float2 psi[kRing3][RH][RW];
+};
+
+// sum_j c_j s(x + e_j) e_j over the 5 x 5 x 5 neighbourhood from differences
+// D(dx, dy, dz) = s(x + e) - s(x - e), outer shells first; c[|e|^2].
+template <class Diff>
+__device__ __forceinline__ void psi_sums3(const Diff &D, const float (&c)[9], float2 &sx, float2 &sy, float2 &sz)
+{
+    float2 s[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    // in-plane pairs (a, b) of the axes (A, B): (e_A, e_B) and (e_A, -e_B)
+    auto plane = [&](auto Ac, auto Bc, int a, int b, float w) {
+        constexpr int A = decltype(Ac)::value, B = decltype(Bc)::value;
+        int e[3] = {0, 0, 0};
+        e[A] = a;
+        e[B] = b;
+        const float2 p = D(e[0], e[1], e[2]);
+        e[B] = -b;
+        const float2 m = D(e[0], e[1], e[2]);
+        s[A] = cfma(w * (float)a, vadd(p, m), s[A]);
+        s[B] = cfma(w * (float)b, vsub(p, m), s[B]);
+    };
+    auto corner = [&](int a, int b, int d, float w) {
+        const float2 d1 = D(a, b, d), d2 = D(a, b, -d), d3 = D(a, -b, d), d4 = D(a, -b, -d);
+        const float2 s12 = vadd(d1, d2), s34 = vadd(d3, d4), m12 = vsub(d1, d2), m34 = vsub(d3, d4);
+        s[0] = cfma(w * (float)a, vadd(s12, s34), s[0]);
+        s[1] = cfma(w * (float)b, vsub(s12, s34), s[1]);
+        s[2] = cfma(w * (float)d, vadd(m12, m34), s[2]);
+    };
+    using I0 = std::integral_constant<int, 0>;
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    auto planes = [&](int a, int b, float w) {
+        plane(I0{}, I1{}, a, b, w);
+        plane(I0{}, I2{}, a, b, w);
+        plane(I1{}, I2{}, a, b, w);
+    };
+    planes(2, 2, c[8]);
+    corner(2, 1, 1, c[6]);
+    corner(1, 2, 1, c[6]);
+    corner(1, 1, 2, c[6]);
+    planes(2, 1, c[5]);
+    planes(1, 2, c[5]);
+    s[0] = cfma(2.f * c[4], D(2, 0, 0), s[0]);
+    s[1] = cfma(2.f * c[4], D(0, 2, 0), s[1]);
+    s[2] = cfma(2.f * c[4], D(0, 0, 2), s[2]);
+    corner(1, 1, 1, c[3]);
+    planes(1, 1, c[2]);
+    sx = cfma(c[1], D(1, 0, 0), s[0]);
+    sy = cfma(c[1], D(0, 1, 0), s[1]);
+    sz = cfma(c[1], D(0, 0, 1), s[2]);
+}
+
+// sum_i w_i s(x + e_i) e_i over D3Q19 from the same differences.
+template <class Diff>
+__device__ __forceinline__ void rho_sums3(const Diff &D, float2 &sx, float2 &sy, float2 &sz)
+{
+    const float w1 = (float)(1.0 / 18.0), w2 = (float)(1.0 / 36.0);
+    const float2 xy = D(1, 1, 0), xm = D(1, -1, 0), xz = D(1, 0, 1), xn = D(1, 0, -1), yz = D(0, 1, 1), yn = D(0, 1, -1);
+    sx = cfma(w1, D(1, 0, 0), cmul(w2, vadd(vadd(xy, xm), vadd(xz, xn))));
+    sy = cfma(w1, D(0, 1, 0), cmul(w2, vadd(vsub(xy, xm), vadd(yz, yn))));
+    sz = cfma(w1, D(0, 0, 1), cmul(w2, vadd(vsub(xz, xn), vsub(yz, yn))));
+}
+
+// Densities (both species) of a node from its offset populations, in the
+// order of k3_density; f, R: the node in the first population plane and in
+// the reference densities.
+__device__ __forceinline__ float2 node_density3(const float *__restrict__ f, const float *__restrict__ R, size_t plane)
+{
+    float2 v[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) v[i] = make_float2(f[(size_t)i * plane], f[(size_t)(19 + i) * plane]);
+    const float2 r0 = make_float2(R[0], R[plane]);
+    float2 r = v[0];
+#pragma unroll
+    for (int i = 1; i < 19; ++i) r = vadd(r, v[i]);
+    return vadd(r0, r);
+}
+
+template <int kBlocks>
+__global__ void __launch_bounds__(TX *RY, kBlocks) k3_march(const Lat3<float> L, int parity, int tiles_y, int lz)
+{
+    March3 &sm = *reinterpret_cast<March3 *>(lb3_smem);
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    const int bx = blockIdx.x % L.tiles_x, by = (blockIdx.x / L.tiles_x) % tiles_y;
+    const int z0 = (blockIdx.x / (L.tiles_x * tiles_y)) * lz, z1 = min(z0 + lz, L.nz);
+    const int x0 = bx * TX, y0 = by * RY;
+    const size_t plane = L.plane, pxy = (size_t)L.ny * L.pitch;
+    const float *__restrict__ f = L.f[parity], *__restrict__ R = L.rho[parity];
+    // the thread's slots: its own node's, and one of the halo ring's
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    const bool valid = x < L.nx && y < L.ny, ring = tid < kRingSlots;
+    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
+    int rx = 0, ry = 0;
+    if (tid < 2 * RW) {
+        ry = tid / RW;
+        rx = tid % RW;
+    } else if (tid < 4 * RW) {
+        ry = RY + HALO + (tid - 2 * RW) / RW;
+        rx = (tid - 2 * RW) % RW;
+    } else if (ring) {
+        const int q = tid - 4 * RW;
+        ry = HALO + q / 4;
+        rx = (q % 4 < 2) ? q % 4 : TX + q % 4;
+    }
+    const size_t own = (size_t)wrap3(y, L.ny) * L.pitch + wrap3(x, L.nx);
+    const size_t rim = (size_t)wrap3(y0 + ry - HALO, L.ny) * L.pitch + wrap3(x0 + rx - HALO, L.nx);
+    // densities and psi of plane z (any integer) into ring plane q
+    auto stage = [&](int z, int q) {
+        const size_t zo = (size_t)wrap3(z, L.nz) * pxy;
+        if (ring) {
+            const float2 r = node_density3(f + zo + rim, R + zo + rim, plane);
+            sm.rho[q][ry][rx] = r;
+            sm.psi[q][ry][rx] = make_float2(psi3<float>(r.x), psi3<float>(r.y));
+        }
+        const float2 r = node_density3(f + zo + own, R + zo + own, plane);
+        sm.rho[q][cy][cx] = r;
+        sm.psi[q][cy][cx] = make_float2(psi3<float>(r.x), psi3<float>(r.y));
+        if (valid && z >= z0 && z < z1) {   // the next step's reference density
+            float *rn = L.rho[parity ^ 1] + zo + own;
+            rn[0] = r.x;
+            rn[plane] = r.y;
+        }
+    };
+#pragma unroll 1
+    for (int z = z0 - 2; z < z0 + 2; ++z) stage(z, z - z0 + 2);
+    int q = 4;   // ring plane of z + 2
+    // push offsets in x and y
+    const int oE = x + 1 < L.nx ? 1 : 1 - L.nx, oW = x > 0 ? -1 : L.nx - 1;
+    const long long oN = y + 1 < L.ny ? (long long)L.pitch : -(long long)L.pitch * (L.ny - 1);
+    const long long oS = y > 0 ? -(long long)L.pitch : (long long)L.pitch * (L.ny - 1);
+#pragma unroll 1
+    for (int z = z0; z < z1; ++z) {
+        stage(z + 2, q);
+        __syncthreads();
+        // ring planes of z - 2 .. z + 2
+        int rp[5];
+#pragma unroll
+        for (int d = 0; d < 5; ++d) rp[d] = q + d - 4 + (q + d - 4 < 0 ? kRing3 : 0);
+        q = q == kRing3 - 1 ? 0 : q + 1;
+        if (!valid) continue;
+        const size_t c = (size_t)z * pxy + own;
+        float2 h[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) h[i] = make_float2(f[(size_t)i * plane + c], f[(size_t)(19 + i) * plane + c]);
+        const float2 R2 = make_float2(R[c], R[plane + c]);
+        auto dpsi = [&](int dx, int dy, int dz) {
+            return vsub(sm.psi[rp[2 + dz]][cy + dy][cx + dx], sm.psi[rp[2 - dz]][cy - dy][cx - dx]);
+        };
+        auto drho = [&](int dx, int dy, int dz) {
+            return vsub(sm.rho[rp[2 + dz]][cy + dy][cx + dx], sm.rho[rp[2 - dz]][cy - dy][cx - dx]);
+        };
+        const float2 rho = sm.rho[rp[2]][cy][cx];
+        float2 F[3];
+        {
+            float2 m[3], s[3];
+            psi_sums3(dpsi, L.cw, m[0], m[1], m[2]);
+            rho_sums3(drho, s[0], s[1], s[2]);
+            const float2 psi = sm.psi[rp[2]][cy][cx], cr = cmul(-L.GAB, rho);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) F[a] = vfma(psi, m[a], vfma(cr, vswap(s[a]), cmul(L.g[a], rho)));
+        }
+        // first moment from differences of opposite offsets; then the offsets
+        // from the node's current density and their sum (as in 2-D)
+        float2 j[3];
+        {
+            float2 d[10];
+#pragma unroll
+            for (int p = 1; p < 10; ++p) d[p] = vsub(h[2 * p - 1], h[2 * p]);
+            // pairs: 1 x, 2 y, 3 z, 4 xy, 5 x-y, 6 xz, 7 x-z, 8 yz, 9 y-z
+            j[0] = vadd(d[1], vadd(vadd(d[4], d[5]), vadd(d[6], d[7])));
+            j[1] = vadd(d[2], vadd(vsub(d[4], d[5]), vadd(d[8], d[9])));
+            j[2] = vadd(d[3], vadd(vsub(d[6], d[7]), vsub(d[8], d[9])));
+        }
+        const float2 delta = vsub(rho, R2);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) h[i] = cfma(-(float)w19(i), delta, h[i]);
+        float2 dg = h[0];
+#pragma unroll
+        for (int p = 1; p < 10; ++p) dg = vadd(dg, vadd(h[2 * p - 1], h[2 * p]));
+        // u^eq of Eq. (3) from the half-force momenta (Eq. 6)
+        const float2 om = make_float2(L.omega[0], L.omega[1]);
+        const float den = vfma(om.y, rho.y, vmul(om.x, rho.x));
+        float u[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float2 m = cfma(0.5f, F[a], j[a]);
+            u[a] = vdiv(vfma(om.y, m.y, vmul(om.x, m.x)), den);
+        }
+        const float m15uu = cmul(-1.5f, vfma(u[2], u[2], vfma(u[1], u[1], vmul(u[0], u[0]))));
+        float2 nuF = vmul(vsplat(u[0], F[0]), F[0]);
+        nuF = vneg(vfma(vsplat(u[2], F[2]), F[2], vfma(vsplat(u[1], F[1]), F[1], nuF)));
+        const size_t zp = (size_t)(z + 1 < L.nz ? z + 1 : 0) * pxy + own, zm = (size_t)(z > 0 ? z - 1 : L.nz - 1) * pxy + own;
+        float *__restrict__ fn = L.f[parity ^ 1];
+        // post-collision value of direction i: Eq. (2) less w rho as geq,
+        // Eq. (5) as 3 (1 - omega/2) w [(e.F)(1 + 3 e.u) - u.F], re-referenced
+        // to the destination's density
+        auto push = [&](auto Ic, float qv, float2 X) {
+            constexpr int I = decltype(Ic)::value, EX = ex(I), EY = ey(I), EZ = ez(I), C = e2(I);
+            constexpr float w = (float)w19(I);
+            const float2 aw3 = make_float2(3.f * L.aw[0][C], 3.f * L.aw[1][C]);
+            const float2 geq = vfma(cmul(w, rho), vsplat(qv, rho), cmul(w, dg));
+            float2 v = vfma(aw3, X, vfma(om, vsub(geq, h[I]), h[I]));
+            if constexpr (I != 0) v = cfma(w, vsub(rho, sm.rho[rp[2 + EZ]][cy + EY][cx + EX]), v);
+            float *d = fn + ((EZ > 0 ? zp : EZ < 0 ? zm : c) + (long long)(EX > 0 ? oE : EX < 0 ? oW : 0) +
+                             (EY > 0 ? oN : EY < 0 ? oS : 0));
+            d[(size_t)I * plane] = v.x;
+            d[(size_t)(19 + I) * plane] = v.y;
+        };
+        push(std::integral_constant<int, 0>{}, m15uu, nuF);
+        auto pair = [&](auto Ic) {
+            constexpr int I = decltype(Ic)::value, E[3] = {ex(I), ey(I), ez(I)};
+            // e.u and e.F of direction I; its opposite has them negated
+            float eu = 0.f;
+            float2 eF = make_float2(0.f, 0.f);
+            bool first = true;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (E[a] == 0) continue;
+                eu = first ? u[a] : (E[a] > 0 ? vadd(eu, u[a]) : vsub(eu, u[a]));
+                eF = first ? F[a] : (E[a] > 0 ? vadd(eF, F[a]) : vsub(eF, F[a]));
+                first = false;
+            }
+            const float sq = vfma(cmul(4.5f, eu), eu, m15uu);
+            push(Ic, cfma(3.f, eu, sq), vfma(eF, vsplat(cfma(3.f, eu, 1.f), eF), nuF));
+            push(std::integral_constant<int, I + 1>{}, cfma(-3.f, eu, sq), vfma(eF, vsplat(cfma(3.f, eu, -1.f), eF), nuF));
+        };
+        pair(std::integral_constant<int, 1>{});
+        pair(std::integral_constant<int, 3>{});
+        pair(std::integral_constant<int, 5>{});
+        pair(std::integral_constant<int, 7>{});
+        pair(std::integral_constant<int, 9>{});
+        pair(std::integral_constant<int, 11>{});
+        pair(std::integral_constant<int, 13>{});
+        pair(std::integral_constant<int, 15>{});
+        pair(std::integral_constant<int, 17>{});
     }
 }
 

@@ -10,7 +10,8 @@ namespace lbk3 {
 
 template <typename real>
 struct Launch3 {
-    static cudaError_t step(const Lat3<real> &L, int parity, cudaStream_t s);      // density pass + collide
+    // one time step: FP32 in one pass (k3_march), FP64 density pass + collide
+    static cudaError_t step(const Lat3<real> &L, int parity, int sms, cudaStream_t s);
     static cudaError_t density(const Lat3<real> &L, int parity, cudaStream_t s);
     static cudaError_t collide(const Lat3<real> &L, int parity, cudaStream_t s);
     static cudaError_t observe(const Lat3<real> &L, int parity, double *partials, double *rho, double *u,

@@ -17,20 +17,59 @@ cudaError_t Launch3<real>::density(const Lat3<real> &L, int parity, cudaStream_t
 template <typename real>
 cudaError_t Launch3<real>::collide(const Lat3<real> &L, int parity, cudaStream_t s)
 {
-    const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
-    cudaError_t e = cudaFuncSetAttribute(k3_collide<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kCollideSmem3<real>);
-    if (e != cudaSuccess) return e;
-    k3_collide<real><<<n, dim3(TX, TY, TZ), kCollideSmem3<real>, s>>>(L, parity);
-    return cudaGetLastError();
+    if constexpr (kOffset3<real>) {
+        return cudaErrorInvalidValue;   // FP32 steps in one pass
+    } else {
+        const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
+        cudaError_t e = cudaFuncSetAttribute(k3_collide<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kCollideSmem3<real>);
+        if (e != cudaSuccess) return e;
+        k3_collide<real><<<n, dim3(TX, TY, TZ), kCollideSmem3<real>, s>>>(L, parity);
+        return cudaGetLastError();
+    }
+}
+
+// Resident blocks per SM of the marching kernels.
+constexpr int kMarchBlocks = 2;
+
+// Planes a block marches along z: the whole column, or segments of it where
+// columns alone do not fill the device evenly.  A segment forms the densities
+// of 4 more planes than it steps, `rim` of a plane's work each.
+inline int march_planes(int64_t columns, int nz, int slots, double rim)
+{
+    int best = nz;
+    double cost = 1e300;
+    for (int segs = 1; segs <= nz; ++segs) {
+        const int lz = (nz + segs - 1) / segs;
+        if ((nz + lz - 1) / lz != segs) continue;
+        const int64_t waves = (columns * segs + slots - 1) / slots;
+        const double c = (double)waves * (lz + 4.0 * rim);
+        if (c < cost * 0.999) {
+            cost = c;
+            best = lz;
+        }
+    }
+    return best;
 }
 
 template <typename real>
-cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, cudaStream_t s)
+cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, int sms, cudaStream_t s)
 {
-    cudaError_t e = density(L, parity, s);
-    if (e == cudaSuccess) e = collide(L, parity, s);
-    return e;
+    if constexpr (kOffset3<real>) {
+        const int tiles_y = (L.ny + RY - 1) / RY;
+        const int64_t columns = (int64_t)L.tiles_x * tiles_y;
+        const int lz = march_planes(columns, L.nz, kMarchBlocks * sms, 0.4);
+        cudaError_t e = cudaFuncSetAttribute(k3_march<kMarchBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(March3));
+        if (e != cudaSuccess) return e;
+        const unsigned n = (unsigned)(columns * ((L.nz + lz - 1) / lz));
+        k3_march<kMarchBlocks><<<n, dim3(TX, RY), sizeof(March3), s>>>(L, parity, tiles_y, lz);
+        return cudaGetLastError();
+    } else {
+        cudaError_t e = density(L, parity, s);
+        if (e == cudaSuccess) e = collide(L, parity, s);
+        return e;
+    }
 }
 
 template <typename real>
