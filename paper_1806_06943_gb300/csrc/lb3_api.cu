@@ -49,7 +49,7 @@ void fill3(lbk3::Lat3<real> &L, const lb3_params &p)
     for (int k = 0; k < 2; ++k) {
         const double omega = 1.0 / p.tau[k];
         L.omega[k] = (real)omega;
-        for (int c = 0; c < 3; ++c) L.aw[k][c] = (real)((1.0 - 0.5 * omega) * wcls[c]);
+        for (int c = 0; c < 3; ++c) L.aw3[k][c] = (real)(3.0 * ((1.0 - 0.5 * omega) * wcls[c]));
     }
     const double q[9] = {0.0, lbk3::q125(1), lbk3::q125(2), lbk3::q125(3), lbk3::q125(4), lbk3::q125(5), lbk3::q125(6), 0.0,
                          lbk3::q125(8)};

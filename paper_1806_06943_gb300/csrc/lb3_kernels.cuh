@@ -85,7 +85,8 @@ struct Lat3 {
     size_t plane;        // elements per [nz][ny][pitch] volume
     int32_t nx, ny, nz, pitch;
     int32_t tiles_x, tiles_y, tiles_z, has_probe;
-    real omega[2], aw[2][3];   // 1 / tau_k; (1 - omega_k / 2) w(|e|^2) for |e|^2 = 0, 1, 2
+    real omega[2];       // 1 / tau_k
+    real aw3[2][3];      // 3 (1 - omega_k / 2) w(|e|^2) for |e|^2 = 0, 1, 2
     real cw[9];          // -(G1 w + G2 q) for |e|^2 = 0 .. 8 (FP32: the two psi sums of Eq. 8 as one)
     real G1, G2, GAB;
     real g[3];
@@ -202,6 +203,95 @@ __device__ __forceinline__ void q125_sum(const real (*s)[SY][SX], int cx, int cy
     }
 }
 
+// ---- stencil sums from differences of opposite neighbours -----------------------
+
+// Arithmetic on both species at once (FP32) and on one value (FP64).
+struct Pair32 {
+    using V = float2;
+    using S = float;
+    __device__ __forceinline__ V zero() const { return make_float2(0.f, 0.f); }
+    __device__ __forceinline__ V add(V a, V b) const { return vadd(a, b); }
+    __device__ __forceinline__ V sub(V a, V b) const { return vsub(a, b); }
+    __device__ __forceinline__ V scale(S c, V a) const { return cmul(c, a); }
+    __device__ __forceinline__ V fma(S c, V a, V b) const { return cfma(c, a, b); }
+};
+// FP64: sums as fmas with the factor 1 in a register, the cheapest FP64
+// instruction of the chip (lb_f64.cuh).
+struct One64 {
+    using V = double;
+    using S = double;
+    double one;
+    __device__ __forceinline__ V zero() const { return 0.0; }
+    __device__ __forceinline__ V add(V a, V b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ V sub(V a, V b) const { return __fma_rn(-b, one, a); }
+    __device__ __forceinline__ V scale(S c, V a) const { return c * a; }
+    __device__ __forceinline__ V fma(S c, V a, V b) const { return __fma_rn(c, a, b); }
+};
+
+// sum_j c_j s(x + e_j) e_j over the 5 x 5 x 5 neighbourhood from differences
+// D(dx, dy, dz) = s(x + e) - s(x - e), outer shells first; c[|e|^2].
+template <class Ops, class Diff>
+__device__ __forceinline__ void psi_sums3(const Ops &o, const Diff &D, const typename Ops::S (&c)[9], typename Ops::V (&s)[3])
+{
+    using V = typename Ops::V;
+    using S = typename Ops::S;
+    s[0] = s[1] = s[2] = o.zero();
+    // in-plane pairs (a, b) of the axes (A, B): (e_A, e_B) and (e_A, -e_B)
+    auto plane = [&](auto Ac, auto Bc, int a, int b, S w) {
+        constexpr int A = decltype(Ac)::value, B = decltype(Bc)::value;
+        int e[3] = {0, 0, 0};
+        e[A] = a;
+        e[B] = b;
+        const V p = D(e[0], e[1], e[2]);
+        e[B] = -b;
+        const V m = D(e[0], e[1], e[2]);
+        s[A] = o.fma(w * (S)a, o.add(p, m), s[A]);
+        s[B] = o.fma(w * (S)b, o.sub(p, m), s[B]);
+    };
+    auto corner = [&](int a, int b, int d, S w) {
+        const V d1 = D(a, b, d), d2 = D(a, b, -d), d3 = D(a, -b, d), d4 = D(a, -b, -d);
+        const V s12 = o.add(d1, d2), s34 = o.add(d3, d4), m12 = o.sub(d1, d2), m34 = o.sub(d3, d4);
+        s[0] = o.fma(w * (S)a, o.add(s12, s34), s[0]);
+        s[1] = o.fma(w * (S)b, o.sub(s12, s34), s[1]);
+        s[2] = o.fma(w * (S)d, o.add(m12, m34), s[2]);
+    };
+    using I0 = std::integral_constant<int, 0>;
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    auto planes = [&](int a, int b, S w) {
+        plane(I0{}, I1{}, a, b, w);
+        plane(I0{}, I2{}, a, b, w);
+        plane(I1{}, I2{}, a, b, w);
+    };
+    planes(2, 2, c[8]);
+    corner(2, 1, 1, c[6]);
+    corner(1, 2, 1, c[6]);
+    corner(1, 1, 2, c[6]);
+    planes(2, 1, c[5]);
+    planes(1, 2, c[5]);
+    s[0] = o.fma((S)2 * c[4], D(2, 0, 0), s[0]);
+    s[1] = o.fma((S)2 * c[4], D(0, 2, 0), s[1]);
+    s[2] = o.fma((S)2 * c[4], D(0, 0, 2), s[2]);
+    corner(1, 1, 1, c[3]);
+    planes(1, 1, c[2]);
+    s[0] = o.fma(c[1], D(1, 0, 0), s[0]);
+    s[1] = o.fma(c[1], D(0, 1, 0), s[1]);
+    s[2] = o.fma(c[1], D(0, 0, 1), s[2]);
+}
+
+// sum_i w_i s(x + e_i) e_i over D3Q19 from the same differences.
+template <class Ops, class Diff>
+__device__ __forceinline__ void rho_sums3(const Ops &o, const Diff &D, typename Ops::V (&s)[3])
+{
+    using V = typename Ops::V;
+    using S = typename Ops::S;
+    const S w1 = (S)(1.0 / 18.0), w2 = (S)(1.0 / 36.0);
+    const V xy = D(1, 1, 0), xm = D(1, -1, 0), xz = D(1, 0, 1), xn = D(1, 0, -1), yz = D(0, 1, 1), yn = D(0, 1, -1);
+    s[0] = o.fma(w1, D(1, 0, 0), o.scale(w2, o.add(o.add(xy, xm), o.add(xz, xn))));
+    s[1] = o.fma(w1, D(0, 1, 0), o.scale(w2, o.add(o.sub(xy, xm), o.add(yz, yn))));
+    s[2] = o.fma(w1, D(0, 0, 1), o.scale(w2, o.add(o.sub(xz, xn), o.sub(yz, yn))));
+}
+
 // total force on species k at the staged node: Eq. (8) + Eq. (9) + rho_k g
 template <typename real>
 __device__ __forceinline__ void force3(const Lat3<real> &L, const Stage3<real> &sm, int k, int cx, int cy, int cz,
@@ -232,6 +322,9 @@ __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int p
         for (int i = 0; i < 19; ++i) r += f[(size_t)(k * 19 + i) * L.plane + c];
         if constexpr (kOffset3<real>) r = L.rho[parity][(size_t)k * L.plane + c] + r;
         L.rho[parity ^ 1][(size_t)k * L.plane + c] = r;
+        // FP64 keeps no reference densities: copy parity holds psi for the
+        // collide kernel, so that exp() runs once per node
+        if constexpr (!kOffset3<real>) L.rho[parity][(size_t)k * L.plane + c] = psi3<real>(r);
     }
 }
 
@@ -239,67 +332,140 @@ __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int p
 // 48 KB of static shared memory): the stage, then the observation partials.
 extern __shared__ __align__(16) unsigned char lb3_smem[];
 
-// The FP64 step after its density pass.
+// The FP64 step after its density pass.  It is bound by the FP64 pipe (one
+// warp instruction per 16 to 19 clocks and SM), so what counts is the number
+// of FP64 instructions: the two psi sums of Eq. (8) as one stencil of paired
+// differences, products fused into the sums that take them, the terms of the
+// directions shared by opposite ones and by the species, psi from the density
+// pass.  704 a node (2132 as direct sums in raster order with every product on
+// its own), the pipe 86 % busy; a 61 x 66 x 70 step 1.22 -> 0.44 ms, 32^3
+// 160 -> 64 us.
 template <typename real>
-__global__ void __launch_bounds__(kThreads) k3_collide(const Lat3<real> L, int parity)
+__global__ void __launch_bounds__(kThreads, 2) k3_collide(const Lat3<real> L, int parity)
 {
     static_assert(!kOffset3<real>, "FP32 steps in one pass (k3_march)");
     Stage3<real> &sm = *reinterpret_cast<Stage3<real> *>(lb3_smem);
     int x0, y0, z0;
     tile_origin(L.tiles_x, L.tiles_y, blockIdx.x, x0, y0, z0);
     const int tid = (threadIdx.z * TY + threadIdx.y) * TX + threadIdx.x;
-    stage3<real>(L, L.rho[parity ^ 1], x0, y0, z0, sm, tid);
+    {
+        const real *__restrict__ rho = L.rho[parity ^ 1], *__restrict__ psi = L.rho[parity];
+        const bool near = L.nx >= SX && L.ny >= SY && L.nz >= SZ;
+        for (int idx = tid; idx < SX * SY * SZ; idx += kThreads) {
+            const int sx = idx % SX, sy = (idx / SX) % SY, sz = idx / (SX * SY);
+            const int ax = x0 + sx - HALO, ay = y0 + sy - HALO, az = z0 + sz - HALO;
+            const int gx = near ? wrap1(ax, L.nx) : wrap3(ax, L.nx), gy = near ? wrap1(ay, L.ny) : wrap3(ay, L.ny);
+            const int gz = near ? wrap1(az, L.nz) : wrap3(az, L.nz);
+            const size_t c = ((size_t)gz * L.ny + gy) * L.pitch + gx;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                sm.rho[k][sz][sy][sx] = rho[(size_t)k * L.plane + c];
+                sm.psi[k][sz][sy][sx] = psi[(size_t)k * L.plane + c];
+            }
+        }
+    }
     __syncthreads();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
     if (x >= L.nx || y >= L.ny || z >= L.nz) return;
     const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO, cz = threadIdx.z + HALO;
     const size_t c = ((size_t)z * L.ny + y) * L.pitch + x;
-    const real *__restrict__ fc = L.f[parity];
-    real *__restrict__ fn = L.f[parity ^ 1];
-    real F[2][3], rho[2], m[2][3];
+    const real *__restrict__ fc = L.f[parity] + c;
+    One64 o;
+    asm volatile("mov.f64 %0, 0d3FF0000000000000;" : "=d"(o.one));
+    real F[2][3], m[2][3];
+    const real rho[2] = {sm.rho[0][cz][cy][cx], sm.rho[1][cz][cy][cx]};
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        force3<real>(L, sm, k, cx, cy, cz, F[k]);
-        rho[k] = sm.rho[k][cz][cy][cx];
-        real j[3] = {(real)0, (real)0, (real)0};
+        real p[3], s[3];
+        auto dpsi = [&](int dx, int dy, int dz) {
+            return o.sub(sm.psi[k][cz + dz][cy + dy][cx + dx], sm.psi[k][cz - dz][cy - dy][cx - dx]);
+        };
+        auto drho = [&](int dx, int dy, int dz) {
+            return o.sub(sm.rho[1 - k][cz + dz][cy + dy][cx + dx], sm.rho[1 - k][cz - dz][cy - dy][cx - dx]);
+        };
+        psi_sums3(o, dpsi, L.cw, p);
+        rho_sums3(o, drho, s);
+        const real psi = sm.psi[k][cz][cy][cx], cr = -L.GAB * rho[k];
 #pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const real fi = fc[(size_t)(k * 19 + i) * L.plane + c];
-            if (ex(i)) j[0] += ex(i) > 0 ? fi : -fi;
-            if (ey(i)) j[1] += ey(i) > 0 ? fi : -fi;
-            if (ez(i)) j[2] += ez(i) > 0 ? fi : -fi;
+        for (int a = 0; a < 3; ++a) F[k][a] = __fma_rn(psi, p[a], __fma_rn(cr, s[a], rho[k] * L.g[a]));
+        // half-force momenta (Eq. 6) from differences of opposite populations
+        real j[3];
+#pragma unroll
+        for (int q = 1; q < 10; ++q) {
+            const real d = o.sub(fc[(size_t)(k * 19 + 2 * q - 1) * L.plane], fc[(size_t)(k * 19 + 2 * q) * L.plane]);
+            const int e[3] = {ex(2 * q - 1), ey(2 * q - 1), ez(2 * q - 1)};
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if (e[a] != 0) j[a] = q == a + 1 ? d : (e[a] > 0 ? o.add(j[a], d) : o.sub(j[a], d));
         }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) m[k][a] = j[a] + (real)0.5 * F[k][a];   // Eq. (6), half force
+        for (int a = 0; a < 3; ++a) m[k][a] = __fma_rn((real)0.5, F[k][a], j[a]);
     }
     // Eq. (3)
     const real om0 = L.omega[0], om1 = L.omega[1];
-    const real den = om0 * rho[0] + om1 * rho[1];
+    const real den = __fma_rn(om0, rho[0], om1 * rho[1]);
     real u[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] = (om0 * m[0][a] + om1 * m[1][a]) / den;
-    const real uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    for (int a = 0; a < 3; ++a) u[a] = __fma_rn(om0, m[0][a], om1 * m[1][a]) / den;
+    const real m15uu = (real)-1.5 * __fma_rn(u[0], u[0], __fma_rn(u[1], u[1], u[2] * u[2]));
+    const int oE = x + 1 < L.nx ? 1 : 1 - L.nx, oW = x > 0 ? -1 : L.nx - 1;
+    const long long oN = y + 1 < L.ny ? (long long)L.pitch : -(long long)L.pitch * (L.ny - 1);
+    const long long oS = y > 0 ? -(long long)L.pitch : (long long)L.pitch * (L.ny - 1);
+    const long long pxy = (long long)L.ny * L.pitch;
+    const long long oU = z + 1 < L.nz ? pxy : -pxy * (L.nz - 1), oD = z > 0 ? -pxy : pxy * (L.nz - 1);
+    real *__restrict__ fn = L.f[parity ^ 1] + c;
+    real wr[2][3], uF[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const real om = L.omega[k];
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const int EX = ex(i), EY = ey(i), EZ = ez(i), C = e2(i);
-            const real w = (real)w19(i);
-            const real eu = (real)EX * u[0] + (real)EY * u[1] + (real)EZ * u[2];
-            const real f = fc[(size_t)(k * 19 + i) * L.plane + c];
-            // Eqs. (1), (2), (5)
-            const real feq = w * rho[k] * ((real)1 + (real)3 * eu + (real)4.5 * eu * eu - (real)1.5 * uu);
-            real Cg = (real)0;
-            const real e[3] = {(real)EX, (real)EY, (real)EZ};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) Cg += ((real)3 * (e[a] - u[a]) + (real)9 * eu * e[a]) * F[k][a];
-            Cg = L.aw[k][C] * Cg;
-            const real v = f - om * (f - feq) + Cg;
-            const int xd = wrap1(x + EX, L.nx), yd = wrap1(y + EY, L.ny), zd = wrap1(z + EZ, L.nz);
-            fn[(size_t)(k * 19 + i) * L.plane + ((size_t)zd * L.ny + yd) * L.pitch + xd] = v;
-        }
+        uF[k] = __fma_rn(u[0], F[k][0], __fma_rn(u[1], F[k][1], u[2] * F[k][2]));
+        wr[k][0] = (real)w19(0) * rho[k];
+        wr[k][1] = (real)w19(1) * rho[k];
+        wr[k][2] = (real)w19(7) * rho[k];
     }
+    // direction I of both species: f + omega (w rho q - f) + 3 (1 - omega/2) w X,
+    // q the polynomial of Eq. (2) and X = (e.F)(1 + 3 e.u) - u.F (Eqs. 1, 2, 5)
+    auto push = [&](auto Ic, real q, real XA, real XB) {
+        constexpr int I = decltype(Ic)::value, C = e2(I);
+        const long long off = (long long)(ex(I) > 0 ? oE : ex(I) < 0 ? oW : 0) + (ey(I) > 0 ? oN : ey(I) < 0 ? oS : 0) +
+                              (ez(I) > 0 ? oU : ez(I) < 0 ? oD : 0);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const size_t pl = (size_t)(k * 19 + I) * L.plane;
+            const real f = fc[pl];
+            const real v = __fma_rn(k ? om1 : om0, __fma_rn(wr[k][C], q, -f), f);
+            fn[(long long)pl + off] = __fma_rn(L.aw3[k][C], k ? XB : XA, v);
+        }
+    };
+    const real c0 = o.add((real)1, m15uu);
+    push(std::integral_constant<int, 0>{}, c0, -uF[0], -uF[1]);
+    auto pair = [&](auto Ic) {
+        constexpr int I = decltype(Ic)::value, E[3] = {ex(I), ey(I), ez(I)};
+        real eu = (real)0, eF[2] = {(real)0, (real)0};
+        bool first = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (E[a] == 0) continue;
+            eu = first ? u[a] : (E[a] > 0 ? o.add(eu, u[a]) : o.sub(eu, u[a]));
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                eF[k] = first ? F[k][a] : (E[a] > 0 ? o.add(eF[k], F[k][a]) : o.sub(eF[k], F[k][a]));
+            first = false;
+        }
+        const real sq = __fma_rn((real)4.5 * eu, eu, c0);
+        const real tp = __fma_rn((real)3, eu, (real)1), tm = __fma_rn((real)3, eu, (real)-1);
+        push(Ic, __fma_rn((real)3, eu, sq), __fma_rn(eF[0], tp, -uF[0]), __fma_rn(eF[1], tp, -uF[1]));
+        push(std::integral_constant<int, I + 1>{}, __fma_rn((real)-3, eu, sq), __fma_rn(eF[0], tm, -uF[0]),
+             __fma_rn(eF[1], tm, -uF[1]));
+    };
+    pair(std::integral_constant<int, 1>{});
+    pair(std::integral_constant<int, 3>{});
+    pair(std::integral_constant<int, 5>{});
+    pair(std::integral_constant<int, 7>{});
+    pair(std::integral_constant<int, 9>{});
+    pair(std::integral_constant<int, 11>{});
+    pair(std::integral_constant<int, 13>{});
+    pair(std::integral_constant<int, 15>{});
+    pair(std::integral_constant<int, 17>{});
 }
 
 // ---- the FP32 step in one pass ------------------------------------------------
@@ -326,66 +492,6 @@ struct March3 {
     float2 rho[kRing3][RH][RW];
     float2 psi[kRing3][RH][RW];
 };
-
-// sum_j c_j s(x + e_j) e_j over the 5 x 5 x 5 neighbourhood from differences
-// D(dx, dy, dz) = s(x + e) - s(x - e), outer shells first; c[|e|^2].
-template <class Diff>
-__device__ __forceinline__ void psi_sums3(const Diff &D, const float (&c)[9], float2 &sx, float2 &sy, float2 &sz)
-{
-    float2 s[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    // in-plane pairs (a, b) of the axes (A, B): (e_A, e_B) and (e_A, -e_B)
-    auto plane = [&](auto Ac, auto Bc, int a, int b, float w) {
-        constexpr int A = decltype(Ac)::value, B = decltype(Bc)::value;
-        int e[3] = {0, 0, 0};
-        e[A] = a;
-        e[B] = b;
-        const float2 p = D(e[0], e[1], e[2]);
-        e[B] = -b;
-        const float2 m = D(e[0], e[1], e[2]);
-        s[A] = cfma(w * (float)a, vadd(p, m), s[A]);
-        s[B] = cfma(w * (float)b, vsub(p, m), s[B]);
-    };
-    auto corner = [&](int a, int b, int d, float w) {
-        const float2 d1 = D(a, b, d), d2 = D(a, b, -d), d3 = D(a, -b, d), d4 = D(a, -b, -d);
-        const float2 s12 = vadd(d1, d2), s34 = vadd(d3, d4), m12 = vsub(d1, d2), m34 = vsub(d3, d4);
-        s[0] = cfma(w * (float)a, vadd(s12, s34), s[0]);
-        s[1] = cfma(w * (float)b, vsub(s12, s34), s[1]);
-        s[2] = cfma(w * (float)d, vadd(m12, m34), s[2]);
-    };
-    using I0 = std::integral_constant<int, 0>;
-    using I1 = std::integral_constant<int, 1>;
-    using I2 = std::integral_constant<int, 2>;
-    auto planes = [&](int a, int b, float w) {
-        plane(I0{}, I1{}, a, b, w);
-        plane(I0{}, I2{}, a, b, w);
-        plane(I1{}, I2{}, a, b, w);
-    };
-    planes(2, 2, c[8]);
-    corner(2, 1, 1, c[6]);
-    corner(1, 2, 1, c[6]);
-    corner(1, 1, 2, c[6]);
-    planes(2, 1, c[5]);
-    planes(1, 2, c[5]);
-    s[0] = cfma(2.f * c[4], D(2, 0, 0), s[0]);
-    s[1] = cfma(2.f * c[4], D(0, 2, 0), s[1]);
-    s[2] = cfma(2.f * c[4], D(0, 0, 2), s[2]);
-    corner(1, 1, 1, c[3]);
-    planes(1, 1, c[2]);
-    sx = cfma(c[1], D(1, 0, 0), s[0]);
-    sy = cfma(c[1], D(0, 1, 0), s[1]);
-    sz = cfma(c[1], D(0, 0, 1), s[2]);
-}
-
-// sum_i w_i s(x + e_i) e_i over D3Q19 from the same differences.
-template <class Diff>
-__device__ __forceinline__ void rho_sums3(const Diff &D, float2 &sx, float2 &sy, float2 &sz)
-{
-    const float w1 = (float)(1.0 / 18.0), w2 = (float)(1.0 / 36.0);
-    const float2 xy = D(1, 1, 0), xm = D(1, -1, 0), xz = D(1, 0, 1), xn = D(1, 0, -1), yz = D(0, 1, 1), yn = D(0, 1, -1);
-    sx = cfma(w1, D(1, 0, 0), cmul(w2, vadd(vadd(xy, xm), vadd(xz, xn))));
-    sy = cfma(w1, D(0, 1, 0), cmul(w2, vadd(vsub(xy, xm), vadd(yz, yn))));
-    sz = cfma(w1, D(0, 0, 1), cmul(w2, vadd(vsub(xz, xn), vsub(yz, yn))));
-}
 
 // Densities (both species) of a node from its offset populations, in the
 // order of k3_density; f, R: the node in the first population plane and in
@@ -479,8 +585,8 @@ __global__ void __launch_bounds__(TX *RY, kBlocks) k3_march(const Lat3<float> L,
         float2 F[3];
         {
             float2 m[3], s[3];
-            psi_sums3(dpsi, L.cw, m[0], m[1], m[2]);
-            rho_sums3(drho, s[0], s[1], s[2]);
+            psi_sums3(Pair32{}, dpsi, L.cw, m);
+            rho_sums3(Pair32{}, drho, s);
             const float2 psi = sm.psi[rp[2]][cy][cx], cr = cmul(-L.GAB, rho);
 #pragma unroll
             for (int a = 0; a < 3; ++a) F[a] = vfma(psi, m[a], vfma(cr, vswap(s[a]), cmul(L.g[a], rho)));
@@ -523,7 +629,7 @@ __global__ void __launch_bounds__(TX *RY, kBlocks) k3_march(const Lat3<float> L,
         auto push = [&](auto Ic, float qv, float2 X) {
             constexpr int I = decltype(Ic)::value, EX = ex(I), EY = ey(I), EZ = ez(I), C = e2(I);
             constexpr float w = (float)w19(I);
-            const float2 aw3 = make_float2(3.f * L.aw[0][C], 3.f * L.aw[1][C]);
+            const float2 aw3 = make_float2(L.aw3[0][C], L.aw3[1][C]);
             const float2 geq = vfma(cmul(w, rho), vsplat(qv, rho), cmul(w, dg));
             float2 v = vfma(aw3, X, vfma(om, vsub(geq, h[I]), h[I]));
             if constexpr (I != 0) v = cfma(w, vsub(rho, sm.rho[rp[2 + EZ]][cy + EY][cx + EX]), v);

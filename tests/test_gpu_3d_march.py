@@ -1,7 +1,9 @@
 """The FP32 3-D step (one launch, blocks marching along z) at the sizes where
 its tiles, rings and wraps have edges, against the FP64 3-D step: 20 steps
 from the same fields, within the 1e-5 (normwise) that the FP32 form is held to
-after 300 steps."""
+after 300 steps.  That bound comes from the interface's momentum balance and
+the 0.0095 spurious currents around a drop; a box too small for an interface
+(5^3) moves at 3e-4, so velocities are measured against at least 0.0095."""
 import numpy as np
 import pytest
 
@@ -32,6 +34,6 @@ def test_march_matches_fp64(lbmod, nx, ny, nz):
         got.append((L.fields(), L.get_populations()))
         L.close()
     (f32, p32), (f64, p64) = got
-    for key in ("rho", "ubar"):
-        assert np.max(np.abs(f32[key] - f64[key])) <= 1e-5 * np.max(np.abs(f64[key])), key
+    for key, floor in (("rho", 0.0), ("ubar", 0.0095)):
+        assert np.max(np.abs(f32[key] - f64[key])) <= 1e-5 * max(np.max(np.abs(f64[key])), floor), key
     assert np.max(np.abs(p32 - p64)) <= 1e-5 * np.max(np.abs(p64))
