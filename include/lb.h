@@ -299,7 +299,7 @@ int lb_profile(lb_handle *h, int32_t nsteps, void *flush_buf, size_t flush_bytes
  * the adjoint populations and the gradients stay FP64.  LB_OBJ_DP needs a
  * probe.  Device memory, allocated for the call: nsteps/ckpt_every + 1
  * states of the lattice's precision, ckpt_every + 2 (FP32: + 3) FP64
- * population copies, plus 22 FP64 planes.  Synchronises. */
+ * population copies, plus 25 FP64 planes.  Synchronises. */
 int lb_grad(lb_handle *h, int64_t nsteps, int32_t ckpt_every, int32_t objective, double *J, double dJ[5]);
 
 /* One step of the discrete adjoint at the current state (the transpose of
@@ -309,7 +309,7 @@ int lb_grad(lb_handle *h, int64_t nsteps, int32_t ckpt_every, int32_t objective,
  * for theta = (G_AB, G1, G2, tau_A, tau_B), Step the map from the
  * populations at time t to those at t + 1.  Either output may be NULL.
  * LB_FP64 lattices with Guo forcing only (else LB_EINVAL).  The state is
- * not changed.  Device memory: two FP64 population copies and 22 FP64
+ * not changed.  Device memory: two FP64 population copies and 25 FP64
  * planes, allocated for the call.  Synchronises. */
 int lb_step_vjp(lb_handle *h, const double *w, double *out, double dtheta[5]);
 

@@ -33,7 +33,7 @@ UNITS = {
     "lb_fp32.cu": [],
     "lb_tma.cu": [],
     "lb_noalloc.cu": ["-fmad=false"],
-    "lb_adjoint.cu": ["-fmad=false"],
+    "lb_adjoint.cu": [],
     "lb_device.cu": [],
     "lb3_api.cu": [],
     "lb3_fp64.cu": ["-fmad=false"],

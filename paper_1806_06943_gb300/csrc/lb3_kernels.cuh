@@ -33,6 +33,7 @@
 
 #include <type_traits>
 
+#include "lb_f64.cuh"
 #include "lb_vops.cuh"
 
 namespace lbk3 {
@@ -370,8 +371,7 @@ __global__ void __launch_bounds__(kThreads, 2) k3_collide(const Lat3<real> L, in
     const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO, cz = threadIdx.z + HALO;
     const size_t c = ((size_t)z * L.ny + y) * L.pitch + x;
     const real *__restrict__ fc = L.f[parity] + c;
-    One64 o;
-    asm volatile("mov.f64 %0, 0d3FF0000000000000;" : "=d"(o.one));
+    const One64 o{lbk::opaque_one()};
     real F[2][3], m[2][3];
     const real rho[2] = {sm.rho[0][cz][cy][cx], sm.rho[1][cz][cy][cx]};
 #pragma unroll

@@ -16,7 +16,7 @@
 //   phase A (local at x): the adjoints of u, F_k, m_k, the local parts of
 //     the adjoints of rho_k and psi_k, the stencil sources
 //     S1bar = -G1 psi F_bar, S2bar = -G2 psi F_bar, S3bar = -G_AB rho F_bar,
-//     and the parameter-gradient contributions (block partials, FP64)
+//     and the parameter-gradient contributions (per-node sums, FP64)
 //   phase B (gather at y): psi_bar(y) += sum over the nodes x whose stencils
 //     read y of w e . S1bar(x) + p e . S2bar(x); rho_bar(y) += exp(-rho) psi_bar
 //     + w e . S3bar_kbar(x); lam_k,i(y, t) = (1 - om_k) lam*_k,i + m_bar_k . e_i + rho_bar_k.
@@ -35,13 +35,14 @@ namespace {
 enum AdjSlot {
     aPsiA = 0, aPsiB, aRhoA, aRhoB,             // local psi_bar, rho_bar
     aMAx, aMAy, aMBx, aMBy,                      // m_bar
-    aS1Ax, aS1Ay, aS1Bx, aS1By,                  // S1bar
-    aS2Ax, aS2Ay, aS2Bx, aS2By,                  // S2bar
-    aS3Ax, aS3Ay, aS3Bx, aS3By,                  // S3bar
+    aTAx, aTAy, aTBx, aTBy,                      // psi F_bar: S1bar = -G1 T, S2bar = -G2 T
+    aQAx, aQAy, aQBx, aQBy,                      // rho F_bar: S3bar = -G_AB Q
     kAdjSlots
 };
-// parameter-gradient accumulators per tile
+static_assert(kAdjSlots == kAdjSlotCount, "the host sizes the buffer");
+// parameter-gradient accumulators, a plane each
 enum AdjGrad { gGAB = 0, gG1, gG2, gOmA, gOmB, kAdjGrads };
+static_assert(kAdjGrads == kAdjGradPlanes, "the host sizes the buffer");
 
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
@@ -65,239 +66,328 @@ __device__ __forceinline__ double pull_lam(const Lat<double> &L, const double *_
 
 }  // namespace
 
+// D2Q9 and D2Q25 sums sum_j w_j s(x + e_j) e_j of a staged plane from
+// differences of opposite neighbours (the inner ones serve both).
+__device__ __forceinline__ void adj_sums(const Arith64<false> &A, const double (*s)[SW], int cx, int cy, double (&s9)[2],
+                                         double (*s25)[2])
+{
+    constexpr double W1 = 1.0 / 9.0, W2 = 1.0 / 36.0;
+    auto D = [&](int dx, int dy) { return A.sub(s[cy + dy][cx + dx], s[cy - dy][cx - dx]); };
+    const double dE = D(1, 0), dN = D(0, 1), d1 = D(1, 1), d2 = D(1, -1);
+    const double p = A.add(d1, d2), q = A.sub(d1, d2);
+    s9[0] = __fma_rn(W1, dE, W2 * p);
+    s9[1] = __fma_rn(W1, dN, W2 * q);
+    if (!s25) return;
+    double x = (2.0 * p25(4)) * D(2, 0), y = (2.0 * p25(4)) * D(0, 2);
+#pragma unroll
+    for (int a = 1; a <= 2; ++a)
+#pragma unroll
+        for (int b = 1; b <= 2; ++b) {
+            if (a == 1 && b == 1) continue;
+            const double e1 = D(a, b), e2 = D(a, -b);
+            x = __fma_rn(p25(a * a + b * b) * a, A.add(e1, e2), x);
+            y = __fma_rn(p25(a * a + b * b) * b, A.sub(e1, e2), y);
+        }
+    (*s25)[0] = __fma_rn(p25(1), dE, __fma_rn(p25(2), p, x));
+    (*s25)[1] = __fma_rn(p25(1), dN, __fma_rn(p25(2), q, y));
+}
+
 // Phase A.  seed_kind: 0 = adjoint of a time step (lam_next given); 1 = seed
 // of mu_r at this state (d J / d Q in seed_a, per-node m_bar from ubar); 2 =
 // seed of the Laplace pressure jump (c_in = seed_a for r < R/2, c_out = seed_b
-// for r > R + 6, probe in L.probe).
-__global__ void __launch_bounds__(kThreads) k_adj_local(const Lat<double> L, const double *__restrict__ f,
-                                                        const double *__restrict__ rho, const double *__restrict__ lam_next,
-                                                        double *__restrict__ abuf, double *__restrict__ gpart, int seed_kind,
-                                                        double seed_a, double seed_b)
+// for r > R + 6, probe in L).  rho: the densities and exp(-rho) of k_adj_density.
+//
+// Everything the collision's adjoint needs of lam* are its moments of second
+// order with the weights w_i: with M0, M1, M2 the sums of w_i lam*_i (1, e,
+// e e), V = 3 M1 - 3 u M0 + 9 M2 u and a = 1 - omega/2,
+//   u_bar = omega rho V + a (9 M2 F - 3 F M0),   F_bar = a V,
+//   rho_bar = omega P,  P = M0 + 3 M1.u + 4.5 u.M2 u - 1.5 u.u M0,
+//   omega_bar = rho P - sum_i lam*_i f_i - V.F / 2,
+// which takes a third of the FP64 instructions (they bound the kernel) of the
+// sums written per direction: 397 a node instead of 1414, 214 -> 64 us on a
+// 512 x 128 lattice; k_adj_gather, with one combined stencil, 158 instead of
+// 559, 90 -> 31 us.
+__global__ void __launch_bounds__(kThreads, 4) k_adj_local(const Lat<double> L, const double *__restrict__ f,
+                                                           const double *__restrict__ rho, const double *__restrict__ lam_next,
+                                                           double *__restrict__ abuf, double *__restrict__ gpart, int seed_kind,
+                                                           double seed_a, double seed_b)
 {
     __shared__ double srho[2][SH][SW];
     __shared__ double spsi[2][SH][SW];
-    __shared__ double sred[kThreads / 32][8];
     const int tiles_x = (L.nx + TX - 1) / TX;
     const int x0 = (blockIdx.x % tiles_x) * TX, y0 = (blockIdx.x / tiles_x) * TY;
     const int tid = threadIdx.y * TX + threadIdx.x;
-    stage_tile<double, SH>(L, rho, x0, y0, srho, spsi, tid, kThreads);
+    const Arith64<false> A(opaque_one());
+    for (int idx = tid; idx < SW * SH; idx += kThreads) {
+        const int sx = idx % SW, sy = idx / SW;
+        const int gx = wrap_index(x0 + sx - HALO, L.nx);
+        int gy = y0 + sy - HALO;
+        bool fixed = false;
+        if (gy < 0 || gy >= L.ny) {
+            if (!L.walls) {
+                gy = wrap_index(gy, L.ny);
+            } else if (L.wall_mode == 1) {
+                fixed = true;
+            } else {
+                gy = gy < 0 ? -1 - gy : 2 * L.ny - 1 - gy;
+                gy = gy < 0 ? 0 : (gy >= L.ny ? L.ny - 1 : gy);  // rows no valid node reads
+            }
+        }
+        const size_t c = (size_t)gy * L.pitch + gx;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            srho[k][sy][sx] = fixed ? L.wall_rho[k] : rho[(size_t)k * L.plane + c];
+            spsi[k][sy][sx] = fixed ? psi_of<double>(L.wall_rho[k]) : A.sub(1.0, rho[(size_t)(2 + k) * L.plane + c]);
+        }
+    }
     __syncthreads();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    if (x >= L.nx || y >= L.ny) return;
+    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
+    const size_t c = (size_t)y * L.pitch + x;
+    double S1[2][2], S2[2][2], S3[2][2], F[2][2], m[2][2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        double fk[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fk[i] = f[(size_t)(k * 9 + i) * L.plane + c];
+        adj_sums(A, spsi[k], cx, cy, S1[k], &S2[k]);
+        adj_sums(A, srho[1 - k], cx, cy, S3[k], nullptr);
+        const double r = srho[k][cy][cx], ps = spsi[k][cy][cx];
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+            F[k][a] = __fma_rn(-ps, __fma_rn(L.G1, S1[k][a], L.G2 * S2[k][a]), r * __fma_rn(-L.GAB, S3[k][a], L.g[a]));
+        const double d57 = A.sub(fk[5], fk[7]), d86 = A.sub(fk[8], fk[6]);
+        m[k][0] = __fma_rn(0.5, F[k][0], A.add(A.sub(fk[1], fk[3]), A.add(d57, d86)));
+        m[k][1] = __fma_rn(0.5, F[k][1], A.add(A.sub(fk[2], fk[4]), A.sub(d57, d86)));
+    }
+    const double r[2] = {srho[0][cy][cx], srho[1][cy][cx]};
+    const double om[2] = {L.omega[0], L.omega[1]};
+    double aV[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, rb[2] = {0.0, 0.0}, mb[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, omb[2] = {0.0, 0.0};
     double gr[kAdjGrads] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (x < L.nx && y < L.ny) {
-        const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
-        const size_t c = (size_t)y * L.pitch + x;
-        double r[2], ps[2], S1[2][2], S2[2][2], S3[2][2], F[2][2], m[2][2], fk[2][9];
+    if (seed_kind == 0) {
+        const double rD = 1.0 / __fma_rn(om[0], r[0], om[1] * r[1]);
+        const double u[2] = {__fma_rn(om[0], m[0][0], om[1] * m[1][0]) * rD, __fma_rn(om[0], m[0][1], om[1] * m[1][1]) * rD};
+        const double uu15 = 1.5 * __fma_rn(u[0], u[0], u[1] * u[1]);
+        double ub[2] = {0.0, 0.0};
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
-            for (int i = 0; i < 9; ++i) fk[k][i] = f[(size_t)(k * 9 + i) * L.plane + c];
-            q9_sum<double>(spsi[k], cx, cy, S1[k][0], S1[k][1]);
-            q25_sum<double>(spsi[k], cx, cy, S2[k][0], S2[k][1]);
-            q9_sum<double>(srho[1 - k], cx, cy, S3[k][0], S3[k][1]);
-            r[k] = srho[k][cy][cx];
-            ps[k] = spsi[k][cy][cx];
-            for (int a = 0; a < 2; ++a)
-                F[k][a] = -L.G1 * ps[k] * S1[k][a] - L.G2 * ps[k] * S2[k][a] - L.GAB * r[k] * S3[k][a] + r[k] * L.g[a];
-            double jx, jy;
-            first_moment<double>(fk[k], jx, jy);
-            m[k][0] = jx + 0.5 * F[k][0];
-            m[k][1] = jy + 0.5 * F[k][1];
+            constexpr double w0 = 4.0 / 9.0, w1 = 1.0 / 9.0, w2 = 1.0 / 36.0;
+            double l[9], lf = 0.0;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) l[i] = pull_lam(L, lam_next, k, i, x, y);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) lf = __fma_rn(l[i], f[(size_t)(k * 9 + i) * L.plane + c], lf);
+            const double ax = A.add(l[1], l[3]), ay = A.add(l[2], l[4]), p57 = A.add(l[5], l[7]), p68 = A.add(l[6], l[8]);
+            const double m57 = A.sub(l[5], l[7]), m68 = A.sub(l[6], l[8]), dg = w2 * A.add(p57, p68);
+            const double M0 = __fma_rn(w0, l[0], __fma_rn(w1, A.add(ax, ay), dg));
+            const double M1x = __fma_rn(w1, A.sub(l[1], l[3]), w2 * A.sub(m57, m68));
+            const double M1y = __fma_rn(w1, A.sub(l[2], l[4]), w2 * A.add(m57, m68));
+            const double Mxx = __fma_rn(w1, ax, dg), Myy = __fma_rn(w1, ay, dg), Mxy = w2 * A.sub(p57, p68);
+            const double Mux = __fma_rn(Mxx, u[0], Mxy * u[1]), Muy = __fma_rn(Mxy, u[0], Myy * u[1]);
+            const double Vx = __fma_rn(9.0, Mux, 3.0 * __fma_rn(-u[0], M0, M1x));
+            const double Vy = __fma_rn(9.0, Muy, 3.0 * __fma_rn(-u[1], M0, M1y));
+            const double a = __fma_rn(-0.5, om[k], 1.0), omr = om[k] * r[k], a9 = 9.0 * a, a3M = -3.0 * a * M0;
+            ub[0] = __fma_rn(omr, Vx, __fma_rn(a9, __fma_rn(Mxx, F[k][0], Mxy * F[k][1]), __fma_rn(a3M, F[k][0], ub[0])));
+            ub[1] = __fma_rn(omr, Vy, __fma_rn(a9, __fma_rn(Mxy, F[k][0], Myy * F[k][1]), __fma_rn(a3M, F[k][1], ub[1])));
+            aV[k][0] = a * Vx;
+            aV[k][1] = a * Vy;
+            double P = __fma_rn(-uu15, M0, M0);
+            P = __fma_rn(3.0, __fma_rn(M1x, u[0], M1y * u[1]), P);
+            P = __fma_rn(4.5, __fma_rn(u[0], Mux, u[1] * Muy), P);
+            rb[k] = om[k] * P;
+            omb[k] = __fma_rn(-0.5, __fma_rn(Vx, F[k][0], Vy * F[k][1]), __fma_rn(r[k], P, -lf));
         }
-        const double om[2] = {L.omega[0], L.omega[1]};
-        const double D = om[0] * r[0] + om[1] * r[1];
-        const double u[2] = {(om[0] * m[0][0] + om[1] * m[1][0]) / D, (om[0] * m[0][1] + om[1] * m[1][1]) / D};
-        const double uu = u[0] * u[0] + u[1] * u[1];
-
-        double ub[2] = {0.0, 0.0}, Fb[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, rb[2] = {0.0, 0.0};
-        double mb[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, omb[2] = {0.0, 0.0};
-        if (seed_kind == 0) {
-            for (int k = 0; k < 2; ++k) {
-                const double a = 1.0 - 0.5 * om[k];
-                for (int i = 0; i < 9; ++i) {
-                    const double ls = pull_lam(L, lam_next, k, i, x, y);
-                    const double e[2] = {(double)ex9(i), (double)ey9(i)}, w = w9(i);
-                    const double eu = e[0] * u[0] + e[1] * u[1], eF = e[0] * F[k][0] + e[1] * F[k][1];
-                    const double poly = 1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * uu;
-                    const double feq = w * r[k] * poly;
-                    for (int d = 0; d < 2; ++d) {
-                        // d feq / d u and d C / d u
-                        ub[d] += ls * (om[k] * w * r[k] * (3.0 * e[d] + 9.0 * eu * e[d] - 3.0 * u[d])
-                                       + a * w * (-3.0 * F[k][d] + 9.0 * eF * e[d]));
-                        // d C / d F
-                        Fb[k][d] += ls * a * w * (3.0 * (e[d] - u[d]) + 9.0 * eu * e[d]);
-                    }
-                    rb[k] += ls * om[k] * w * poly;
-                    const double guo = w * (3.0 * ((e[0] - u[0]) * F[k][0] + (e[1] - u[1]) * F[k][1]) + 9.0 * eu * eF);
-                    omb[k] += ls * (-(fk[k][i] - feq) - 0.5 * guo);
-                }
-            }
-            // u = N / D
-            const double Nb[2] = {ub[0] / D, ub[1] / D};
-            const double Db = -(ub[0] * u[0] + ub[1] * u[1]) / D;
-            for (int k = 0; k < 2; ++k) {
-                mb[k][0] = om[k] * Nb[0];
-                mb[k][1] = om[k] * Nb[1];
-                omb[k] += Nb[0] * m[k][0] + Nb[1] * m[k][1] + Db * r[k];
-                rb[k] += om[k] * Db;
-            }
-        } else if (seed_kind == 1) {
-            // J = Q0 / Q, Q = (1/nx) sum ubar_x, ubar = (m_A + m_B) / (rho_A + rho_B)
-            const double rt = r[0] + r[1], ubx = (m[0][0] + m[1][0]) / rt;
-            const double s = seed_a / L.nx;
-            for (int k = 0; k < 2; ++k) {
-                mb[k][0] = s / rt;
-                rb[k] = -s * ubx / rt;
-            }
-        } else {
-            // J = <p_b>_in - <p_b>_out, Eq. (11)
-            double dx = fabs((double)x - L.probe[0]), dy = fabs((double)y - L.probe[1]);
-            if (dx > 0.5 * L.nx) dx = L.nx - dx;
-            if (!L.walls && dy > 0.5 * L.ny) dy = L.ny - dy;
-            const double rr = sqrt(dx * dx + dy * dy), R = L.probe[2];
-            const double cw = (rr < 0.5 * R ? seed_a : 0.0) + (rr > R + 6.0 ? seed_b : 0.0);
-            if (cw != 0.0) {
-                const double Gs = L.G1 + L.G2;
-                for (int k = 0; k < 2; ++k)
-                    rb[k] = cw * ((1.0 + Gs * ps[k] * exp(-r[k])) / 3.0 + L.GAB * r[1 - k] / 3.0);
-                gr[gG1] += cw * 0.5 * (ps[0] * ps[0] + ps[1] * ps[1]) / 3.0;
-                gr[gG2] += cw * 0.5 * (ps[0] * ps[0] + ps[1] * ps[1]) / 3.0;
-                gr[gGAB] += cw * r[0] * r[1] / 3.0;
-            }
-        }
-        // m = j + F/2
+        // u = N / D
+        const double Nb[2] = {ub[0] * rD, ub[1] * rD};
+        const double Db = -__fma_rn(Nb[0], u[0], Nb[1] * u[1]);
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
-            Fb[k][0] += 0.5 * mb[k][0];
-            Fb[k][1] += 0.5 * mb[k][1];
+            mb[k][0] = om[k] * Nb[0];
+            mb[k][1] = om[k] * Nb[1];
+            omb[k] = __fma_rn(Nb[0], m[k][0], __fma_rn(Nb[1], m[k][1], __fma_rn(Db, r[k], omb[k])));
+            rb[k] = __fma_rn(om[k], Db, rb[k]);
         }
-        // F = -G1 psi S1 - G2 psi S2 - G_AB rho S3 + rho g
-        double psb[2], S1b[2][2], S2b[2][2], S3b[2][2];
+    } else if (seed_kind == 1) {
+        // J = Q0 / Q, Q = (1/nx) sum ubar_x, ubar = (m_A + m_B) / (rho_A + rho_B)
+        const double rt = r[0] + r[1], ubx = (m[0][0] + m[1][0]) / rt;
+        const double s = seed_a / L.nx;
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
-            psb[k] = -(Fb[k][0] * (L.G1 * S1[k][0] + L.G2 * S2[k][0]) + Fb[k][1] * (L.G1 * S1[k][1] + L.G2 * S2[k][1]));
-            rb[k] += Fb[k][0] * (L.g[0] - L.GAB * S3[k][0]) + Fb[k][1] * (L.g[1] - L.GAB * S3[k][1]);
-            for (int d = 0; d < 2; ++d) {
-                S1b[k][d] = -L.G1 * ps[k] * Fb[k][d];
-                S2b[k][d] = -L.G2 * ps[k] * Fb[k][d];
-                S3b[k][d] = -L.GAB * r[k] * Fb[k][d];
-            }
-            gr[gG1] += -ps[k] * (Fb[k][0] * S1[k][0] + Fb[k][1] * S1[k][1]);
-            gr[gG2] += -ps[k] * (Fb[k][0] * S2[k][0] + Fb[k][1] * S2[k][1]);
-            gr[gGAB] += -r[k] * (Fb[k][0] * S3[k][0] + Fb[k][1] * S3[k][1]);
+            mb[k][0] = s / rt;
+            rb[k] = -s * ubx / rt;
         }
-        gr[gOmA] += omb[0];
-        gr[gOmB] += omb[1];
-        const double vals[kAdjSlots] = {psb[0], psb[1], rb[0], rb[1], mb[0][0], mb[0][1], mb[1][0], mb[1][1],
-                                        S1b[0][0], S1b[0][1], S1b[1][0], S1b[1][1], S2b[0][0], S2b[0][1],
-                                        S2b[1][0], S2b[1][1], S3b[0][0], S3b[0][1], S3b[1][0], S3b[1][1]};
-        for (int s = 0; s < kAdjSlots; ++s) abuf[(size_t)s * L.plane + c] = vals[s];
+    } else {
+        // J = <p_b>_in - <p_b>_out, Eq. (11)
+        double dx = fabs((double)x - L.probe[0]), dy = fabs((double)y - L.probe[1]);
+        if (dx > 0.5 * L.nx) dx = L.nx - dx;
+        if (!L.walls && dy > 0.5 * L.ny) dy = L.ny - dy;
+        const double rr = sqrt(dx * dx + dy * dy), R = L.probe[2];
+        const double cw = (rr < 0.5 * R ? seed_a : 0.0) + (rr > R + 6.0 ? seed_b : 0.0);
+        if (cw != 0.0) {
+            const double Gs = L.G1 + L.G2, ps[2] = {spsi[0][cy][cx], spsi[1][cy][cx]};
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                rb[k] = cw * ((1.0 + Gs * ps[k] * rho[(size_t)(2 + k) * L.plane + c]) / 3.0 + L.GAB * r[1 - k] / 3.0);
+            gr[gG1] += cw * 0.5 * (ps[0] * ps[0] + ps[1] * ps[1]) / 3.0;
+            gr[gG2] += cw * 0.5 * (ps[0] * ps[0] + ps[1] * ps[1]) / 3.0;
+            gr[gGAB] += cw * r[0] * r[1] / 3.0;
+        }
     }
-    // per-tile gradient partials, added to the tile's running sums (one block
-    // per tile per step: a fixed order)
+    auto put = [&](int slot, double v) { abuf[(size_t)slot * L.plane + c] = v; };
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        // m = j + F/2, then F = -psi (G1 S1 + G2 S2) - G_AB rho S3 + rho g
+        const double Fb[2] = {__fma_rn(0.5, mb[k][0], aV[k][0]), __fma_rn(0.5, mb[k][1], aV[k][1])};
+        const double ps = spsi[k][cy][cx], T[2] = {ps * Fb[0], ps * Fb[1]}, Q[2] = {r[k] * Fb[0], r[k] * Fb[1]};
+        const double f1 = __fma_rn(Fb[0], S1[k][0], Fb[1] * S1[k][1]), f2 = __fma_rn(Fb[0], S2[k][0], Fb[1] * S2[k][1]);
+        const double f3 = __fma_rn(Fb[0], S3[k][0], Fb[1] * S3[k][1]);
+        put(aPsiA + k, -__fma_rn(L.G1, f1, L.G2 * f2));
+        put(aRhoA + k, __fma_rn(-L.GAB, f3, __fma_rn(Fb[0], L.g[0], __fma_rn(Fb[1], L.g[1], rb[k]))));
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            put(aMAx + 2 * k + a, mb[k][a]);
+            put(aTAx + 2 * k + a, T[a]);
+            put(aQAx + 2 * k + a, Q[a]);
+        }
+        gr[gG1] = __fma_rn(-ps, f1, gr[gG1]);
+        gr[gG2] = __fma_rn(-ps, f2, gr[gG2]);
+        gr[gGAB] = __fma_rn(-r[k], f3, gr[gGAB]);
+    }
+    gr[gOmA] = omb[0];
+    gr[gOmB] = omb[1];
+    // the node's running sums over the steps (reduced once, by k_adj_reduce:
+    // a reduction per step would cost as many FP64 instructions as a stencil)
+#pragma unroll
     for (int a = 0; a < kAdjGrads; ++a) {
-        const double v = warp_sum(gr[a]);
-        if ((tid & 31) == 0) sred[tid >> 5][a] = v;
-    }
-    __syncthreads();
-    if (tid < kAdjGrads) {
-        double v = sred[0][tid];
-        for (int w = 1; w < kThreads / 32; ++w) v += sred[w][tid];
-        gpart[(size_t)blockIdx.x * 8 + tid] += v;
+        double *g = &gpart[(size_t)a * L.plane + c];
+        *g = A.add(*g, gr[a]);
     }
 }
 
-// Rows x_y of the nodes whose stencil vector of y-component ey reads row y_y
-// (mirror ghosts included): writes up to 3 rows into rows[], returns count.
-__device__ __forceinline__ int source_rows(const Lat<double> &L, int yy, int ey, int rows[3])
+// sum_e c(|e|^2) e_x v(x + e) over D2Q25 of a staged plane (AX = 0; e_y for
+// AX = 1), c(1), c(2) given and c = G2 p beyond.
+template <int AX>
+__device__ __forceinline__ double gather25(const Arith64<false> &A, const double (*v)[SW], int cx, int cy, double c1,
+                                           double c2, double G2)
 {
-    int n = 0;
-    const int r1 = yy - ey;
-    if (!L.walls) {
-        rows[n++] = wrapi(r1 < 0 ? r1 + L.ny : r1, L.ny);   // |ey| <= 2 < ny
-        return n;
-    }
-    if (r1 >= 0 && r1 < L.ny) rows[n++] = r1;
-    if (L.wall_mode == 0) {
-        const int r2 = -1 - yy - ey;                 // read ghost row r2 + ey < 0 mirrored to yy
-        if (r2 >= 0 && r2 < L.ny && r2 + ey < 0) rows[n++] = r2;
-        const int r3 = 2 * L.ny - 1 - yy - ey;       // ghost row >= ny mirrored to yy
-        if (r3 >= 0 && r3 < L.ny && r3 + ey >= L.ny) rows[n++] = r3;
-    }
-    return n;
+    auto at = [&](int along, int across) { return AX == 0 ? v[cy + across][cx + along] : v[cy + along][cx + across]; };
+    auto two = [&](int along, int across) {   // both sides across the axis
+        return A.add(A.sub(at(along, across), at(-along, across)), A.sub(at(along, -across), at(-along, -across)));
+    };
+    double o = p25(8) * 2.0 * two(2, 2);
+    o = __fma_rn(p25(5) * 2.0, two(2, 1), o);
+    o = __fma_rn(p25(5), two(1, 2), o);
+    o = __fma_rn(p25(4) * 2.0, A.sub(at(2, 0), at(-2, 0)), o);
+    return __fma_rn(c1, A.sub(at(1, 0), at(-1, 0)), __fma_rn(c2, two(1, 1), G2 * o));
 }
 
-// Phase B: gather the stencil adjoints and form lam(t).
+template <int AX>
+__device__ __forceinline__ double gather9(const Arith64<false> &A, const double (*v)[SW], int cx, int cy)
+{
+    auto at = [&](int along, int across) { return AX == 0 ? v[cy + across][cx + along] : v[cy + along][cx + across]; };
+    const double d = A.add(A.sub(at(1, 1), at(-1, 1)), A.sub(at(1, -1), at(-1, -1)));
+    return __fma_rn(1.0 / 9.0, A.sub(at(1, 0), at(-1, 0)), (1.0 / 36.0) * d);
+}
+
+// Phase B: gather the stencil adjoints and form lam(t).  psi_bar takes
+// sum_e (G1 w + G2 p) e.T(x + e) and rho_bar of a species G_AB sum_e w e.Q(x + e)
+// of the other (the stencils are odd, so a transposed one is its negative), from
+// T and Q of the tile and its halo staged in shared memory.  Ghost rows beyond
+// a wall hold no node and give nothing; what the stencils of nodes near a
+// mirroring wall read from a ghost row goes to the fluid node it copies.
 __global__ void __launch_bounds__(kThreads) k_adj_gather(const Lat<double> L, const double *__restrict__ rho,
                                                          const double *__restrict__ lam_next,
                                                          const double *__restrict__ abuf, double *__restrict__ lam_out,
                                                          int seed)
 {
-    const int x = blockIdx.x * TX + threadIdx.x;
-    const int y = blockIdx.y * TY + threadIdx.y;
+    __shared__ double sv[8][SH][SW];   // T A x, y, B x, y, then Q
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    for (int idx = tid; idx < SW * SH; idx += kThreads) {
+        const int sx = idx % SW, sy = idx / SW;
+        const int gx = wrap_index(x0 + sx - HALO, L.nx);
+        int gy = y0 + sy - HALO;
+        const bool ghost = L.walls && (gy < 0 || gy >= L.ny);
+        gy = ghost ? 0 : wrap_index(gy, L.ny);
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+            sv[v][sy][sx] = ghost ? 0.0 : abuf[(size_t)(aTAx + v) * L.plane + (size_t)gy * L.pitch + gx];
+    }
+    __syncthreads();
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= L.nx || y >= L.ny) return;
+    const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
     const size_t c = (size_t)y * L.pitch + x;
-    auto A = [&](int slot, int xx, int yy) { return abuf[(size_t)slot * L.plane + (size_t)yy * L.pitch + xx]; };
-    double psb[2] = {A(aPsiA, x, y), A(aPsiB, x, y)};
-    double rb[2] = {A(aRhoA, x, y), A(aRhoB, x, y)};
-    // D2Q25 (p weights) and D2Q9 (w weights) transposed stencils
-    for (int j = 0; j < 25; ++j) {
-        const int dx = j % 5 - 2, dy = j / 5 - 2;
-        if (dx == 0 && dy == 0) continue;
-        const double p = p25(dx * dx + dy * dy);
-        const bool q9 = dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1;
-        const double w = q9 ? w9(dx == 0 ? (dy > 0 ? 2 : 4) : (dy == 0 ? (dx > 0 ? 1 : 3) : 5)) : 0.0;
-        const int xs = wrapi(x - dx, L.nx);
-        int rows[3];
-        const int nr = source_rows(L, y, dy, rows);
-        for (int q = 0; q < nr; ++q) {
-            const int ys = rows[q];
-            for (int k = 0; k < 2; ++k) {
-                psb[k] += p * (dx * A(k == 0 ? aS2Ax : aS2Bx, xs, ys) + dy * A(k == 0 ? aS2Ay : aS2By, xs, ys));
-                if (q9) {
-                    psb[k] += w * (dx * A(k == 0 ? aS1Ax : aS1Bx, xs, ys) + dy * A(k == 0 ? aS1Ay : aS1By, xs, ys));
-                    // S3 of the other species reads this species' density
-                    rb[k] += w * (dx * A(k == 0 ? aS3Bx : aS3Ax, xs, ys) + dy * A(k == 0 ? aS3By : aS3Ay, xs, ys));
+    const Arith64<false> A(opaque_one());
+    const double c1 = -L.cw[0], c2 = -L.cw[1];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        double psb = A.add(gather25<0>(A, sv[2 * k], cx, cy, c1, c2, L.G2), gather25<1>(A, sv[2 * k + 1], cx, cy, c1, c2, L.G2));
+        double q = A.add(gather9<0>(A, sv[6 - 2 * k], cx, cy), gather9<1>(A, sv[7 - 2 * k], cx, cy));
+        if (L.walls && L.wall_mode == 0 && (y < HALO || y >= L.ny - HALO)) {
+            // the mirrored ghost rows this node is copied to: row g of the
+            // ghosts, read by nodes of row g - ey with stencil vectors (dx, ey)
+            for (int side = 0; side < 2; ++side) {
+                const int g = side == 0 ? -1 - y : 2 * L.ny - 1 - y;
+                for (int j = 0; j < 25; ++j) {
+                    const int dx = j % 5 - 2, ey = j / 5 - 2, e2 = dx * dx + ey * ey, row = g - ey;
+                    if (e2 == 0 || row < 0 || row >= L.ny || (side == 0 ? g + HALO < 0 : g - HALO >= L.ny)) continue;
+                    const int xs = wrapi(x - dx, L.nx);
+                    auto V = [&](int slot) { return abuf[(size_t)slot * L.plane + (size_t)row * L.pitch + xs]; };
+                    const double w = e2 == 1 ? 1.0 / 9.0 : e2 == 2 ? 1.0 / 36.0 : 0.0;
+                    psb -= (L.G1 * w + L.G2 * p25(e2)) * (dx * V(aTAx + 2 * k) + ey * V(aTAy + 2 * k));
+                    if (e2 <= 2) q -= w * (dx * V(aQBx - 2 * k) + ey * V(aQBy - 2 * k));
                 }
             }
         }
-    }
-    for (int k = 0; k < 2; ++k) rb[k] += exp(-rho[(size_t)k * L.plane + c]) * psb[k];
-    const double mb[2][2] = {{A(aMAx, x, y), A(aMAy, x, y)}, {A(aMBx, x, y), A(aMBy, x, y)}};
-    for (int k = 0; k < 2; ++k)
+        psb = A.add(psb, abuf[(size_t)(aPsiA + k) * L.plane + c]);
+        const double rb = __fma_rn(rho[(size_t)(2 + k) * L.plane + c], psb,
+                                   __fma_rn(L.GAB, q, abuf[(size_t)(aRhoA + k) * L.plane + c]));
+        const double mx = abuf[(size_t)(aMAx + 2 * k) * L.plane + c], my = abuf[(size_t)(aMAy + 2 * k) * L.plane + c];
+        const double s = A.add(mx, my), d = A.sub(mx, my), h = __fma_rn(-1.0, L.omega[k], 1.0);
+        // m_bar . e_i + rho_bar
+        const double base[9] = {rb, A.add(rb, mx), A.add(rb, my), A.sub(rb, mx), A.sub(rb, my), A.add(rb, s), A.sub(rb, d),
+                                A.sub(rb, s), A.add(rb, d)};
+#pragma unroll
         for (int i = 0; i < 9; ++i) {
             const double ls = seed ? 0.0 : pull_lam(L, lam_next, k, i, x, y);
-            lam_out[(size_t)(k * 9 + i) * L.plane + c] =
-                (1.0 - L.omega[k]) * ls + mb[k][0] * ex9(i) + mb[k][1] * ey9(i) + rb[k];
+            lam_out[(size_t)(k * 9 + i) * L.plane + c] = __fma_rn(h, ls, base[i]);
         }
+    }
 }
 
-// rho_k = sum_i f_k,i for the adjoint's recomputed states
+// rho_k = sum_i f_k,i and exp(-rho_k) (planes 0, 1 and 2, 3 of rho) for the
+// adjoint's recomputed states
 __global__ void k_adj_density(const Lat<double> L, const double *__restrict__ f, double *__restrict__ rho)
 {
     const int x = blockIdx.x * TX + threadIdx.x;
     const int y = blockIdx.y * TY + threadIdx.y;
     if (x >= L.nx || y >= L.ny) return;
     const size_t c = (size_t)y * L.pitch + x;
+    const double one = opaque_one();
     for (int k = 0; k < 2; ++k) {
         double v[9];
         for (int i = 0; i < 9; ++i) v[i] = f[(size_t)(k * 9 + i) * L.plane + c];
-        rho[(size_t)k * L.plane + c] = zeroth_moment<double>(v, L.one);
+        const double r = zeroth_moment<double>(v, one);
+        rho[(size_t)k * L.plane + c] = r;
+        rho[(size_t)(2 + k) * L.plane + c] = exp(-r);
     }
 }
 
-// Fixed-order reduction of the per-tile gradient sums.
-__global__ void k_adj_reduce(const double *__restrict__ gpart, int n_tiles, double *__restrict__ out)
+// Fixed-order reduction of the per-node gradient sums: one block a parameter.
+__global__ void __launch_bounds__(1024) k_adj_reduce(const double *__restrict__ gpart, size_t plane, double *__restrict__ out)
 {
-    __shared__ double s[256];
-    for (int a = 0; a < kAdjGrads; ++a) {
-        double v = 0.0;
-        for (int t = threadIdx.x; t < n_tiles; t += 256) v += gpart[(size_t)t * 8 + a];
-        s[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[a] = s[0];
+    __shared__ double s[1024];
+    double v = 0.0;
+    for (size_t i = threadIdx.x; i < plane; i += 1024) v += gpart[blockIdx.x * plane + i];
+    s[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 512; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[blockIdx.x] = s[0];
 }
 
 cudaError_t adj_density(const Lat<double> &L, const double *f, double *rho, cudaStream_t s)
@@ -318,9 +408,9 @@ cudaError_t adj_step(const Lat<double> &L, const double *f, const double *rho, c
     return cudaGetLastError();
 }
 
-cudaError_t adj_reduce(const double *gpart, int n_tiles, double *out, cudaStream_t s)
+cudaError_t adj_reduce(const Lat<double> &L, const double *gpart, double *out, cudaStream_t s)
 {
-    k_adj_reduce<<<1, 256, 0, s>>>(gpart, n_tiles, out);
+    k_adj_reduce<<<kAdjGrads, 1024, 0, s>>>(gpart, L.plane, out);
     return cudaGetLastError();
 }
 

@@ -806,12 +806,9 @@ struct lb_engine {
         const size_t state = pop_bytes(0) + ref_bytes(0);
         const int64_t nseg = (nsteps + ckpt - 1) / ckpt;
         const int seg_len = (int)std::min<int64_t>(ckpt, nsteps);
-        const int tiles_x = (p.nx + lbk::TX - 1) / lbk::TX, tiles_y = (p.ny + lbk::TY - 1) / lbk::TY;
-        const int ntl = tiles_x * tiles_y;
         char *mem = nullptr;
         const size_t bytes = (size_t)nseg * state + (size_t)seg_len * pop64 + 2 * pop64 + state + (f32 ? pop64 : 0) +
-                             lbk::kAdjSlotCount * plane_b + 2 * plane_b + (size_t)ntl * 8 * sizeof(double) +
-                             8 * sizeof(double);
+                             (lbk::kAdjSlotCount + 4 + lbk::kAdjGradPlanes) * plane_b + 8 * sizeof(double);
         if (cudaMalloc((void **)&mem, bytes) != cudaSuccess) {
             cudaGetLastError();
             return fail(LB_ENOMEM, "lb_grad: no room for checkpoints and adjoint buffers");
@@ -822,9 +819,9 @@ struct lb_engine {
         double *lam[2] = {(double *)take(pop64), (double *)take(pop64)};
         char *final_state = take(state);
         double *fT64 = f32 ? (double *)take(pop64) : nullptr;
-        double *abuf = (double *)take(lbk::kAdjSlotCount * plane_b), *rho = (double *)take(2 * plane_b);
-        double *gpart = (double *)take((size_t)ntl * 8 * sizeof(double)), *gout = (double *)take(8 * sizeof(double));
-        cudaError_t ce = cudaMemsetAsync(gpart, 0, (size_t)ntl * 8 * sizeof(double), stream);
+        double *abuf = (double *)take(lbk::kAdjSlotCount * plane_b), *rho = (double *)take(4 * plane_b);
+        double *gpart = (double *)take(lbk::kAdjGradPlanes * plane_b), *gout = (double *)take(8 * sizeof(double));
+        cudaError_t ce = cudaMemsetAsync(gpart, 0, lbk::kAdjGradPlanes * plane_b, stream);
         auto done = [&](int code) {
             cudaStreamSynchronize(stream);
             cudaFree(mem);
@@ -903,9 +900,9 @@ struct lb_engine {
                 cur ^= 1;
             }
         }
-        if (ce == cudaSuccess) ce = lbk::adj_reduce(gpart, ntl, gout, stream);
+        if (ce == cudaSuccess) ce = lbk::adj_reduce(L, gpart, gout, stream);
         double g[8] = {0};
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(g, gout, 8 * sizeof(double), cudaMemcpyDeviceToHost, stream);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(g, gout, lbk::kAdjGradPlanes * sizeof(double), cudaMemcpyDeviceToHost, stream);
         // put the final state back (the recomputation used both population copies)
         if (ce == cudaSuccess) ce = load_state(final_state, 0);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(stream);
@@ -936,9 +933,7 @@ struct lb_engine {
         const lb_params &p = P[0];
         const lbk::Lat<double> &L = L64[0];
         const size_t plane_b = plane(0) * sizeof(double), pop64 = 18 * plane_b;
-        const int ntl = ((p.nx + lbk::TX - 1) / lbk::TX) * ((p.ny + lbk::TY - 1) / lbk::TY);
-        const size_t bytes = 2 * pop64 + lbk::kAdjSlotCount * plane_b + 2 * plane_b + (size_t)ntl * 8 * sizeof(double) +
-                             8 * sizeof(double);
+        const size_t bytes = 2 * pop64 + (lbk::kAdjSlotCount + 4 + lbk::kAdjGradPlanes) * plane_b + 8 * sizeof(double);
         char *mem = nullptr;
         if (cudaMalloc((void **)&mem, bytes) != cudaSuccess) {
             cudaGetLastError();
@@ -947,19 +942,19 @@ struct lb_engine {
         char *q = mem;
         auto take = [&](size_t b) { char *r = q; q += b; return r; };
         double *lam_in = (double *)take(pop64), *lam_out = (double *)take(pop64);
-        double *abuf = (double *)take(lbk::kAdjSlotCount * plane_b), *rho = (double *)take(2 * plane_b);
-        double *gpart = (double *)take((size_t)ntl * 8 * sizeof(double)), *gout = (double *)take(8 * sizeof(double));
+        double *abuf = (double *)take(lbk::kAdjSlotCount * plane_b), *rho = (double *)take(4 * plane_b);
+        double *gpart = (double *)take(lbk::kAdjGradPlanes * plane_b), *gout = (double *)take(8 * sizeof(double));
         const double *f = (const double *)fbuf(0, parity);
         const size_t row = (size_t)p.nx * sizeof(double), prow = (size_t)L.pitch * sizeof(double);
         cudaError_t ce = cudaMemsetAsync(mem, 0, 2 * pop64, stream);   // the pitch padding stays zero
-        if (ce == cudaSuccess) ce = cudaMemsetAsync(gpart, 0, (size_t)ntl * 8 * sizeof(double), stream);
+        if (ce == cudaSuccess) ce = cudaMemsetAsync(gpart, 0, lbk::kAdjGradPlanes * plane_b, stream);
         if (ce == cudaSuccess)
             ce = cudaMemcpy2DAsync(lam_in, prow, w, row, row, (size_t)18 * p.ny, cudaMemcpyHostToDevice, stream);
         if (ce == cudaSuccess) ce = lbk::adj_density(L, f, rho, stream);
         if (ce == cudaSuccess) ce = lbk::adj_step(L, f, rho, lam_in, abuf, gpart, lam_out, 0, 0.0, 0.0, stream);
-        if (ce == cudaSuccess) ce = lbk::adj_reduce(gpart, ntl, gout, stream);
+        if (ce == cudaSuccess) ce = lbk::adj_reduce(L, gpart, gout, stream);
         double g[8] = {0};
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(g, gout, 8 * sizeof(double), cudaMemcpyDeviceToHost, stream);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(g, gout, lbk::kAdjGradPlanes * sizeof(double), cudaMemcpyDeviceToHost, stream);
         if (ce == cudaSuccess && out)
             ce = cudaMemcpy2DAsync(out, row, lam_out, prow, row, (size_t)18 * p.ny, cudaMemcpyDeviceToHost, stream);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(stream);

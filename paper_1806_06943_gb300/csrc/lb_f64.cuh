@@ -101,6 +101,14 @@ __device__ __forceinline__ uint32_t velocity_outside(double x)
     return (((hi & 0x7fffffffu) | lo) == 0u) ? 0u : ((hi + 0x10000000u) ^ 0x40000000u) & 0x60000000u;
 }
 
+// 1.0 in a register, for kernels without a lattice descriptor in memory.
+__device__ __forceinline__ double opaque_one()
+{
+    double v;
+    asm volatile("mov.f64 %0, 0d3FF0000000000000;" : "=d"(v));
+    return v;
+}
+
 // Arithmetic of a node: sums as register fmas, products by factor_mul (kInt)
 // or the FP64 pipe (the same bits).
 template <bool kInt>

@@ -91,18 +91,20 @@ cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile
                              const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, int ty, cudaStream_t s);
 
 // Discrete adjoint of the FP64 step (lb_adjoint.cu).  Buffers use the
-// lattice's pitched layout; abuf holds 20 planes, gpart 8 doubles per tile of
-// 32 x 4 nodes.  seed_kind: 0 adjoint step (lam_next = dJ/df(t+1)), 1 seed of
+// lattice's pitched layout: rho 4 planes (densities and exp(-rho)), abuf
+// kAdjSlotCount, gpart kAdjGradPlanes (zero before the first step; the pitch
+// padding stays zero).  seed_kind: 0 adjoint step (lam_next = dJ/df(t+1)), 1 seed of
 // mu_r (seed_a = dJ/dQ), 2 seed of the Laplace pressure jump (seed_a = 1/n_in,
 // seed_b = -1/n_out, probe in L).
 cudaError_t adj_density(const Lat<double> &L, const double *f, double *rho, cudaStream_t s);
 cudaError_t adj_step(const Lat<double> &L, const double *f, const double *rho, const double *lam_next, double *abuf,
                      double *gpart, double *lam_out, int seed_kind, double seed_a, double seed_b, cudaStream_t s);
-cudaError_t adj_reduce(const double *gpart, int n_tiles, double *out, cudaStream_t s);
+cudaError_t adj_reduce(const Lat<double> &L, const double *gpart, double *out, cudaStream_t s);
 // FP64 populations f_i = h_i + w_i R of an FP32 state (18 offset planes h,
 // 2 reference-density planes R), pitched like the lattice (lb_fp32.cu).
 cudaError_t offset_to_f64(const Lat<float> &L, const float *h, const float *R, double *out, cudaStream_t s);
-constexpr int kAdjSlotCount = 20;
+constexpr int kAdjSlotCount = 16;
+constexpr int kAdjGradPlanes = 5;
 
 // Record msg as the calling thread's lb_last_error() message.
 void set_last_error(const char *msg);
