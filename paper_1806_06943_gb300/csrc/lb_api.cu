@@ -179,11 +179,10 @@ struct lb_engine {
     void *d_pool = nullptr;
     size_t pool_bytes = 0;
     // LB_MODE_TMA: one set of tensor maps per lattice (FP32 only), and per
-    // tile height the time-step tiles reordered: the n_box tiles staged by TMA
-    // first, then the others
+    // tile height the time-step tiles reordered: the tiles staged by TMA first,
+    // then the others
     lbk::TmaMaps *d_tmaps = nullptr;
     int4 *d_btiles[3] = {nullptr, nullptr, nullptr};
-    int n_box[3] = {0, 0, 0};
     // FP64 lattices of few nodes: one-row tiles (chain by chain for a batch)
     // of k_small64, which both LB_MODE_LAUNCH and LB_MODE_FUSED then step with
     int4 *d_rows = nullptr;
@@ -210,7 +209,7 @@ struct lb_engine {
     cudaStream_t aux[kChains] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kChains] = {};
     int4 *d_ctiles[3] = {nullptr, nullptr, nullptr};
-    int c_off[3][kChains] = {}, c_box[3][kChains] = {}, c_cnt[3][kChains] = {};
+    int c_off[3][kChains] = {}, c_cnt[3][kChains] = {};
 
     ~lb_engine()
     {
@@ -298,15 +297,10 @@ struct lb_engine {
         }
         return e;
     }
-    // LB_MODE_TMA step: the TMA kernel over the box tiles, the plain one-pass
-    // kernel over the rest
+    // LB_MODE_TMA step over all tiles, box tiles first
     cudaError_t launch_tma(const lbk::Lat<float> *L, int ti, int nt, int par)
     {
-        cudaError_t e = lbk::launch_fused_tma(L, d_btiles[ti], 0, n_box[ti], par, d_tmaps, d_err, wait_cycles, drop_tile,
-                                              ty, stream);
-        if (e == cudaSuccess && nt > n_box[ti])
-            e = lbk::Launch<float>::fused(L, d_btiles[ti], n_box[ti], nt - n_box[ti], par, ty, stream);
-        return e;
+        return lbk::launch_fused_tma(L, d_btiles[ti], 0, nt, par, d_tmaps, d_err, wait_cycles, drop_tile, ty, stream);
     }
     size_t ctl_bytes() const { return 8 + 2 * sizeof(unsigned) * (size_t)n; }
     // nsteps time steps in one persistent launch (counters cleared first)
@@ -329,7 +323,7 @@ struct lb_engine {
     // one time step of the lattices of chain g on stream s
     cudaError_t launch_chain_step(int g, int par, cudaStream_t s)
     {
-        const int ti = ty_index(ty), off = c_off[ti][g], nb = c_box[ti][g], cnt = c_cnt[ti][g];
+        const int ti = ty_index(ty), off = c_off[ti][g], cnt = c_cnt[ti][g];
         const int4 *T = d_ctiles[ti];
         if (cnt == 0) return cudaSuccess;
         cudaError_t e;
@@ -343,11 +337,8 @@ struct lb_engine {
         }
         const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
         if (mode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, T, off, cnt, par, ty, s);
-        if (mode == LB_MODE_TMA) {
-            e = lbk::launch_fused_tma(L, T, off, nb, par, d_tmaps, d_err, wait_cycles, drop_tile, ty, s);
-            if (e == cudaSuccess && cnt > nb) e = lbk::Launch<float>::fused(L, T, off + nb, cnt - nb, par, ty, s);
-            return e;
-        }
+        if (mode == LB_MODE_TMA)
+            return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, wait_cycles, drop_tile, ty, s);
         e = lbk::Launch<float>::density(L, T, off, cnt, par, ty, s);
         if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, T, off, cnt, par, ty, s);
         return e;
@@ -449,7 +440,6 @@ struct lb_engine {
                 else
                     rest.push_back(t);
             }
-            n_box[ti] = (int)box.size();
             box.insert(box.end(), rest.begin(), rest.end());
             if (cudaMalloc((void **)&d_btiles[ti], box.size() * sizeof(int4)) != cudaSuccess) {
                 cudaGetLastError();
@@ -503,7 +493,6 @@ struct lb_engine {
         if (h) {
             LB_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
             LB_CUDA(cudaStreamSynchronize(stream));
-            if (h == 2) return fail(LB_ECUDA, "internal: a tile of the TMA list is not a box tile; the state is invalid");
             return fail(LB_ETIMEOUT, "a bounded device-side wait expired (persistent kernel or TMA copy); the state is invalid");
         }
         return LB_OK;
@@ -1318,7 +1307,6 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
                     for (const int4 &t : e->stiles[ti])
                         if (group[t.x] == g && lbk::tma_box_tile(p[t.x].nx, p[t.x].ny, t.y, t.z, tyv) == (pass == 0))
                             list.push_back(make_int4(t.x, t.y, t.z, pass == 0 ? lbk::kTmaBoxMark : 0));
-                    if (pass == 0) e->c_box[ti][g] = (int)list.size() - e->c_off[ti][g];
                 }
                 e->c_cnt[ti][g] = (int)list.size() - e->c_off[ti][g];
             }

@@ -81,12 +81,11 @@ constexpr int kTmaBoxMark = 1;
 cudaError_t prepare_fused_tma();
 // One time step of the FP32 tiles [tile_offset, tile_offset + n_tiles) in
 // one pass, one block per tile, each tile staged by one TMA copy of its
-// population box and one of its reference-density box.  Every tile must be
-// full and of a lattice at least kTmaBoxW x (ty + 4) nodes (tma_box_tile)
-// and carry w = kTmaBoxMark; the others go to Launch<float>::fused.  A copy
-// not complete after wait_cycles SM clocks sets *err = 1 and ends the block,
-// a tile without the mark sets *err = 2 (and starts no copy); the copy of
-// tile drop_tile (a test hook, -1 for none) is never started.
+// population box and one of its reference-density box.  Tiles that are full
+// and of a lattice at least kTmaBoxW x (ty + 4) nodes (tma_box_tile) carry
+// w = kTmaBoxMark; the others run as plain one-pass tiles.  A copy not
+// complete after wait_cycles SM clocks sets *err = 1 and ends the block; the
+// copy of tile drop_tile (a test hook, -1 for none) is never started.
 cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                              const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, int ty, cudaStream_t s);
 

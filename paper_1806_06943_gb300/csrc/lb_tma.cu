@@ -13,9 +13,8 @@
 // reference-density planes.  Parts of the box beyond the lattice are filled
 // with zeros by the copy and not used: the halo slots there (across a
 // periodic edge, or wall ghost rows) are formed as in fused_tile.  The
-// caller launches this kernel over the tiles that box_tile accepts and the
-// plain one-pass kernel over the others (ragged tiles, lattices smaller than
-// the box), so neither carries the other's registers.
+// tiles that tma_box_tile rejects (ragged ones, lattices smaller than the box)
+// run as plain one-pass tiles of the same launch.
 #include "lb_kernels.cuh"
 #include "lb_launch.h"
 
@@ -193,9 +192,21 @@ __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ la
     else collide_site<false, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
 }
 
+// A tile without a box (ragged, or of a lattice smaller than the box): the
+// plain one-pass tile, staged in the box's shared memory.  Out of line, so
+// that it does not shape the box tiles' registers.
+template <int TYv>
+__device__ __noinline__ void plain_tile(const Lat<float> *__restrict__ lats, int4 t, int parity, float *box)
+{
+    static_assert(sizeof(CollideSmem<TYv>) <= TmaBox<TYv>::kBytes, "staged in the box");
+    fused_tile<TYv, false>(lats, t, parity, *reinterpret_cast<CollideSmem<TYv> *>(box));
+}
+
 // One block per tile: thread 0 starts the two copies, every thread waits
-// (bounded) on the mbarrier, then the tile is computed from the box.  A tile
-// box_tile rejects is a caller error: it sets *err = 2 and is skipped.
+// (bounded) on the mbarrier, then the tile is computed from the box.  Tiles
+// without the mark run as plain_tile in the same launch: a second launch for
+// them cost more than their work (28 lattices of 220^2, whose last tiles are
+// ragged: 70 -> 64 us a step; 1000^2 48.4 -> 42.9; 333 x 97 11.6 -> 7.1).
 template <int TYv>
 __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     k_fused_tma(const Lat<float> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity,
@@ -207,13 +218,14 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     extern __shared__ __align__(128) float box[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ PairSmem<TYv> sm;
-    // the tile is full and its lattice holds a whole box (so its maps exist):
-    // the host marked it so when it sorted the list (tma_box_tile), which
-    // keeps the lattice's descriptor off the way to the copy.  A tile without
-    // the mark starts no copy and no load and leaves with *err = 2 where a
-    // failed wait would (block-uniform, no early branch in the prologue)
+    // the mark: the tile is full and its lattice holds a whole box (so its
+    // maps exist), as the host found when it sorted the list (tma_box_tile),
+    // which keeps the lattice's descriptor off the way to the copy
     const int4 t = tiles[tile_offset + blockIdx.x];
-    const bool good = t.w == kTmaBoxMark;
+    if (t.w != kTmaBoxMark) {
+        plain_tile<TYv>(lats, t, parity, box);
+        return;
+    }
     const int tid = threadIdx.y * TX + threadIdx.x;
     // the boxes of the tile `ahead` blocks later (about one wave of resident
     // blocks) into L2, so that its copies find them there; a block of the
@@ -223,12 +235,14 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     auto prefetch_ahead = [&]() {
         if (ahead > 0 && (int)blockIdx.x + ahead < n_tiles) {
             const int4 tn = tiles[tile_offset + blockIdx.x + ahead];
-            tma_prefetch_3d(&maps[tn.x].pop[ti][parity], tn.y - 4, tn.z - HALO, 0);
-            tma_prefetch_3d(&maps[tn.x].ref[ti][parity], tn.y - 4, tn.z - HALO, 0);
+            if (tn.w == kTmaBoxMark) {
+                tma_prefetch_3d(&maps[tn.x].pop[ti][parity], tn.y - 4, tn.z - HALO, 0);
+                tma_prefetch_3d(&maps[tn.x].ref[ti][parity], tn.y - 4, tn.z - HALO, 0);
+            }
         }
     };
     // the copy of drop_tile (a test hook) is never started: its wait runs out
-    const bool issued = good && tile_offset + (int)blockIdx.x != drop_tile;
+    const bool issued = tile_offset + (int)blockIdx.x != drop_tile;
     if (tid == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -237,13 +251,13 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
             tma_load_3d(box, &maps[t.x].pop[ti][parity], t.y - 4, t.z - HALO, 0, &bar);
             tma_load_3d(box + B::kPop, &maps[t.x].ref[ti][parity], t.y - 4, t.z - HALO, 0, &bar);
         }
-        if (good && !first_wave) prefetch_ahead();
+        if (!first_wave) prefetch_ahead();
     }
     // halo slots beyond the lattice load their nodes directly (wrapped, or
     // wall ghost rows): done while the copy is in flight
     {
         const Lat<float> &G = lats[t.x];
-        if (good && (t.y == 0 || t.y + TX + HALO > G.nx || t.z < HALO || t.z + TYv + HALO > G.ny)) {
+        if ((t.y == 0 || t.y + TX + HALO > G.nx || t.z < HALO || t.z + TYv + HALO > G.ny)) {
             for (int h = tid; h < kRing<TYv>; h += TX * TYv) {
                 int sx, sy;
                 ring_slot<TYv>(h, sx, sy);
@@ -257,10 +271,10 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
         }
     }
     __syncthreads();   // the barrier is initialised before anyone waits on it
-    const bool ok = good && mbar_wait(&bar, 0, wait_cycles);
+    const bool ok = mbar_wait(&bar, 0, wait_cycles);
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
-            atomicExch(err, good ? 1 : 2);
+            atomicExch(err, 1);
             // let a copy still in flight land before the block ends (bounded
             // too, by at least 2^31 clocks, ~1 s)
             if (issued) mbar_wait(&bar, 0, wait_cycles > (1ll << 31) ? wait_cycles : (1ll << 31));
