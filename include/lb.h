@@ -59,8 +59,11 @@ extern "C" {
 #define LB_WALLS_Y 1      /* half-way bounce-back walls at y = -1/2 and y = ny - 1/2, periodic in x */
 
 /* Execution modes of the time loop (lb_set_config, lb_batch_set_config).
- * LB_MODE_LAUNCH: each time step is a density-pass launch and a fused-kernel
- *   launch over the tiles of all lattices, replayed 32 steps per CUDA graph.
+ * LB_MODE_LAUNCH: each time step is launched by itself, replayed 32 steps per
+ *   CUDA graph: a density-pass launch and a fused-kernel launch over the tiles
+ *   of all lattices, or the one launch of the fastest one-pass form where that
+ *   takes less time (LB_FP32; LB_FP64 lattices of a few thousand nodes, in
+ *   LB_MODE_FUSED too).  lb_profile always times the two launches.
  * LB_MODE_PERSISTENT: one launch advances 64 time steps of all lattices; its
  *   blocks take (step, phase, tile) work items from an atomic queue and wait,
  *   with a bounded spin, only for the tiles of their own lattice that an item
@@ -77,7 +80,7 @@ extern "C" {
  *   reference-density planes), completed on an mbarrier; each block also
  *   prefetches into L2 the box of a tile about a wave of blocks later.  Halo
  *   nodes across a periodic edge or on wall ghost rows, ragged tiles and
- *   smaller lattices load as in LB_MODE_FUSED.  Same arithmetic as
+ *   smaller lattices load as in LB_MODE_FUSED, in the same launch.  Same arithmetic as
  *   LB_MODE_FUSED, same results.  A copy not complete within the wait limit
  *   (default 2 s) ends its block and the next synchronising call returns
  *   LB_ETIMEOUT. */

@@ -48,6 +48,11 @@ constexpr int kGraphSteps = 32;   // steps per captured graph (even: parity retu
 constexpr int kPersistSteps = 64; // time steps per persistent launch
 constexpr int kChains = 2;         // chains of time steps of a batch's step graph
 constexpr int kTileHeights[3] = {2, 4, 8};
+// Tiles of 32 x 8 nodes per SM from which an FP32 step of LB_MODE_LAUNCH is staged
+// by TMA: three waves of blocks.  Below, the plain one-pass kernel is as fast
+// (512^2, 1024 tiles: 13.7 us a step plain, 14.1 by TMA; 1000^2, 4000 tiles: 51.4
+// and 42.9).
+constexpr int kTmaTilesPerSm = 12;
 // rows of 32 nodes per SM up to which an FP64 step runs as k_small64
 constexpr int kSmallRowsPerSm = 3;
 
@@ -165,9 +170,13 @@ struct lb_engine {
     std::vector<int4> stiles[3];
     int4 *d_stiles[3] = {nullptr, nullptr, nullptr};
     int *d_sntiles[3] = {nullptr, nullptr, nullptr};
-    // execution configuration (autotuned or set by the caller)
+    // execution configuration (autotuned or set by the caller), and how a step
+    // that is launched by itself then runs (plan_step): its kernels and the
+    // tile list (index into kTileHeights)
     int mode = LB_MODE_LAUNCH;
     int ty = 4;
+    int smode = LB_MODE_LAUNCH;
+    int sti = 1;
     // persistent launches: control block (queue head + per-lattice counters),
     // sticky error word, blocks per SM per tile height, bounded-wait limit
     void *d_ctl = nullptr;
@@ -276,31 +285,45 @@ struct lb_engine {
             return lbk::Launch<double>::density((const lbk::Lat<double> *)d_lats, d_tiles, off, cnt, par, 4, stream);
         return lbk::Launch<float>::density((const lbk::Lat<float> *)d_lats, d_tiles, off, cnt, par, 4, stream);
     }
-    // one time step over the time-step tiles of height ty: two launches, or
-    // one in the fused mode
+    // The kernels of a step for the current configuration.  The two passes of
+    // LB_MODE_LAUNCH are slower than one in FP32 at every size (64^2 6.2 us a step
+    // and 5.2, 1024 x 256 14.9 and 13.0, 2048^2 222 and 139), and tiles of 32 x 8
+    // are the fastest for it; every choice gives the same bits.
+    void plan_step()
+    {
+        smode = mode;
+        sti = ty_index(ty);
+        if (precision == LB_FP32 && mode == LB_MODE_LAUNCH) {
+            sti = 2;
+            smode = tma_ok && (int64_t)stiles[sti].size() >= (int64_t)kTmaTilesPerSm * sm_count ? LB_MODE_TMA : LB_MODE_FUSED;
+        }
+    }
+    // one time step of all lattices: one launch, or two
     cudaError_t launch_step(int par)
     {
-        const int ti = ty_index(ty), nt = (int)stiles[ti].size();
+        const int ti = sti, nt = (int)stiles[ti].size(), h = kTileHeights[ti];
         cudaError_t e;
         if (precision == LB_FP64) {
             const lbk::Lat<double> *L = (const lbk::Lat<double> *)d_lats;
             if (n_rows) return lbk::Launch<double>::small(L, d_rows, 0, n_rows, par, stream);
-            if (mode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, d_stiles[ti], 0, nt, par, ty, stream);
-            e = lbk::Launch<double>::density(L, d_stiles[ti], 0, nt, par, ty, stream);
-            if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, d_stiles[ti], 0, nt, par, ty, stream);
+            if (smode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, d_stiles[ti], 0, nt, par, h, stream);
+            e = lbk::Launch<double>::density(L, d_stiles[ti], 0, nt, par, h, stream);
+            if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, d_stiles[ti], 0, nt, par, h, stream);
         } else {
             const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
-            if (mode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, par, ty, stream);
-            if (mode == LB_MODE_TMA) return launch_tma(L, ti, nt, par);
-            e = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, par, ty, stream);
-            if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, par, ty, stream);
+            if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, par, h, stream);
+            if (smode == LB_MODE_TMA) return launch_tma(L, d_btiles[ti], 0, nt, par, h, stream);
+            e = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, par, h, stream);
+            if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, par, h, stream);
         }
         return e;
     }
-    // LB_MODE_TMA step over all tiles, box tiles first
-    cudaError_t launch_tma(const lbk::Lat<float> *L, int ti, int nt, int par)
+    // TMA-staged step over a list of tiles, box tiles first (the test hook that
+    // drops a tile's copy belongs to LB_MODE_TMA)
+    cudaError_t launch_tma(const lbk::Lat<float> *L, const int4 *T, int off, int cnt, int par, int h, cudaStream_t s)
     {
-        return lbk::launch_fused_tma(L, d_btiles[ti], 0, nt, par, d_tmaps, d_err, wait_cycles, drop_tile, ty, stream);
+        return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, wait_cycles,
+                                     mode == LB_MODE_TMA ? drop_tile : -1, h, s);
     }
     size_t ctl_bytes() const { return 8 + 2 * sizeof(unsigned) * (size_t)n; }
     // nsteps time steps in one persistent launch (counters cleared first)
@@ -323,24 +346,23 @@ struct lb_engine {
     // one time step of the lattices of chain g on stream s
     cudaError_t launch_chain_step(int g, int par, cudaStream_t s)
     {
-        const int ti = ty_index(ty), off = c_off[ti][g], cnt = c_cnt[ti][g];
+        const int ti = sti, off = c_off[ti][g], cnt = c_cnt[ti][g], h = kTileHeights[ti];
         const int4 *T = d_ctiles[ti];
         if (cnt == 0) return cudaSuccess;
         cudaError_t e;
         if (precision == LB_FP64) {
             const lbk::Lat<double> *L = (const lbk::Lat<double> *)d_lats;
             if (n_rows) return lbk::Launch<double>::small(L, d_rows, r_off[g], r_cnt[g], par, s);
-            if (mode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, T, off, cnt, par, ty, s);
-            e = lbk::Launch<double>::density(L, T, off, cnt, par, ty, s);
-            if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, T, off, cnt, par, ty, s);
+            if (smode == LB_MODE_FUSED) return lbk::Launch<double>::fused(L, T, off, cnt, par, h, s);
+            e = lbk::Launch<double>::density(L, T, off, cnt, par, h, s);
+            if (e == cudaSuccess) e = lbk::Launch<double>::collide(L, T, off, cnt, par, h, s);
             return e;
         }
         const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
-        if (mode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, T, off, cnt, par, ty, s);
-        if (mode == LB_MODE_TMA)
-            return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, wait_cycles, drop_tile, ty, s);
-        e = lbk::Launch<float>::density(L, T, off, cnt, par, ty, s);
-        if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, T, off, cnt, par, ty, s);
+        if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, T, off, cnt, par, h, s);
+        if (smode == LB_MODE_TMA) return launch_tma(L, T, off, cnt, par, h, s);
+        e = lbk::Launch<float>::density(L, T, off, cnt, par, h, s);
+        if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, T, off, cnt, par, h, s);
         return e;
     }
     // time steps in the current mode, as captured into one graph: with
@@ -581,6 +603,7 @@ struct lb_engine {
         if (m != mode || tyv != ty) drop_graph();
         mode = m;
         ty = tyv;
+        plan_step();
         return LB_OK;
     }
 
@@ -618,7 +641,7 @@ struct lb_engine {
                 if (ce == cudaSuccess && !one) ce = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, parity, ty, stream);
                 if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], stream);
                 if (ce == cudaSuccess)
-                    ce = mode == LB_MODE_TMA ? launch_tma(L, ti, nt, parity)
+                    ce = mode == LB_MODE_TMA ? launch_tma(L, d_btiles[ti], 0, nt, parity, ty, stream)
                          : one ? lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, parity, ty, stream)
                                : lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, parity, ty, stream);
             }
@@ -1329,6 +1352,7 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
         chain_of = group;
     }
     if ((rc = e->build_rows(chain_of))) return bail(rc);
+    e->plan_step();
     *out = e;
     return LB_OK;
 }
