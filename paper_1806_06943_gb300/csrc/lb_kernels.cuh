@@ -51,9 +51,8 @@ constexpr bool kOffset = sizeof(real) == 4;
 
 // Resident blocks per SM the fused kernel is compiled for: the FP32 kernel is
 // bound by HBM and needs the warps to keep enough loads in flight; the FP64
-// kernel is bound by the FP64 pipe, which 16 warps fill (8 warps without a
-// spill and 24 with 540 bytes of it measured 5 % and 1 % slower on a 1024^2
-// lattice).
+// kernel is bound by the FP64 pipe, which 16 warps fill (24 with 550 bytes of
+// spill measured 7 % slower on a 1024^2 lattice).
 template <typename real, int TYv>
 constexpr int kCollideMinBlocks = (kOffset<real> ? 32 : 16) / TYv;
 
@@ -746,46 +745,33 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
         outside = velocity_outside(ux) | velocity_outside(uy);
     }
     const Dirs64<kInt> dirs(A, ux, uy);
-    double g[9][2], po[9];
-    dirs.template terms<0>(A, g[0], po[0]);
-    dirs.template terms<1>(A, g[1], po[1]);
-    dirs.template terms<2>(A, g[2], po[2]);
-    dirs.template terms<3>(A, g[3], po[3]);
-    dirs.template terms<4>(A, g[4], po[4]);
-    dirs.template terms<5>(A, g[5], po[5]);
-    dirs.template terms<6>(A, g[6], po[6]);
-    dirs.template terms<7>(A, g[7], po[7]);
-    dirs.template terms<8>(A, g[8], po[8]);
     const Push64 push(L, x, y);
-#pragma unroll 1
-    for (int k = 0; k < 2; ++k) {
-        const double *__restrict__ fk = fc + (size_t)(k * 9) * plane;
-        double *__restrict__ nk = fn + (size_t)(k * 9) * plane;
-        const double r = k ? r1 : r0, om = k ? om1 : om0;
-        const double Fx = k ? F[1][0] : F[0][0], Fy = k ? F[1][1] : F[0][1];
-        double f[9];
+    const double wr[2][3] = {{A.mul(4.0 / 9.0, r0), A.mul(1.0 / 9.0, r0), A.mul(1.0 / 36.0, r0)},
+                             {A.mul(4.0 / 9.0, r1), A.mul(1.0 / 9.0, r1), A.mul(1.0 / 36.0, r1)}};
+    // a direction of both species at once: its terms live no longer than it
+    // does, and its populations are read again where they are used
+    auto dir = [&](auto Ic) {
+        constexpr int I = decltype(Ic)::value, c = cls9(I);
+        double g[2], po;
+        dirs.template terms<I>(A, g, po);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = ldg_state<kCG>(&fk[(size_t)i * plane]);
-        if constexpr (kInt) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) outside |= base_outside(f[i]);
+        for (int k = 0; k < 2; ++k) {
+            const double f = ldg_state<kCG>(&fc[(size_t)(k * 9 + I) * plane]);
+            if constexpr (kInt) outside |= base_outside(f);
+            push.store<I>(fn + (size_t)(k * 9) * plane, plane,
+                          relax64<I>(A, f, wr[k][c], k ? om1 : om0, L.aw[k][c], g, po, F[k][0], F[k][1]));
         }
-        const double wr[3] = {A.mul(4.0 / 9.0, r), A.mul(1.0 / 9.0, r), A.mul(1.0 / 36.0, r)};
-        const double aw[3] = {L.aw[k][0], L.aw[k][1], L.aw[k][2]};
-        auto dir = [&](auto Ic) {
-            constexpr int I = decltype(Ic)::value, c = cls9(I);
-            push.store<I>(nk, plane, relax64<I>(A, f[I], wr[c], om, aw[c], g[I], po[I], Fx, Fy));
-        };
-        dir(std::integral_constant<int, 0>{});
-        dir(std::integral_constant<int, 1>{});
-        dir(std::integral_constant<int, 2>{});
-        dir(std::integral_constant<int, 3>{});
-        dir(std::integral_constant<int, 4>{});
-        dir(std::integral_constant<int, 5>{});
-        dir(std::integral_constant<int, 6>{});
-        dir(std::integral_constant<int, 7>{});
-        dir(std::integral_constant<int, 8>{});
-    }
+    };
+    // opposite directions in turn: they share the products with e.u
+    dir(std::integral_constant<int, 0>{});
+    dir(std::integral_constant<int, 1>{});
+    dir(std::integral_constant<int, 3>{});
+    dir(std::integral_constant<int, 2>{});
+    dir(std::integral_constant<int, 4>{});
+    dir(std::integral_constant<int, 5>{});
+    dir(std::integral_constant<int, 7>{});
+    dir(std::integral_constant<int, 6>{});
+    dir(std::integral_constant<int, 8>{});
     return outside != 0;
 }
 
