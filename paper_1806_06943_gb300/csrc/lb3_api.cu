@@ -170,7 +170,7 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
     const size_t total = 2 * fbytes + 2 * rbytes;
     h->n_tiles = h->L64.tiles_x * h->L64.tiles_y * h->L64.tiles_z;
     if (cudaMalloc(&h->pool, total) != cudaSuccess ||
-        cudaMalloc((void **)&h->partials, (size_t)h->n_tiles * lbk3::kNumAcc * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void **)&h->partials, ((size_t)h->n_tiles + lbk3::kFold3) * lbk3::kNumAcc * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void **)&h->obs, lbk3::kNumAcc * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail3(LB_ENOMEM, "lb3: cudaMalloc of the lattice state failed"));
@@ -259,7 +259,7 @@ int lb3_observables(lb3_handle *h, lb3_obs *o)
         o->mom[0][a] = s[2 + a];
         o->mom[1][a] = s[5 + a];
     }
-    o->umax = s[8];
+    o->umax = std::sqrt(s[8]);
     o->finite = s[9] == 0.0 ? 1 : 0;
     const double nan = std::nan("");
     if (h->L64.has_probe && s[12] > 0.0 && s[15] > 0.0) {

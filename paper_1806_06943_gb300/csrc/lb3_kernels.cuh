@@ -121,10 +121,15 @@ struct Stage3 {
 };
 static_assert(sizeof(Stage3<float>) % 16 == 0 && sizeof(Stage3<double>) % 16 == 0, "partials stay aligned");
 
+// rows of per-thread values for the observation sums, in the stage's place
+constexpr int kSumRun3 = 16, kSumRow3 = kThreads + kThreads / kSumRun3;
+static_assert(kThreads == kNumAcc * kSumRun3, "a thread sums one run of one row");
+constexpr size_t kSumBytes3 = (size_t)kNumAcc * kSumRow3 * sizeof(double);
+
 template <typename real>
 constexpr size_t kCollideSmem3 = sizeof(Stage3<real>);
 template <typename real>
-constexpr size_t kObserveSmem3 = sizeof(Stage3<real>) + (kThreads / 32) * kNumAcc * sizeof(double);
+constexpr size_t kObserveSmem3 = sizeof(Stage3<real>) > kSumBytes3 ? sizeof(Stage3<real>) : kSumBytes3;
 
 // rho and psi of the tile (x0, y0, z0) and its 2-node halo from density copy
 // `rho` (periodic copies across every face).
@@ -677,7 +682,7 @@ __global__ void __launch_bounds__(kThreads) k3_observe(const Lat3<real> L, int p
                                                        double *__restrict__ out_rho, double *__restrict__ out_u)
 {
     Stage3<real> &sm = *reinterpret_cast<Stage3<real> *>(lb3_smem);
-    double(*sacc)[kNumAcc] = reinterpret_cast<double(*)[kNumAcc]>(lb3_smem + sizeof(Stage3<real>));
+    double(*sacc)[kSumRow3] = reinterpret_cast<double(*)[kSumRow3]>(lb3_smem);
     int x0, y0, z0;
     tile_origin(L.tiles_x, L.tiles_y, blockIdx.x, x0, y0, z0);
     const int tid = (threadIdx.z * TY + threadIdx.y) * TX + threadIdx.x;
@@ -723,7 +728,7 @@ __global__ void __launch_bounds__(kThreads) k3_observe(const Lat3<real> L, int p
             acc[2 + a] = m[0][a];
             acc[5 + a] = m[1][a];
         }
-        acc[8] = sqrt(u2);
+        acc[8] = u2;   // the square root is taken of the largest
         acc[9] = fin ? 0.0 : 1.0;
         if (L.has_probe) {
             const int Ls[3] = {L.nx, L.ny, L.nz};
@@ -753,56 +758,47 @@ __global__ void __launch_bounds__(kThreads) k3_observe(const Lat3<real> L, int p
         }
     }
     if (!partials) return;
-    const int warp = tid >> 5, lane = tid & 31;
+    // through shared memory, 16 values a thread (as the 2-D observables)
+    __syncthreads();   // the stage has been read
 #pragma unroll
-    for (int a = 0; a < kNumAcc; ++a) {
-        double v = acc[a];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double w = __shfl_xor_sync(0xffffffffu, v, o);
-            v = a == 8 ? fmax(v, w) : v + w;
-        }
-        if (lane == 0) sacc[warp][a] = v;
-    }
+    for (int a = 0; a < kNumAcc; ++a) sacc[a][tid + tid / kSumRun3] = acc[a];
     __syncthreads();
-    if (tid < kNumAcc) {
-        double v = sacc[0][tid];
-        for (int w = 1; w < kThreads / 32; ++w) v = tid == 8 ? fmax(v, sacc[w][tid]) : v + sacc[w][tid];
-        partials[(size_t)blockIdx.x * kNumAcc + tid] = v;
+    const int a = tid / kSumRun3, l = tid % kSumRun3;
+    double v = sacc[a][l * (kSumRun3 + 1)];
+#pragma unroll
+    for (int q = 1; q < kSumRun3; ++q) {
+        const double w = sacc[a][l * (kSumRun3 + 1) + q];
+        v = a == 8 ? fmax(v, w) : v + w;
     }
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const double w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = a == 8 ? fmax(v, w) : v + w;
+    }
+    if (l == 0) partials[(size_t)blockIdx.x * kNumAcc + a] = v;
 }
 
-// one block: the tile partials summed (max for |u|) in a fixed order
-static __global__ void __launch_bounds__(256) k3_reduce(const double *__restrict__ partials, int n_tiles,
-                                                 double *__restrict__ out)
+// Block b: the b-th of gridDim.x runs of the records, summed (max for |u|^2)
+// in a fixed order into out[b].
+static __global__ void __launch_bounds__(256) k3_reduce(const double *__restrict__ partials, int n_rec,
+                                                        double *__restrict__ out)
 {
-    __shared__ double sred[256 / 32][kNumAcc];
-    const int tid = threadIdx.x;
-    double acc[kNumAcc];
-#pragma unroll
-    for (int a = 0; a < kNumAcc; ++a) acc[a] = 0.0;
-    for (int t = tid; t < n_tiles; t += 256)
-#pragma unroll
-        for (int a = 0; a < kNumAcc; ++a) {
-            const double v = partials[(size_t)t * kNumAcc + a];
-            acc[a] = a == 8 ? fmax(acc[a], v) : acc[a] + v;
-        }
-    const int warp = tid >> 5, lane = tid & 31;
-#pragma unroll
-    for (int a = 0; a < kNumAcc; ++a) {
-        double v = acc[a];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double w = __shfl_xor_sync(0xffffffffu, v, o);
-            v = a == 8 ? fmax(v, w) : v + w;
-        }
-        if (lane == 0) sred[warp][a] = v;
+    __shared__ double s[256 / 32][kNumAcc];
+    const int run = (n_rec + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * run, t1 = min(t0 + run, n_rec);
+    const int a = threadIdx.x % kNumAcc;   // 16 threads a record
+    double v = 0.0;
+    for (int t = t0 + threadIdx.x / kNumAcc; t < t1; t += 256 / kNumAcc) {
+        const double w = partials[(size_t)t * kNumAcc + a];
+        v = a == 8 ? fmax(v, w) : v + w;
     }
+    const double w = __shfl_xor_sync(0xffffffffu, v, 16);
+    v = a == 8 ? fmax(v, w) : v + w;
+    if (threadIdx.x % 32 < kNumAcc) s[threadIdx.x / 32][a] = v;
     __syncthreads();
-    if (tid < kNumAcc) {
-        double v = sred[0][tid];
-        for (int w = 1; w < 8; ++w) v = tid == 8 ? fmax(v, sred[w][tid]) : v + sred[w][tid];
-        out[tid] = v;
+    if (threadIdx.x < kNumAcc) {
+        v = s[0][a];
+        for (int q = 1; q < 256 / 32; ++q) v = a == 8 ? fmax(v, s[q][a]) : v + s[q][a];
+        out[(size_t)blockIdx.x * kNumAcc + a] = v;
     }
 }
 

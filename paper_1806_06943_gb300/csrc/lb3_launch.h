@@ -20,7 +20,10 @@ struct Launch3 {
     static cudaError_t get_pops(const Lat3<real> &L, int parity, double *out, cudaStream_t s);
 };
 
-cudaError_t reduce3(const double *partials, int n_tiles, double *out, cudaStream_t s);
+// The tile partials' sums into out; partials has room for kFold3 records
+// behind the n_tiles.
+constexpr int kFold3 = 64;
+cudaError_t reduce3(double *partials, int n_tiles, double *out, cudaStream_t s);
 
 extern template struct Launch3<double>;
 extern template struct Launch3<float>;

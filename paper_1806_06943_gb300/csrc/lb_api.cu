@@ -200,6 +200,7 @@ struct lb_engine {
     bool tma_ok = false;
     std::string tma_why = "LB_MODE_TMA needs LB_FP32 populations";
     double *d_partials = nullptr;
+    double *d_fold = nullptr;         // kFold records per lattice, where one has more than kFoldTiles tiles
     double *d_obs = nullptr;
     double *d_psum = nullptr;         // pressure-tensor sums, kPStride doubles per lattice
     double *d_tmp = nullptr;
@@ -237,6 +238,7 @@ struct lb_engine {
         cudaFree(d_pool);
         cudaFree(d_tmaps);
         cudaFree(d_partials);
+        cudaFree(d_fold);
         cudaFree(d_obs);
         cudaFree(d_psum);
         cudaFree(d_tmp);
@@ -530,8 +532,8 @@ struct lb_engine {
     cudaError_t launch_finalize()
     {
         if (precision == LB_FP64)
-            return lbk::Launch<double>::finalize((const lbk::Lat<double> *)d_lats, n, d_partials, d_obs, stream);
-        return lbk::Launch<float>::finalize((const lbk::Lat<float> *)d_lats, n, d_partials, d_obs, stream);
+            return lbk::Launch<double>::finalize((const lbk::Lat<double> *)d_lats, n, d_partials, d_fold, d_obs, stream);
+        return lbk::Launch<float>::finalize((const lbk::Lat<float> *)d_lats, n, d_partials, d_fold, d_obs, stream);
     }
 
     int ensure_tmp(size_t elems)
@@ -1254,6 +1256,12 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
         cudaGetLastError();
         return bail(fail(LB_ENOMEM, "cudaMalloc of the descriptors failed"));
     }
+    for (int l = 0; l < n; ++l)
+        if (e->tile_end(l) - e->tile_begin(l) > lbk::kFoldTiles && !e->d_fold &&
+            cudaMalloc((void **)&e->d_fold, (size_t)n * lbk::kFold * lbk::kAccStride * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(fail(LB_ENOMEM, "cudaMalloc of the folded partials failed"));
+        }
     // time-step tiles for every supported tile height, and the persistent
     // launch's control block and error word
     if ((ce = e->precision == LB_FP64 ? lbk::Launch<double>::prepare() : lbk::Launch<float>::prepare()) != cudaSuccess)

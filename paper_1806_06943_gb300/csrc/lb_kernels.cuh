@@ -1377,10 +1377,18 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
+// Sums over a block of kThreads threads: every thread leaves its values in
+// rows of shared memory; kSumLanes threads a row then add kSumRun values each
+// (rows padded so that their accesses spread over the banks) and shuffle.
+constexpr int kSumRun = 16, kSumLanes = kThreads / kSumRun, kSumRow = kThreads + kSumLanes;
+__device__ __forceinline__ int sum_slot(int t) { return t + t / kSumRun; }
+
 // Per-node diagnostics (densities, momenta with half force, barycentric
 // velocity, Eq. 11 bulk pressure) reduced per tile into FP64 partial sums;
 // optionally also written as dense FP64 fields [..][ny][nx].  Reads the
-// density copy parity^1 written by a density pass at the same time.
+// density copy parity^1 written by a density pass at the same time.  The sums
+// of a tile go through shared memory, 16 values a thread: shuffles within the
+// warps took 75 FP64 additions a node (slot kUmax: the largest |u|^2).
 template <typename real>
 __global__ void __launch_bounds__(kThreads) k_observe(const Lat<real> *__restrict__ lats, const int4 *__restrict__ tiles,
                                                       int tile_offset, int parity, double *__restrict__ partials,
@@ -1389,7 +1397,7 @@ __global__ void __launch_bounds__(kThreads) k_observe(const Lat<real> *__restric
 {
     __shared__ real srho[2][SH][SW];
     __shared__ real spsi[2][SH][SW];
-    __shared__ double sacc[kThreads / 32][kAccStride];
+    __shared__ double sacc[kNumAcc][kSumRow];
     const int4 t = tiles[tile_offset + blockIdx.x];
     const Lat<real> &L = lats[t.x];
     const int tid = threadIdx.y * TX + threadIdx.x;
@@ -1425,7 +1433,7 @@ __global__ void __launch_bounds__(kThreads) k_observe(const Lat<real> *__restric
         acc[kMomBx] = m[1][0];
         acc[kMomBy] = m[1][1];
         acc[kSumUx] = ux;
-        acc[kUmax] = sqrt(ux * ux + uy * uy);
+        acc[kUmax] = ux * ux + uy * uy;
         acc[kNonFinite] = (isfinite(r[0]) && isfinite(r[1]) && isfinite(ux) && isfinite(uy)) ? 0.0 : 1.0;
         if (L.has_probe) {
             double dx = fabs((double)x - L.probe[0]), dy = fabs((double)y - L.probe[1]);
@@ -1456,17 +1464,57 @@ __global__ void __launch_bounds__(kThreads) k_observe(const Lat<real> *__restric
         }
     }
     if (!partials) return;
-    const int warp = tid >> 5, lane = tid & 31;
 #pragma unroll
-    for (int a = 0; a < kNumAcc; ++a) {
-        const double v = (a == kUmax) ? warp_max(acc[a]) : warp_sum(acc[a]);
-        if (lane == 0) sacc[warp][a] = v;
-    }
+    for (int a = 0; a < kNumAcc; ++a) sacc[a][sum_slot(tid)] = acc[a];
     __syncthreads();
-    if (tid < kNumAcc) {
-        double v = sacc[0][tid];
-        for (int w = 1; w < kThreads / 32; ++w) v = (tid == kUmax) ? fmax(v, sacc[w][tid]) : v + sacc[w][tid];
-        partials[(size_t)(tile_offset + blockIdx.x) * kAccStride + tid] = v;
+    const int a = tid / kSumLanes, l = tid % kSumLanes;
+    const bool on = a < kNumAcc;
+    double v = on ? sacc[a][sum_slot(kSumRun * l)] : 0.0;
+#pragma unroll
+    for (int q = 1; q < kSumRun; ++q) {
+        const double w = on ? sacc[a][sum_slot(kSumRun * l + q)] : 0.0;
+        v = a == kUmax ? fmax(v, w) : v + w;
+    }
+#pragma unroll
+    for (int o = 1; o < kSumLanes; o <<= 1) {
+        const double w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = a == kUmax ? fmax(v, w) : v + w;
+    }
+    if (on && l == 0) partials[(size_t)(tile_offset + blockIdx.x) * kAccStride + a] = v;
+}
+
+// Lattices of more tiles than this have their partials folded into kFold
+// records by as many blocks before k_finalize, whose one block took 5 ms of a
+// 4096^2 lattice's observables.
+constexpr int kFoldTiles = 2048, kFold = 64;
+
+// Block (b, lattice): the b-th of kFold runs of the lattice's tile partials,
+// in a fixed order.
+template <typename real>
+__global__ void __launch_bounds__(256) k_fold(const Lat<real> *__restrict__ lats, const double *__restrict__ partials,
+                                              double *__restrict__ fold)
+{
+    __shared__ double s[256 / 32][kAccStride];
+    const Lat<real> &L = lats[blockIdx.y];
+    const int nt = L.tile_end - L.tile_begin;
+    if (nt <= kFoldTiles) return;
+    const int run = (nt + kFold - 1) / kFold, t0 = L.tile_begin + blockIdx.x * run, t1 = min(t0 + run, L.tile_end);
+    // 16 threads a tile record, 16 records at a time
+    const int a = threadIdx.x % kAccStride, r = threadIdx.x / kAccStride;
+    double v = 0.0;
+    if (a < kNumAcc)
+        for (int t = t0 + r; t < t1; t += 256 / kAccStride) {
+            const double w = partials[(size_t)t * kAccStride + a];
+            v = a == kUmax ? fmax(v, w) : v + w;
+        }
+    const double w = __shfl_xor_sync(0xffffffffu, v, 16);
+    v = a == kUmax ? fmax(v, w) : v + w;
+    if (threadIdx.x % 32 < kAccStride) s[threadIdx.x / 32][a] = v;
+    __syncthreads();
+    if (threadIdx.x < kNumAcc) {
+        v = s[0][a];
+        for (int q = 1; q < 256 / 32; ++q) v = a == kUmax ? fmax(v, s[q][a]) : v + s[q][a];
+        fold[((size_t)blockIdx.y * kFold + blockIdx.x) * kAccStride + a] = v;
     }
 }
 
@@ -1474,7 +1522,7 @@ __global__ void __launch_bounds__(kThreads) k_observe(const Lat<real> *__restric
 // derive the observables.
 template <typename real>
 __global__ void __launch_bounds__(256) k_finalize(const Lat<real> *__restrict__ lats, const double *__restrict__ partials,
-                                                  double *__restrict__ obs)
+                                                  const double *__restrict__ fold, double *__restrict__ obs)
 {
     __shared__ double sred[256 / 32][kAccStride];
     const Lat<real> &L = lats[blockIdx.x];
@@ -1482,10 +1530,14 @@ __global__ void __launch_bounds__(256) k_finalize(const Lat<real> *__restrict__ 
     double acc[kNumAcc];
 #pragma unroll
     for (int a = 0; a < kNumAcc; ++a) acc[a] = 0.0;
-    for (int tl = L.tile_begin + tid; tl < L.tile_end; tl += 256) {
+    const bool folded = L.tile_end - L.tile_begin > kFoldTiles;
+    const double *__restrict__ rec = folded ? fold + (size_t)blockIdx.x * kFold * kAccStride
+                                            : partials + (size_t)L.tile_begin * kAccStride;
+    const int nrec = folded ? kFold : L.tile_end - L.tile_begin;
+    for (int tl = tid; tl < nrec; tl += 256) {
 #pragma unroll
         for (int a = 0; a < kNumAcc; ++a) {
-            const double v = partials[(size_t)tl * kAccStride + a];
+            const double v = rec[(size_t)tl * kAccStride + a];
             acc[a] = (a == kUmax) ? fmax(acc[a], v) : acc[a] + v;
         }
     }
@@ -1526,7 +1578,7 @@ __global__ void __launch_bounds__(256) k_finalize(const Lat<real> *__restrict__ 
         o[oDp] = __longlong_as_double(0x7ff8000000000000ll);
         o[oReff] = __longlong_as_double(0x7ff8000000000000ll);
     }
-    o[oUmax] = s[kUmax];
+    o[oUmax] = sqrt(s[kUmax]);
     o[oFinite] = s[kNonFinite] == 0.0 ? 1.0 : 0.0;
 }
 

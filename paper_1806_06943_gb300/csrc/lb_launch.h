@@ -39,7 +39,11 @@ struct Launch {
     static int persistent_blocks_per_sm(int ty);
     static cudaError_t observe(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                                double *partials, double *rho, double *mom, double *ubar, cudaStream_t s);
-    static cudaError_t finalize(const Lat<real> *lats, int n_lat, const double *partials, double *obs, cudaStream_t s);
+    // the tile partials of n_lat lattices into their observables; fold: kFold
+    // records per lattice of scratch, NULL where no lattice has more than
+    // kFoldTiles tiles
+    static cudaError_t finalize(const Lat<real> *lats, int n_lat, const double *partials, double *fold, double *obs,
+                                cudaStream_t s);
     // pressure tensor per node of tiles [tile_offset, tile_offset + n_tiles)
     // of height 4 (partials: 8 doubles per tile; out: dense [6][ny][nx] of
     // one lattice, or NULL), and its per-lattice sums (8 doubles per lattice)

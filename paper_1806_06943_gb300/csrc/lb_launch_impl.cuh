@@ -138,10 +138,16 @@ cudaError_t Launch<real>::observe(const Lat<real> *lats, const int4 *tiles, int 
 }
 
 template <typename real>
-cudaError_t Launch<real>::finalize(const Lat<real> *lats, int n_lat, const double *partials, double *obs, cudaStream_t s)
+cudaError_t Launch<real>::finalize(const Lat<real> *lats, int n_lat, const double *partials, double *fold, double *obs,
+                                   cudaStream_t s)
 {
     if (n_lat <= 0) return cudaSuccess;
-    k_finalize<real><<<n_lat, 256, 0, s>>>(lats, partials, obs);
+    if (fold) {
+        k_fold<real><<<dim3(kFold, n_lat), 256, 0, s>>>(lats, partials, fold);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    k_finalize<real><<<n_lat, 256, 0, s>>>(lats, partials, fold, obs);
     return cudaGetLastError();
 }
 
