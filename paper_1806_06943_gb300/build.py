@@ -35,6 +35,7 @@ UNITS = {
     "lb_noalloc.cu": ["-fmad=false"],
     "lb_adjoint.cu": [],
     "lb_device.cu": [],
+    "lb_tables.cu": [],
     "lb3_api.cu": [],
     "lb3_fp64.cu": ["-fmad=false"],
     "lb3_fp32.cu": [],

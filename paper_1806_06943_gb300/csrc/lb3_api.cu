@@ -70,6 +70,7 @@ struct lb3_handle {
     lbk3::Lat3<double> L64;
     lbk3::Lat3<float> L32;
     void *pool = nullptr;
+    double2 *exp_table = nullptr;
     double *partials = nullptr, *obs = nullptr, *tmp = nullptr;
     size_t tmp_elems = 0;
     int n_tiles = 0;
@@ -81,6 +82,7 @@ struct lb3_handle {
     {
         if (stream) cudaStreamSynchronize(stream);
         cudaFree(pool);
+        cudaFree(exp_table);
         cudaFree(partials);
         cudaFree(obs);
         cudaFree(tmp);
@@ -178,6 +180,11 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
     if (cudaMemsetAsync(h->pool, 0, total, h->stream) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail3(LB_ECUDA, "cudaMemsetAsync failed"));
+    }
+    if (h->f64()) {
+        const cudaError_t e = lbk::make_exp_table(&h->exp_table, h->stream);
+        if (e != cudaSuccess) return bail(cuda_fail3(e, "exp table"));
+        h->L64.exp_table = h->exp_table;
     }
     char *b = (char *)h->pool;
     void *f0 = b, *f1 = b + fbytes, *r0 = b + 2 * fbytes, *r1 = b + 2 * fbytes + rbytes;

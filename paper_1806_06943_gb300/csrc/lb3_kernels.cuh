@@ -88,6 +88,7 @@ struct Lat3 {
     int32_t tiles_x, tiles_y, tiles_z, has_probe;
     real omega[2];       // 1 / tau_k
     real aw3[2][3];      // 3 (1 - omega_k / 2) w(|e|^2) for |e|^2 = 0, 1, 2
+    const double2 *exp_table;   // exp(-j/512) for the FP64 density pass (lb_f64.cuh)
     real cw[9];          // -(G1 w + G2 q) for |e|^2 = 0 .. 8 (FP32: the two psi sums of Eq. 8 as one)
     real G1, G2, GAB;
     real g[3];
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int p
         L.rho[parity ^ 1][(size_t)k * L.plane + c] = r;
         // FP64 keeps no reference densities: copy parity holds psi for the
         // collide kernel, so that exp() runs once per node
-        if constexpr (!kOffset3<real>) L.rho[parity][(size_t)k * L.plane + c] = psi3<real>(r);
+        if constexpr (!kOffset3<real>) L.rho[parity][(size_t)k * L.plane + c] = lbk::psi64(r, lbk::opaque_one(), L.exp_table);
     }
 }
 

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_adj_local(const Lat<double> L, 
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             srho[k][sy][sx] = fixed ? L.wall_rho[k] : rho[(size_t)k * L.plane + c];
-            spsi[k][sy][sx] = fixed ? psi_of<double>(L.wall_rho[k]) : A.sub(1.0, rho[(size_t)(2 + k) * L.plane + c]);
+            spsi[k][sy][sx] = fixed ? psi64(L.wall_rho[k], A.one, L.exp_table) : A.sub(1.0, rho[(size_t)(2 + k) * L.plane + c]);
         }
     }
     __syncthreads();
@@ -371,7 +371,7 @@ __global__ void k_adj_density(const Lat<double> L, const double *__restrict__ f,
         for (int i = 0; i < 9; ++i) v[i] = f[(size_t)(k * 9 + i) * L.plane + c];
         const double r = zeroth_moment<double>(v, one);
         rho[(size_t)k * L.plane + c] = r;
-        rho[(size_t)(2 + k) * L.plane + c] = exp(-r);
+        rho[(size_t)(2 + k) * L.plane + c] = exp_minus(r, one, L.exp_table);
     }
 }
 

@@ -199,6 +199,7 @@ struct lb_engine {
     int r_off[kChains] = {}, r_cnt[kChains] = {};
     bool tma_ok = false;
     std::string tma_why = "LB_MODE_TMA needs LB_FP32 populations";
+    double2 *d_exp = nullptr;         // table of the FP64 kernels (also the adjoint of FP32 lattices)
     double *d_partials = nullptr;
     double *d_fold = nullptr;         // kFold records per lattice, where one has more than kFoldTiles tiles
     double *d_obs = nullptr;
@@ -238,6 +239,7 @@ struct lb_engine {
         cudaFree(d_pool);
         cudaFree(d_tmaps);
         cudaFree(d_partials);
+        cudaFree(d_exp);
         cudaFree(d_fold);
         cudaFree(d_obs);
         cudaFree(d_psum);
@@ -800,6 +802,7 @@ struct lb_engine {
             L = L64[0];
         } else {
             fill_lat(L, p);
+            L.exp_table = d_exp;
             L.pitch = L32[0].pitch;
             L.plane = L32[0].plane;
             L.has_probe = L32[0].has_probe;
@@ -1218,6 +1221,7 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
     }
     if ((ce = cudaMemsetAsync(e->d_pool, 0, total, e->stream)) != cudaSuccess) return bail(cuda_fail(ce, "cudaMemsetAsync"));
 
+    if ((ce = lbk::make_exp_table(&e->d_exp, e->stream)) != cudaSuccess) return bail(cuda_fail(ce, "exp table"));
     // tiles in raster order, lattice by lattice
     for (int l = 0; l < n; ++l) {
         const int begin = (int)e->tiles.size();
@@ -1232,6 +1236,7 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
             L.f[1] = (double *)(base + off_f1[l]);
             L.rho[0] = (double *)(base + off_r0[l]);
             L.rho[1] = (double *)(base + off_r1[l]);
+            L.exp_table = e->d_exp;
             L.tile_begin = begin;
             L.tile_end = end;
             e->L64.push_back(L);

@@ -330,7 +330,7 @@ __device__ __forceinline__ void density_tile(const Lat<real> *__restrict__ lats,
         L.rho[parity ^ 1][(size_t)k * L.plane + c] = r;
         // FP64 keeps no reference densities: copy parity holds psi, so that
         // exp() runs once per node instead of once per staged slot
-        if constexpr (!kOffset<real>) L.rho[parity][(size_t)k * L.plane + c] = psi_of<real>(r);
+        if constexpr (!kOffset<real>) L.rho[parity][(size_t)k * L.plane + c] = psi64(r, L.one, L.exp_table);
     }
 }
 
@@ -739,8 +739,17 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
     const double r0 = sm.v[0][sRho][cy][cx], r1 = sm.v[1][sRho][cy][cx];
     const double om0 = L.omega[0], om1 = L.omega[1];
     const double den = A.add(A.mul(om0, r0), A.mul(om1, r1));
-    const double ux = A.add(A.mul(om0, m[0][0]), A.mul(om1, m[1][0])) / den;
-    const double uy = A.add(A.mul(om0, m[0][1]), A.mul(om1, m[1][1])) / den;
+    const double nx = A.add(A.mul(om0, m[0][0]), A.mul(om1, m[1][0]));
+    const double ny = A.add(A.mul(om0, m[0][1]), A.mul(om1, m[1][1]));
+    double ux, uy;
+    if constexpr (kInt) {
+        const double rden = reciprocal64(den, A.one);
+        ux = quotient64(nx, den, rden);
+        uy = quotient64(ny, den, rden);
+    } else {
+        ux = nx / den;
+        uy = ny / den;
+    }
     if constexpr (kInt) {
         outside = velocity_outside(ux) | velocity_outside(uy);
     }
@@ -1051,7 +1060,7 @@ __device__ __forceinline__ void collide_tile64(const Lat<double> *__restrict__ l
 #pragma unroll 1
         for (int k = 0; k < 2; ++k) {
             const double r = fixed ? G.wall_rho[k] : ldg_state<kCG>(&rho[(size_t)k * G.plane + c]);
-            const double p = fixed ? psi_of<double>(r) : ldg_state<kCG>(&psi[(size_t)k * G.plane + c]);
+            const double p = fixed ? psi64(r, G.one, G.exp_table) : ldg_state<kCG>(&psi[(size_t)k * G.plane + c]);
             outside |= sm.put(k, sy, sx, r, p);
         }
     }
@@ -1094,7 +1103,7 @@ __device__ __forceinline__ void fused_tile64(const Lat<double> *__restrict__ lat
 #pragma unroll 1
         for (int k = 0; k < 2; ++k) {
             const double rk = k ? r[1] : r[0];
-            outside |= sm.put(k, sy, sx, rk, psi_of<double>(rk));
+            outside |= sm.put(k, sy, sx, rk, psi64(rk, G.one, G.exp_table));
         }
     }
     const bool plain = __syncthreads_or(outside != 0);
@@ -1194,7 +1203,9 @@ __device__ __forceinline__ double small_velocity(const Small64 &sm, int a)
     const int lane = threadIdx.x, cx = lane + HALO, cy = HALO;
     const double om0 = sm.st.L.omega[0], om1 = sm.st.L.omega[1];
     const double den = A.add(A.mul(om0, sm.st.v[0][sRho][cy][cx]), A.mul(om1, sm.st.v[1][sRho][cy][cx]));
-    return A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane])) / den;
+    const double n = A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane]));
+    if constexpr (kInt) return quotient64(n, den, reciprocal64(den, A.one));
+    else return n / den;
 }
 
 // Collision and push of half a's directions of species k at node (x, y):
@@ -1263,7 +1274,7 @@ __global__ void __launch_bounds__(TX *kWarps, 2)
     for (int q = tid; q < 2 * SW * (1 + 2 * HALO); q += TX * kWarps) {
         const int sp = q / (SW * (1 + 2 * HALO)), slot = q % (SW * (1 + 2 * HALO)), sx = slot % SW, sy = slot / SW;
         const double r = slot_density<double, false>(G, t, parity, sx, sy, sp);
-        outside |= sm.st.put(sp, sy, sx, r, psi_of<double>(r));
+        outside |= sm.st.put(sp, sy, sx, r, psi64(r, G.one, G.exp_table));
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) outside |= base_outside(p.f[i]);

@@ -109,6 +109,10 @@ cudaError_t offset_to_f64(const Lat<float> &L, const float *h, const float *R, d
 constexpr int kAdjSlotCount = 16;
 constexpr int kAdjGradPlanes = 5;
 
+// The table of exp_minus (lb_f64.cuh) in memory of the current device, which the
+// caller frees.
+cudaError_t make_exp_table(double2 **out, cudaStream_t s);
+
 // Record msg as the calling thread's lb_last_error() message.
 void set_last_error(const char *msg);
 // The parameter check of lb_create for lattice `index` of a batch: LB_OK,

@@ -17,6 +17,8 @@
 #include <stdint.h>
 #include <cstdint>
 
+#include <vector_types.h>
+
 namespace lbk {
 
 // Accumulator slots of the observable reduction, per tile and per lattice.
@@ -38,6 +40,7 @@ struct Lat {
     real *f[2];          // ping-pong population buffers
     real *rho[2];        // density of the previous step (FP32 reference) / of this step
     size_t plane;        // elements per [y][pitch] plane = ny * pitch
+    const double2 *exp_table;   // exp(-j/512) for the FP64 kernels (lb_f64.cuh)
     int32_t nx, ny, pitch;
     int32_t walls;       // 0 periodic, 1 bounce-back walls in y
     int32_t wall_mode;   // 0 mirror, 1 fixed ghost densities
