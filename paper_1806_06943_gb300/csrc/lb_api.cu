@@ -297,6 +297,10 @@ struct lb_engine {
     {
         smode = mode;
         sti = ty_index(ty);
+        // The two passes in FP64 stage fewer slots per node in tiles of 32 x 8, as
+        // long as these leave no SM idle (128^2, 64 tiles: 31.0 us a step against
+        // 25.6 in tiles of 32 x 4; 144^2, 90 tiles: 31.0 and 32.5; 1024^2 641, 655).
+        if (precision == LB_FP64 && mode == LB_MODE_LAUNCH) sti = 2 * (int64_t)stiles[2].size() >= sm_count ? 2 : 1;
         if (precision == LB_FP32 && mode == LB_MODE_LAUNCH) {
             sti = 2;
             smode = tma_ok && (int64_t)stiles[sti].size() >= (int64_t)kTmaTilesPerSm * sm_count ? LB_MODE_TMA : LB_MODE_FUSED;

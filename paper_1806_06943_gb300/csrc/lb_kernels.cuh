@@ -85,8 +85,10 @@ template <> __device__ __forceinline__ double psi_of<double>(double r) { return 
 // same function, written through expm1 so small densities keep their digits
 template <> __device__ __forceinline__ float psi_of<float>(float r) { return -expm1f(-r); }
 
+// a modulo n, the remainder never negative; the division only outside [0, n)
 __device__ __forceinline__ int wrap_index(int a, int n)
 {
+    if ((unsigned)a < (unsigned)n) return a;
     a %= n;
     return a < 0 ? a + n : a;
 }
