@@ -465,7 +465,7 @@ struct lb_engine {
             const int tyv = kTileHeights[ti];
             std::vector<int4> box, rest;
             for (const int4 &t : stiles[ti]) {
-                if (lbk::tma_box_tile(P[t.x].nx, P[t.x].ny, t.y, t.z, tyv))
+                if (lbk::tma_box_tile(P[t.x].nx, P[t.x].ny, tyv))
                     box.push_back(make_int4(t.x, t.y, t.z, lbk::kTmaBoxMark));
                 else
                     rest.push_back(t);
@@ -1345,7 +1345,7 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
                 e->c_off[ti][g] = (int)list.size();
                 for (int pass = 0; pass < 2; ++pass) {
                     for (const int4 &t : e->stiles[ti])
-                        if (group[t.x] == g && lbk::tma_box_tile(p[t.x].nx, p[t.x].ny, t.y, t.z, tyv) == (pass == 0))
+                        if (group[t.x] == g && lbk::tma_box_tile(p[t.x].nx, p[t.x].ny, tyv) == (pass == 0))
                             list.push_back(make_int4(t.x, t.y, t.z, pass == 0 ? lbk::kTmaBoxMark : 0));
                 }
                 e->c_cnt[ti][g] = (int)list.size() - e->c_off[ti][g];

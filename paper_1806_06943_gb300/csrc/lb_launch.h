@@ -71,11 +71,9 @@ struct TmaMaps {
     CUtensorMap ref[3][2];
 };
 constexpr int kTmaBoxW = 40;             // 32 + 2 x 4 columns: x offsets stay 16-byte aligned
-// The tile (x0, y0) of height ty of an nx x ny lattice is staged by TMA.
-__host__ __device__ inline bool tma_box_tile(int nx, int ny, int x0, int y0, int ty)
-{
-    return x0 + 32 <= nx && y0 + ty <= ny && nx >= kTmaBoxW && ny >= ty + 4;
-}
+// Tiles of height ty of an nx x ny lattice are staged by TMA (ragged ones too:
+// the copy fills what lies beyond the lattice with zeros).
+__host__ __device__ inline bool tma_box_tile(int nx, int ny, int ty) { return nx >= kTmaBoxW && ny >= ty + 4; }
 // Fourth field (w) of a tile record that tma_box_tile accepted, set where
 // the host sorts a list into box tiles and the rest (the others keep 0), so
 // that the TMA kernel checks its tile without loading its lattice first.
@@ -85,9 +83,9 @@ constexpr int kTmaBoxMark = 1;
 cudaError_t prepare_fused_tma();
 // One time step of the FP32 tiles [tile_offset, tile_offset + n_tiles) in
 // one pass, one block per tile, each tile staged by one TMA copy of its
-// population box and one of its reference-density box.  Tiles that are full
-// and of a lattice at least kTmaBoxW x (ty + 4) nodes (tma_box_tile) carry
-// w = kTmaBoxMark; the others run as plain one-pass tiles.  A copy not
+// population box and one of its reference-density box.  Tiles of a lattice of
+// at least kTmaBoxW x (ty + 4) nodes (tma_box_tile) carry w = kTmaBoxMark; the
+// others run as plain one-pass tiles.  A copy not
 // complete after wait_cycles SM clocks sets *err = 1 and ends the block; the
 // copy of tile drop_tile (a test hook, -1 for none) is never started.
 cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,

@@ -13,8 +13,8 @@
 // reference-density planes.  Parts of the box beyond the lattice are filled
 // with zeros by the copy and not used: the halo slots there (across a
 // periodic edge, or wall ghost rows) are formed as in fused_tile.  The
-// tiles that tma_box_tile rejects (ragged ones, lattices smaller than the box)
-// run as plain one-pass tiles of the same launch.
+// tiles that tma_box_tile rejects (lattices smaller than the box) run as plain
+// one-pass tiles of the same launch.
 #include "lb_kernels.cuh"
 #include "lb_launch.h"
 
@@ -133,8 +133,9 @@ __device__ __forceinline__ bool slot_outside(const Lat<float> &G, int4 t, int sx
 }
 
 // fused_tile with the tile's and the halo's populations and reference
-// densities read from the box (pop: [18][H][40], ref: [2][H][40]).  The tile
-// is full.  Halo slots beyond the lattice were staged by the caller.
+// densities read from the box (pop: [18][H][40], ref: [2][H][40]).  Slots beyond
+// the lattice (of the halo, and of a ragged tile's missing nodes) were staged
+// by the caller.
 template <int TYv>
 __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ lats, int4 t, int parity,
                                                PairSmem<TYv> &sm, const float *__restrict__ pop,
@@ -155,7 +156,8 @@ __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ la
     const float *own = pop + cy * W + cx + 2;
     float fk[2][9], Rn[2];
     NodeMoments nm;
-    {
+    const bool valid = x < G.nx && y < G.ny;
+    if (valid) {
         float2 v[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) v[i] = make_float2(own[i * H * W], own[(9 + i) * H * W]);
@@ -186,14 +188,14 @@ __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ la
         sm.sp[sy][sx] = make_float2(psi_of<float>(r.x), psi_of<float>(r.y));
     }
     __syncthreads();
+    if (!valid) return;
     const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
     const PairStage<SHv> sg{sm.sr, sm.sp};
     if (inner) collide_site<true, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
     else collide_site<false, true>(sm.L, G.f[parity ^ 1], sg, fk, Rn, x, y, cx, cy, own, H * W, &nm);
 }
 
-// A tile without a box (ragged, or of a lattice smaller than the box): the
-// plain one-pass tile, staged in the box's shared memory.  Out of line, so
+// A tile of a lattice smaller than the box: the plain one-pass tile, staged in the box's shared memory.  Out of line, so
 // that it does not shape the box tiles' registers.
 template <int TYv>
 __device__ __noinline__ void plain_tile(const Lat<float> *__restrict__ lats, int4 t, int parity, float *box)
@@ -204,9 +206,9 @@ __device__ __noinline__ void plain_tile(const Lat<float> *__restrict__ lats, int
 
 // One block per tile: thread 0 starts the two copies, every thread waits
 // (bounded) on the mbarrier, then the tile is computed from the box.  Tiles
-// without the mark run as plain_tile in the same launch: a second launch for
-// them cost more than their work (28 lattices of 220^2, whose last tiles are
-// ragged: 70 -> 64 us a step; 1000^2 48.4 -> 42.9; 333 x 97 11.6 -> 7.1).
+// without the mark run as plain_tile in the same launch.  (With ragged tiles in
+// a second launch 28 lattices of 220^2 took 70 us a step, 1000^2 48.4, 333 x 97
+// 11.6; as plain tiles of the one launch 64, 42.9, 7.1; boxed 57, 41.5, 6.6.)
 template <int TYv>
 __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     k_fused_tma(const Lat<float> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity,
@@ -218,8 +220,7 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     extern __shared__ __align__(128) float box[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ PairSmem<TYv> sm;
-    // the mark: the tile is full and its lattice holds a whole box (so its
-    // maps exist), as the host found when it sorted the list (tma_box_tile),
+    // the mark: the tile's lattice holds a whole box (so its maps exist), as the host found when it sorted the list (tma_box_tile),
     // which keeps the lattice's descriptor off the way to the copy
     const int4 t = tiles[tile_offset + blockIdx.x];
     if (t.w != kTmaBoxMark) {
@@ -253,15 +254,19 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
         }
         if (!first_wave) prefetch_ahead();
     }
-    // halo slots beyond the lattice load their nodes directly (wrapped, or
-    // wall ghost rows): done while the copy is in flight
+    // slots beyond the lattice load their nodes directly (wrapped, or wall
+    // ghost rows): done while the copy is in flight.  They lie in the halo ring,
+    // and in a ragged tile also among its own, up to two beyond its last node
     {
         const Lat<float> &G = lats[t.x];
         if ((t.y == 0 || t.y + TX + HALO > G.nx || t.z < HALO || t.z + TYv + HALO > G.ny)) {
-            for (int h = tid; h < kRing<TYv>; h += TX * TYv) {
-                int sx, sy;
-                ring_slot<TYv>(h, sx, sy);
-                if (slot_outside(G, t, sx, sy)) {
+            const int w = G.nx - t.y, hh = G.ny - t.z;
+            const bool ragged = w < TX || hh < TYv;
+            const int slots = ragged ? SW * (TYv + 2 * HALO) : kRing<TYv>;
+            for (int h = tid; h < slots; h += TX * TYv) {
+                int sx = h % SW, sy = h / SW;
+                if (!ragged) ring_slot<TYv>(h, sx, sy);
+                if (sx < w + 2 * HALO && sy < hh + 2 * HALO && slot_outside(G, t, sx, sy)) {
                     float rA, rB;
                     slot_densities<float, false>(G, t, parity, sx, sy, rA, rB);
                     sm.sr[sy][sx] = make_float2(rA, rB);
