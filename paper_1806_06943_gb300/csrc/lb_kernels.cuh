@@ -211,27 +211,28 @@ __device__ __forceinline__ void force_at(const Lat<real> &L, const real (*srho)[
     }
 }
 
-// The staged density and psi tiles of the species as one [row][col] plane
-// per species and field, as the FP32 collide_site reads them: both species'
-// forces and densities at a staged node as (A, B) pairs.
+// The staged pair planes as collide_site reads them: both species' forces of Eqs. (8), (9) and rho_k g, their densities, and
+// the densities a push re-references with, each as an (A, B) pair.
 template <int SHv>
-struct SplitStage {
-    const float (*srho)[SHv][SW];
-    const float (*spsi)[SHv][SW];
+struct PairStage {
+    const float2 (*sr)[SW];
+    const float2 (*sp)[SW];
+    __device__ __forceinline__ float2 density2(int cy, int cx) const { return sr[cy][cx]; }
+    // Eq. (8) + Eq. (9) + rho_k g, the operations of force_at on each lane
     __device__ __forceinline__ void force2(const Lat<float> &L, int cx, int cy, float2 &Fx, float2 &Fy) const
     {
-        force_at<float, SHv>(L, srho, spsi, 0, cx, cy, Fx.x, Fy.x);
-        force_at<float, SHv>(L, srho, spsi, 1, cx, cy, Fx.y, Fy.y);
+        auto at_psi = [&](int dy, int dx) { return sp[cy + dy][cx + dx]; };
+        auto at_rho = [&](int dy, int dx) { return sr[cy + dy][cx + dx]; };
+        float2 msx, msy, s3x, s3y;
+        vq25c<float2>(at_psi, L.cw, p25f, msx, msy);
+        vq9<float2>(at_rho, s3x, s3y);   // lane j: sums over species j's density
+        // each species is pushed by the other's density sum
+        vforce<float2>(sp[cy][cx], sr[cy][cx], msx, msy, vswap(s3x), vswap(s3y), L.GAB, L.g[0], L.g[1], Fx, Fy);
     }
-    __device__ __forceinline__ float2 density2(int cy, int cx) const
-    {
-        return make_float2(srho[0][cy][cx], srho[1][cy][cx]);
-    }
-    // both species' densities at the staged node (cx + EX, cy + EY)
     template <int EX, int EY>
     __device__ __forceinline__ float2 dest(int cx, int cy) const
     {
-        return make_float2(srho[0][cy + EY][cx + EX], srho[1][cy + EY][cx + EX]);
+        return sr[cy + EY][cx + EX];
     }
 };
 
@@ -343,12 +344,19 @@ __global__ void __launch_bounds__(TX *TYv) k_density(const Lat<real> *__restrict
     density_tile<real, TYv, false>(lats, tiles[tile_offset + blockIdx.x], parity);
 }
 
-// Shared memory of the FP32 step kernels for a tile of height TYv.
+// Shared memory of the FP32 step kernels for a tile of height TYv: density and
+// psi of the tile and its halo as (species A, species B) pairs per node, so that
+// one 64-bit shared load serves both species.
 template <int TYv>
 struct CollideSmem {
-    float srho[2][TYv + 2 * HALO][SW];
-    float spsi[2][TYv + 2 * HALO][SW];
+    float2 sr[TYv + 2 * HALO][SW];
+    float2 sp[TYv + 2 * HALO][SW];
     Lat<float> L;   // descriptor copy: stores to the populations cannot alias it
+    __device__ __forceinline__ void put(int sy, int sx, float rA, float rB)
+    {
+        sr[sy][sx] = make_float2(rA, rB);
+        sp[sy][sx] = make_float2(psi_of<float>(rA), psi_of<float>(rB));
+    }
 };
 
 // Moments of a node's FP32 offset populations that need no force, as
@@ -477,6 +485,9 @@ __device__ __forceinline__ void collide_site(const Lat<float> &L, float *__restr
     dir(std::integral_constant<int, 8>{});
 }
 
+template <typename real>
+__device__ __forceinline__ bool slot_node(const Lat<real> &G, int4 t, int sx, int sy, int &gx, int &gy);
+
 // Fused force + collision + push-streaming + bounce-back for one tile.  Every
 // thread of the block calls it and returns from it; it ends after the tile's
 // pushes are issued (the caller synchronises before reusing sm).
@@ -500,43 +511,17 @@ __device__ __forceinline__ void collide_tile(const Lat<float> *__restrict__ lats
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (float)0;
-    if constexpr (kCG) {
-        // staging reads the density copy through L2 as well
-        constexpr int SHv = TYv + 2 * HALO;
-        const int nx = G.nx, ny = G.ny;
-        const float *__restrict__ rho = G.rho[parity ^ 1];
-        for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
-            const int sx = idx % SW, sy = idx / SW;
-            const int gx = wrap_index(t.y + sx - HALO, nx);
-            int gy = t.z + sy - HALO;
-            float rA, rB;
-            bool fixed = false;
-            if (gy < 0 || gy >= ny) {
-                if (G.walls) {
-                    if (G.wall_mode == 1) {
-                        rA = G.wall_rho[0];
-                        rB = G.wall_rho[1];
-                        fixed = true;
-                    } else {
-                        gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
-                        gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);
-                    }
-                } else {
-                    gy = wrap_index(gy, ny);
-                }
-            }
-            if (!fixed) {
-                const size_t cc = (size_t)gy * G.pitch + gx;
-                rA = __ldcg(&rho[cc]);
-                rB = __ldcg(&rho[G.plane + cc]);
-            }
-            sm.srho[0][sy][sx] = rA;
-            sm.srho[1][sy][sx] = rB;
-            sm.spsi[0][sy][sx] = psi_of<float>(rA);
-            sm.spsi[1][sy][sx] = psi_of<float>(rB);
+    constexpr int SHv = TYv + 2 * HALO;
+    const float *__restrict__ rho = G.rho[parity ^ 1];
+    for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
+        const int sx = idx % SW, sy = idx / SW;
+        int gx, gy;
+        if (!slot_node(G, t, sx, sy, gx, gy)) {
+            sm.put(sy, sx, G.wall_rho[0], G.wall_rho[1]);
+            continue;
         }
-    } else {
-        stage_tile<float, TYv + 2 * HALO>(G, G.rho[parity ^ 1], t.y, t.z, sm.srho, sm.spsi, tid, TX * TYv);
+        const size_t cc = (size_t)gy * G.pitch + gx;
+        sm.put(sy, sx, ldg_state<kCG>(&rho[cc]), ldg_state<kCG>(&rho[G.plane + cc]));
     }
     __syncthreads();
     if (!valid) return;
@@ -546,7 +531,7 @@ __device__ __forceinline__ void collide_tile(const Lat<float> *__restrict__ lats
     Rn[1] = ldg_state<kCG>(&G.rho[parity][G.plane + c]);
     // tiles whose pushes stay inside the lattice (no wrap, no wall) take constant offsets
     const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
-    const SplitStage<TYv + 2 * HALO> sg{sm.srho, sm.spsi};
+    const PairStage<TYv + 2 * HALO> sg{sm.sr, sm.sp};
     if (inner) collide_site<true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
     else collide_site<false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
 }
@@ -874,34 +859,62 @@ __device__ __forceinline__ real node_density(const Lat<real> &L, int k, int gx, 
     return r;
 }
 
-// Density of species k at staged slot (sx, sy) of tile t (slot (HALO, HALO)
-// is the tile's first node) from the populations of its node: x wraps; beyond
-// the lattice in y, periodic wrap, or a wall ghost row (the mirrored fluid
-// row, or the fixed wall densities).
+// The node whose densities staged slot (sx, sy) of tile t holds (slot (HALO,
+// HALO) is the tile's first node): x wraps; beyond the lattice in y, periodic
+// wrap, or a wall ghost row (the mirrored fluid row, or, returning false, the
+// fixed wall densities).
+template <typename real>
+__device__ __forceinline__ bool slot_node(const Lat<real> &G, int4 t, int sx, int sy, int &gx, int &gy)
+{
+    gx = wrap_index(t.y + sx - HALO, G.nx);
+    gy = t.z + sy - HALO;
+    if (gy < 0 || gy >= G.ny) {
+        if (!G.walls) {
+            gy = wrap_index(gy, G.ny);
+        } else if (G.wall_mode == 1) {
+            return false;
+        } else {
+            gy = gy < 0 ? -1 - gy : 2 * G.ny - 1 - gy;
+            gy = gy < 0 ? 0 : (gy >= G.ny ? G.ny - 1 : gy);  // rows no valid node reads
+        }
+    }
+    return true;
+}
+
+// Density of species k at a staged slot from the populations of its node.
 template <typename real, bool kCG>
 __device__ __forceinline__ real slot_density(const Lat<real> &G, int4 t, int parity, int sx, int sy, int k)
 {
-    const int nx = G.nx, ny = G.ny;
-    const int gx = wrap_index(t.y + sx - HALO, nx);
-    int gy = t.z + sy - HALO;
-    if (gy < 0 || gy >= ny) {
-        if (G.walls) {
-            if (G.wall_mode == 1) return G.wall_rho[k];
-            gy = gy < 0 ? -1 - gy : 2 * ny - 1 - gy;
-            gy = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);  // rows no valid node reads
-        } else {
-            gy = wrap_index(gy, ny);
-        }
-    }
-    return node_density<real, kCG>(G, k, gx, gy, parity);
+    int gx, gy;
+    return slot_node(G, t, sx, sy, gx, gy) ? node_density<real, kCG>(G, k, gx, gy, parity) : G.wall_rho[k];
 }
 
+// Both species' densities at a staged slot (FP32: as a pair, lane by lane the
+// sums of node_density).
 template <typename real, bool kCG>
 __device__ __forceinline__ void slot_densities(const Lat<real> &G, int4 t, int parity, int sx, int sy, real &rA,
                                                real &rB)
 {
-    rA = slot_density<real, kCG>(G, t, parity, sx, sy, 0);
-    rB = slot_density<real, kCG>(G, t, parity, sx, sy, 1);
+    int gx, gy;
+    if (!slot_node(G, t, sx, sy, gx, gy)) {
+        rA = G.wall_rho[0];
+        rB = G.wall_rho[1];
+        return;
+    }
+    if constexpr (kOffset<real>) {
+        const size_t c = (size_t)gy * G.pitch + gx;
+        const real *__restrict__ f = G.f[parity], *__restrict__ R = G.rho[parity];
+        float2 v[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            v[i] = make_float2(ldg_state<kCG>(&f[(size_t)i * G.plane + c]), ldg_state<kCG>(&f[(size_t)(9 + i) * G.plane + c]));
+        const float2 r = vadd(make_float2(ldg_state<kCG>(&R[c]), ldg_state<kCG>(&R[G.plane + c])), vzeroth<float2>(v));
+        rA = r.x;
+        rB = r.y;
+    } else {
+        rA = node_density<real, kCG>(G, 0, gx, gy, parity);
+        rB = node_density<real, kCG>(G, 1, gx, gy, parity);
+    }
 }
 
 // Staged slot (sx, sy) of the h-th position of a tile's halo ring, enumerated
@@ -932,10 +945,7 @@ __device__ __forceinline__ void stage_slot(const Lat<float> &G, int4 t, int pari
 {
     float rA, rB;
     slot_densities<float, kCG>(G, t, parity, sx, sy, rA, rB);
-    sm.srho[0][sy][sx] = rA;
-    sm.srho[1][sy][sx] = rB;
-    sm.spsi[0][sy][sx] = psi_of<float>(rA);
-    sm.spsi[1][sy][sx] = psi_of<float>(rB);
+    sm.put(sy, sx, rA, rB);
 }
 
 // One time step of one tile in a single pass: each thread forms its node's
@@ -981,20 +991,20 @@ __device__ __forceinline__ void fused_tile(const Lat<float> *__restrict__ lats, 
     const int cx = threadIdx.x + HALO, cy = threadIdx.y + HALO;
     float Rn[2] = {(float)0, (float)0};
     if (valid) {
+        float2 v[9];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            float r = zeroth_moment<float>(fk[k], 1.f);
-            Rn[k] = ldg_state<kCG>(&G.rho[parity][(size_t)k * G.plane + c]);
-            r = Rn[k] + r;
-            G.rho[parity ^ 1][(size_t)k * G.plane + c] = r;
-            sm.srho[k][cy][cx] = r;
-            sm.spsi[k][cy][cx] = psi_of<float>(r);
-        }
+        for (int i = 0; i < 9; ++i) v[i] = make_float2(fk[0][i], fk[1][i]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) Rn[k] = ldg_state<kCG>(&G.rho[parity][(size_t)k * G.plane + c]);
+        const float2 r = vadd(make_float2(Rn[0], Rn[1]), vzeroth<float2>(v));
+        G.rho[parity ^ 1][c] = r.x;
+        G.rho[parity ^ 1][G.plane + c] = r.y;
+        sm.put(cy, cx, r.x, r.y);
     }
     __syncthreads();
     if (!valid) return;
     const bool inner = t.y >= 1 && t.y + TX + 1 <= sm.L.nx && t.z >= 1 && t.z + TYv + 1 <= sm.L.ny;
-    const SplitStage<SHv> sg{sm.srho, sm.spsi};
+    const PairStage<SHv> sg{sm.sr, sm.sp};
     if (inner) collide_site<true>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
     else collide_site<false>(sm.L, fn, sg, fk, Rn, x, y, cx, cy);
 }

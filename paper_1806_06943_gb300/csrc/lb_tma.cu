@@ -89,41 +89,6 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
-// Staged density and psi of the tile and its halo as (species A, species B)
-// pairs per node, so that one 64-bit shared load serves both species.
-template <int TYv>
-struct PairSmem {
-    float2 sr[TYv + 2 * HALO][SW];
-    float2 sp[TYv + 2 * HALO][SW];
-    Lat<float> L;   // descriptor copy: stores to the populations cannot alias it
-};
-
-// The pair planes as collide_site reads them (the interface of SplitStage):
-// both species' forces of Eqs. (8), (9) and rho_k g, their densities, and
-// the densities a push re-references with, each as an (A, B) pair.
-template <int SHv>
-struct PairStage {
-    const float2 (*sr)[SW];
-    const float2 (*sp)[SW];
-    __device__ __forceinline__ float2 density2(int cy, int cx) const { return sr[cy][cx]; }
-    // Eq. (8) + Eq. (9) + rho_k g, the operations of force_at on each lane
-    __device__ __forceinline__ void force2(const Lat<float> &L, int cx, int cy, float2 &Fx, float2 &Fy) const
-    {
-        auto at_psi = [&](int dy, int dx) { return sp[cy + dy][cx + dx]; };
-        auto at_rho = [&](int dy, int dx) { return sr[cy + dy][cx + dx]; };
-        float2 msx, msy, s3x, s3y;
-        vq25c<float2>(at_psi, L.cw, p25f, msx, msy);
-        vq9<float2>(at_rho, s3x, s3y);   // lane j: sums over species j's density
-        // each species is pushed by the other's density sum
-        vforce<float2>(sp[cy][cx], sr[cy][cx], msx, msy, vswap(s3x), vswap(s3y), L.GAB, L.g[0], L.g[1], Fx, Fy);
-    }
-    template <int EX, int EY>
-    __device__ __forceinline__ float2 dest(int cx, int cy) const
-    {
-        return sr[cy + EY][cx + EX];
-    }
-};
-
 // The slot's node lies beyond the lattice (across a periodic edge, or a wall
 // ghost row): not in the box's lattice part.
 __device__ __forceinline__ bool slot_outside(const Lat<float> &G, int4 t, int sx, int sy)
@@ -138,7 +103,7 @@ __device__ __forceinline__ bool slot_outside(const Lat<float> &G, int4 t, int sx
 // by the caller.
 template <int TYv>
 __device__ __forceinline__ void fused_tile_box(const Lat<float> *__restrict__ lats, int4 t, int parity,
-                                               PairSmem<TYv> &sm, const float *__restrict__ pop,
+                                               CollideSmem<TYv> &sm, const float *__restrict__ pop,
                                                const float *__restrict__ ref)
 {
     constexpr int SHv = TYv + 2 * HALO, H = SHv, W = kTmaBoxW;
@@ -219,7 +184,7 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     constexpr int ti = TYv == 2 ? 0 : (TYv == 4 ? 1 : 2);
     extern __shared__ __align__(128) float box[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ PairSmem<TYv> sm;
+    __shared__ CollideSmem<TYv> sm;
     // the mark: the tile's lattice holds a whole box (so its maps exist), as the host found when it sorted the list (tma_box_tile),
     // which keeps the lattice's descriptor off the way to the copy
     const int4 t = tiles[tile_offset + blockIdx.x];
