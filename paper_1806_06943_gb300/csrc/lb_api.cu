@@ -49,9 +49,9 @@ constexpr int kPersistSteps = 64; // time steps per persistent launch
 constexpr int kChains = 2;         // chains of time steps of a batch's step graph
 constexpr int kTileHeights[3] = {2, 4, 8};
 // Tiles of 32 x 8 nodes per SM from which an FP32 step of LB_MODE_LAUNCH is staged
-// by TMA: three waves of blocks.  Below, the plain one-pass kernel is as fast
-// (512^2, 1024 tiles: 13.7 us a step plain, 14.1 by TMA; 1000^2, 4000 tiles: 51.4
-// and 42.9).
+// by TMA: three waves of blocks.  Below, the plain one-pass kernel is faster
+// (512^2, 1024 tiles: 12.7 us a step plain, 13.5 by TMA; 1000^2, 4000 tiles: 45.3
+// and 40.4).
 constexpr int kTmaTilesPerSm = 12;
 // rows of 32 nodes per SM up to which an FP64 step runs as k_small64
 constexpr int kSmallRowsPerSm = 3;
@@ -291,8 +291,9 @@ struct lb_engine {
     }
     // The kernels of a step for the current configuration.  The two passes of
     // LB_MODE_LAUNCH are slower than one in FP32 at every size (64^2 6.2 us a step
-    // and 5.2, 1024 x 256 14.9 and 13.0, 2048^2 222 and 139), and tiles of 32 x 8
-    // are the fastest for it; every choice gives the same bits.
+    // and 5.2, 1024 x 256 14.9 and 13.0, 2048^2 222 and 139 when this was chosen;
+    // one pass now 4.4, 12.3, 137), and tiles of 32 x 8 are the fastest for it;
+    // every choice gives the same bits.
     void plan_step()
     {
         smode = mode;

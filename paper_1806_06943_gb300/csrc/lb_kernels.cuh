@@ -2,9 +2,10 @@
 // Boltzmann step (Fei et al., arXiv:1806.06943, Sec. II), templated on the
 // population format:
 //   real = double : plain populations f; this instantiation is compiled
-//                   without fused multiply-add and evaluates every sum in the
-//                   same order as a direct evaluation of the equations, so it
-//                   reproduces a plain FP64 evaluation up to the last bit of exp().
+//                   without fused multiply-add and rounds every operation of a
+//                   direct evaluation of the equations, in its order (lb_f64.cuh
+//                   says on which pipe), so it reproduces a plain FP64 evaluation
+//                   up to the last bit of exp().
 //   real = float  : offset populations h_i = f_i - w_i R, R the node's density
 //                   at the previous step (kept in the other density copy), so
 //                   the stored numbers are the small deviations from the local
@@ -21,6 +22,7 @@
 //               BGK relaxation to Eq. (2) with the Guo term of Eq. (5), and
 //               pushes each post-collision population to x + e_i, reflecting
 //               it at a half-way bounce-back wall (Sec. III A).
+// or one: k_fused, k_fused_tma (lb_tma.cu, FP32), k_small64 (small FP64 lattices).
 // The populations at a node are the pre-collision values of the current time,
 // so both passes read them at their own node with coalesced loads.
 #pragma once
@@ -1180,7 +1182,8 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
 // operation is that of node64.  64^2: 25.6 us a step as tiles of 32 x 4 nodes
 // in two launches, 13.4 here with the products on the FP64 pipe, 12.0 with
 // them in integers, which fill the 64 clocks between FP64 instructions
-// (unrolling the staging loop: 14.1, its code outgrows the instruction cache).
+// (unrolling the staging loop: 14.1, its code outgrows the instruction cache),
+// 11.4 with exp() by table.
 constexpr int kSmallWarps = 4;
 
 struct Small64 {
