@@ -57,13 +57,14 @@ FLOOR_BYTES = {1: 144, 0: 288}
 BYTES_FUSED = {1: 160, 0: 288}     # one-pass: 18 pops read + 18 written (+ 2 reference rho read, 2 written)
 BYTES_COLLIDE = {1: 160, 0: 304}   # two-pass fused kernel: 18 pops read + 18 written + 2 rho read (+ 2 reference rho read)
 BYTES_DENSITY = {1: 88, 0: 160}    # density pass: 18 pops read + 2 rho written (+ 2 reference rho read)
-# FP64 operations per node of the FP64 one-pass kernel (k_fused<double, 8>):
-# DADD + DMUL + 2 DFMA thread instructions per node (344 + 236 + 2 x 61.25),
-# counted by ncu on the 512^2 dense emulsion
-# (profiles/k_fused_fp64_dense_emulsion_512.md); FP64 pipe instructions per
-# node (DADD + DMUL + DFMA) beside it.
+# FP64 operations per node of the plain evaluation of the FP64 one-pass step
+# (sums, products and 2 per fma of exp and the divisions: 344 + 236 + 2 x 61.25,
+# counted by ncu on the 512^2 dense emulsion when every one of them ran on the
+# FP64 pipe), and the FP64 pipe instructions per node that k_fused<double, 8>
+# issues for them now that its products are formed in integer instructions
+# (profiles/k_fused_fp64_dense_emulsion_512.md).
 FP64_FLOPS_PER_NODE = 702.6
-FP64_PIPE_OPS_PER_NODE = 641.3
+FP64_PIPE_OPS_PER_NODE = 365.1
 
 
 def parse():
