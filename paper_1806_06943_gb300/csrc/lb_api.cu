@@ -184,6 +184,7 @@ struct lb_engine {
     int sm_count = 0;
     int persist_bps[3] = {0, 0, 0};
     long long wait_cycles = 0;
+    long long default_wait = 0;       // 2 s
     int drop_tile = -1;
     void *d_pool = nullptr;
     size_t pool_bytes = 0;
@@ -327,12 +328,14 @@ struct lb_engine {
         }
         return e;
     }
-    // TMA-staged step over a list of tiles, box tiles first (the test hook that
-    // drops a tile's copy belongs to LB_MODE_TMA)
+    // TMA-staged step over a list of tiles, box tiles first (the wait limit and
+    // the test hook that drops a tile's copy belong to LB_MODE_TMA: a step of
+    // LB_MODE_LAUNCH takes neither)
     cudaError_t launch_tma(const lbk::Lat<float> *L, const int4 *T, int off, int cnt, int par, int h, cudaStream_t s)
     {
-        return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, wait_cycles,
-                                     mode == LB_MODE_TMA ? drop_tile : -1, h, s);
+        const bool tma = mode == LB_MODE_TMA;
+        return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, tma ? wait_cycles : default_wait,
+                                     tma ? drop_tile : -1, h, s);
     }
     size_t ctl_bytes() const { return 8 + 2 * sizeof(unsigned) * (size_t)n; }
     // nsteps time steps in one persistent launch (counters cleared first)
@@ -1308,7 +1311,8 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
         int khz = 0;
         cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, e->device);
         cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, e->device);
-        e->wait_cycles = (long long)(2.0 * (khz > 0 ? khz : 2000000) * 1000.0);   // 2 s
+        e->default_wait = (long long)(2.0 * (khz > 0 ? khz : 2000000) * 1000.0);
+        e->wait_cycles = e->default_wait;
     }
     if ((ce = cudaMemcpyAsync(e->d_lats, lat_src, lat_bytes, cudaMemcpyHostToDevice, e->stream)) != cudaSuccess ||
         (ce = cudaMemcpyAsync(e->d_tiles, e->tiles.data(), e->tiles.size() * sizeof(int4), cudaMemcpyHostToDevice,

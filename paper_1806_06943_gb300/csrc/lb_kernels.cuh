@@ -388,8 +388,7 @@ __device__ __forceinline__ void node_moments(const float2 (&h)[9], float2 rho, f
 
 // ---- velocity-shift forcing of the original model (FP64 only) ---------------
 
-// Second-order equilibrium of direction I (Eq. 2), the same expression as
-// collide_dir's.
+// Second-order equilibrium of direction I (Eq. 2), the operations of relax64.
 template <typename real, int I>
 __device__ __forceinline__ real feq_dir(real rho, real ux, real uy, real uu)
 {
@@ -704,7 +703,7 @@ __device__ __forceinline__ double relax64(const Arith64<kInt> &A, double f, doub
 
 // Force, half-force momenta, u^eq, collision with the Guo term and push of
 // both species at node (x, y), staged at (cx, cy): Eqs. (1)-(3), (5), (6),
-// (8), (9), operation by operation as collide_dir writes them.  j: the
+// (8), (9), each operation rounded once, in the oracle's order.  j: the
 // species' momenta sum_i f e_i; fc, fn: the node's first population plane in
 // the current and the next copy.  Returns whether a value lay outside the
 // range the integer products cover (lb_f64.cuh; the caller then redoes the
