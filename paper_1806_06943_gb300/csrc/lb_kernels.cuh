@@ -731,15 +731,13 @@ __device__ __forceinline__ bool node64(const Stage64<TYv> &sm, double one, const
     const double ny = A.add(A.mul(om0, m[0][1]), A.mul(om1, m[1][1]));
     double ux, uy;
     if constexpr (kInt) {
-        const double rden = reciprocal64(den, A.one);
+        const double rden = __drcp_rn(den);
         ux = quotient64(nx, den, rden);
         uy = quotient64(ny, den, rden);
+        outside = velocity_outside(ux) | velocity_outside(uy);
     } else {
         ux = nx / den;
         uy = ny / den;
-    }
-    if constexpr (kInt) {
-        outside = velocity_outside(ux) | velocity_outside(uy);
     }
     const Dirs64<kInt> dirs(A, ux, uy);
     const Push64 push(L, x, y);
@@ -1218,8 +1216,7 @@ __device__ __forceinline__ double small_velocity(const Small64 &sm, int a)
     const double om0 = sm.st.L.omega[0], om1 = sm.st.L.omega[1];
     const double den = A.add(A.mul(om0, sm.st.v[0][sRho][cy][cx]), A.mul(om1, sm.st.v[1][sRho][cy][cx]));
     const double n = A.add(A.mul(om0, sm.m[0][a][lane]), A.mul(om1, sm.m[1][a][lane]));
-    if constexpr (kInt) return quotient64(n, den, reciprocal64(den, A.one));
-    else return n / den;
+    return n / den;
 }
 
 // Collision and push of half a's directions of species k at node (x, y):
