@@ -189,10 +189,11 @@ struct lb_engine {
     void *d_pool = nullptr;
     size_t pool_bytes = 0;
     // LB_MODE_TMA: one set of tensor maps per lattice (FP32 only), and per
-    // tile height the time-step tiles reordered: the tiles staged by TMA first,
-    // then the others
+    // tile height the time-step tiles reordered: the n_box tiles staged by TMA
+    // first, then the others
     lbk::TmaMaps *d_tmaps = nullptr;
     int4 *d_btiles[3] = {nullptr, nullptr, nullptr};
+    int n_box[3] = {0, 0, 0};
     // FP64 lattices of few nodes: one-row tiles (chain by chain for a batch)
     // of k_small64, which both LB_MODE_LAUNCH and LB_MODE_FUSED then step with
     int4 *d_rows = nullptr;
@@ -221,7 +222,7 @@ struct lb_engine {
     cudaStream_t aux[kChains] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kChains] = {};
     int4 *d_ctiles[3] = {nullptr, nullptr, nullptr};
-    int c_off[3][kChains] = {}, c_cnt[3][kChains] = {};
+    int c_off[3][kChains] = {}, c_box[3][kChains] = {}, c_cnt[3][kChains] = {};
 
     ~lb_engine()
     {
@@ -322,7 +323,7 @@ struct lb_engine {
         } else {
             const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
             if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, par, h, stream);
-            if (smode == LB_MODE_TMA) return launch_tma(L, d_btiles[ti], 0, nt, par, h, stream);
+            if (smode == LB_MODE_TMA) return launch_tma(L, d_btiles[ti], 0, nt, n_box[ti], par, h, stream);
             e = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, par, h, stream);
             if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, par, h, stream);
         }
@@ -331,10 +332,10 @@ struct lb_engine {
     // TMA-staged step over a list of tiles, box tiles first (the wait limit and
     // the test hook that drops a tile's copy belong to LB_MODE_TMA: a step of
     // LB_MODE_LAUNCH takes neither)
-    cudaError_t launch_tma(const lbk::Lat<float> *L, const int4 *T, int off, int cnt, int par, int h, cudaStream_t s)
+    cudaError_t launch_tma(const lbk::Lat<float> *L, const int4 *T, int off, int cnt, int box, int par, int h, cudaStream_t s)
     {
         const bool tma = mode == LB_MODE_TMA;
-        return lbk::launch_fused_tma(L, T, off, cnt, par, d_tmaps, d_err, tma ? wait_cycles : default_wait,
+        return lbk::launch_fused_tma(L, T, off, cnt, box, par, d_tmaps, d_err, tma ? wait_cycles : default_wait,
                                      tma ? drop_tile : -1, h, s);
     }
     size_t ctl_bytes() const { return 8 + 2 * sizeof(unsigned) * (size_t)n; }
@@ -372,7 +373,7 @@ struct lb_engine {
         }
         const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
         if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, T, off, cnt, par, h, s);
-        if (smode == LB_MODE_TMA) return launch_tma(L, T, off, cnt, par, h, s);
+        if (smode == LB_MODE_TMA) return launch_tma(L, T, off, cnt, c_box[ti][g], par, h, s);
         e = lbk::Launch<float>::density(L, T, off, cnt, par, h, s);
         if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, T, off, cnt, par, h, s);
         return e;
@@ -474,6 +475,7 @@ struct lb_engine {
                 else
                     rest.push_back(t);
             }
+            n_box[ti] = (int)box.size();
             box.insert(box.end(), rest.begin(), rest.end());
             if (cudaMalloc((void **)&d_btiles[ti], box.size() * sizeof(int4)) != cudaSuccess) {
                 cudaGetLastError();
@@ -653,7 +655,7 @@ struct lb_engine {
                 if (ce == cudaSuccess && !one) ce = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, parity, ty, stream);
                 if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], stream);
                 if (ce == cudaSuccess)
-                    ce = mode == LB_MODE_TMA ? launch_tma(L, d_btiles[ti], 0, nt, parity, ty, stream)
+                    ce = mode == LB_MODE_TMA ? launch_tma(L, d_btiles[ti], 0, nt, n_box[ti], parity, ty, stream)
                          : one ? lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, parity, ty, stream)
                                : lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, parity, ty, stream);
             }
@@ -1352,6 +1354,7 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
                     for (const int4 &t : e->stiles[ti])
                         if (group[t.x] == g && lbk::tma_box_tile(p[t.x].nx, p[t.x].ny, tyv) == (pass == 0))
                             list.push_back(make_int4(t.x, t.y, t.z, pass == 0 ? lbk::kTmaBoxMark : 0));
+                    if (pass == 0) e->c_box[ti][g] = (int)list.size() - e->c_off[ti][g];
                 }
                 e->c_cnt[ti][g] = (int)list.size() - e->c_off[ti][g];
             }

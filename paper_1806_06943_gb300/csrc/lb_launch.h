@@ -83,12 +83,13 @@ constexpr int kTmaBoxMark = 1;
 cudaError_t prepare_fused_tma();
 // One time step of the FP32 tiles [tile_offset, tile_offset + n_tiles) in
 // one pass, one block per tile, each tile staged by one TMA copy of its
-// population box and one of its reference-density box.  Tiles of a lattice of
-// at least kTmaBoxW x (ty + 4) nodes (tma_box_tile) carry w = kTmaBoxMark; the
-// others run as plain one-pass tiles.  A copy not
-// complete after wait_cycles SM clocks sets *err = 1 and ends the block; the
-// copy of tile drop_tile (a test hook, -1 for none) is never started.
-cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
+// population box and one of its reference-density box.  The first n_box tiles
+// belong to lattices of at least kTmaBoxW x (ty + 4) nodes (tma_box_tile) and
+// carry w = kTmaBoxMark; the others run as plain one-pass tiles (all of them:
+// as k_fused).  A copy not complete after wait_cycles SM clocks sets *err = 1
+// and ends the block; the copy of tile drop_tile (a test hook, -1 for none) is
+// never started.
+cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int n_box, int parity,
                              const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, int ty, cudaStream_t s);
 
 // Discrete adjoint of the FP64 step (lb_adjoint.cu).  Buffers use the

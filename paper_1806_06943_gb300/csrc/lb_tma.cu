@@ -14,7 +14,8 @@
 // with zeros by the copy and not used: the halo slots there (across a
 // periodic edge, or wall ghost rows) are formed as in fused_tile.  The
 // tiles that tma_box_tile rejects (lattices smaller than the box) run as plain
-// one-pass tiles of the same launch.
+// one-pass tiles: of the same launch where a list holds both kinds, of k_fused
+// where it holds no other.
 #include "lb_kernels.cuh"
 #include "lb_launch.h"
 
@@ -170,11 +171,15 @@ __device__ __noinline__ void plain_tile(const Lat<float> *__restrict__ lats, int
 }
 
 // One block per tile: thread 0 starts the two copies, every thread waits
-// (bounded) on the mbarrier, then the tile is computed from the box.  Tiles
-// without the mark run as plain_tile in the same launch.  (With ragged tiles in
-// a second launch 28 lattices of 220^2 took 70 us a step, 1000^2 48.4, 333 x 97
-// 11.6; as plain tiles of the one launch 64, 42.9, 7.1; boxed 57, 41.5, 6.6.)
-template <int TYv>
+// (bounded) on the mbarrier, then the tile is computed from the box.  (With
+// ragged tiles in a second launch 28 lattices of 220^2 took 70 us a step, 1000^2
+// 48.4, 333 x 97 11.6; as plain tiles of the one launch 64, 42.9, 7.1; boxed 57,
+// 41.5, 6.6.)  kMixed: tiles without the mark run as plain_tile.  The call costs
+// registers (height 2: 94 a thread against 72, 4: 78 against 72, 8: 64 both), so
+// at heights 2 and 4 a list of boxes alone takes the form without it (512^2 in
+// tiles of 4: 14.8 and 14.0 us a step; 1000^2 in tiles of 8: 40.2 with, 41.3
+// without).
+template <int TYv, bool kMixed>
 __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     k_fused_tma(const Lat<float> *__restrict__ lats, const int4 *__restrict__ tiles, int tile_offset, int parity,
                 const TmaMaps *__restrict__ maps, int *err, long long wait_cycles, int drop_tile, int n_tiles,
@@ -188,10 +193,11 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     // the mark: the tile's lattice holds a whole box (so its maps exist), as the host found when it sorted the list (tma_box_tile),
     // which keeps the lattice's descriptor off the way to the copy
     const int4 t = tiles[tile_offset + blockIdx.x];
-    if (t.w != kTmaBoxMark) {
-        plain_tile<TYv>(lats, t, parity, box);
-        return;
-    }
+    if constexpr (kMixed)
+        if (t.w != kTmaBoxMark) {
+            plain_tile<TYv>(lats, t, parity, box);
+            return;
+        }
     const int tid = threadIdx.y * TX + threadIdx.x;
     // the boxes of the tile `ahead` blocks later (about one wave of resident
     // blocks) into L2, so that its copies find them there; a block of the
@@ -201,7 +207,7 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
     auto prefetch_ahead = [&]() {
         if (ahead > 0 && (int)blockIdx.x + ahead < n_tiles) {
             const int4 tn = tiles[tile_offset + blockIdx.x + ahead];
-            if (tn.w == kTmaBoxMark) {
+            if (!kMixed || tn.w == kTmaBoxMark) {
                 tma_prefetch_3d(&maps[tn.x].pop[ti][parity], tn.y - 4, tn.z - HALO, 0);
                 tma_prefetch_3d(&maps[tn.x].ref[ti][parity], tn.y - 4, tn.z - HALO, 0);
             }
@@ -261,51 +267,72 @@ __global__ void __launch_bounds__(TX *TYv, kTmaMinBlocks<TYv>)
 // beyond it the boxes are prefetched too early.
 constexpr int kPrefetchQuarterWaves = 3;
 
-template <int TYv>
+template <int TYv, bool kMixed>
 struct TmaKernel {
     static constexpr size_t kSmem = TmaBox<TYv>::kBytes;
     static int grid_wave;   // resident blocks on the device
     static cudaError_t prepare()
     {
-        cudaError_t e = cudaFuncSetAttribute(k_fused_tma<TYv>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        cudaError_t e = cudaFuncSetAttribute(k_fused_tma<TYv, kMixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         int dev = 0, sms = 0, occ = 0;
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fused_tma<TYv>, TX * TYv, kSmem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fused_tma<TYv, kMixed>, TX * TYv, kSmem);
         if (e == cudaSuccess) grid_wave = sms * occ;
         return e;
     }
     static cudaError_t launch(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                               const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, cudaStream_t s)
     {
-        k_fused_tma<TYv><<<n_tiles, dim3(TX, TYv), kSmem, s>>>(lats, tiles, tile_offset, parity, maps, err, wait_cycles,
+        k_fused_tma<TYv, kMixed><<<n_tiles, dim3(TX, TYv), kSmem, s>>>(lats, tiles, tile_offset, parity, maps, err, wait_cycles,
                                                                drop_tile, n_tiles,
                                                                kPrefetchQuarterWaves * grid_wave / 4, grid_wave);
         return cudaGetLastError();
     }
 };
+template <int TYv, bool kMixed>
+int TmaKernel<TYv, kMixed>::grid_wave = 0;
+
 template <int TYv>
-int TmaKernel<TYv>::grid_wave = 0;
+cudaError_t prepare_height_tma()
+{
+    if constexpr (TYv < 8) {
+        const cudaError_t e = TmaKernel<TYv, false>::prepare();
+        if (e != cudaSuccess) return e;
+    }
+    return TmaKernel<TYv, true>::prepare();
+}
+
+template <int TYv>
+cudaError_t launch_height_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int n_box, int parity,
+                              const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, cudaStream_t s)
+{
+    if constexpr (TYv < 8)
+        if (n_box == n_tiles)
+            return TmaKernel<TYv, false>::launch(lats, tiles, tile_offset, n_tiles, parity, maps, err, wait_cycles, drop_tile, s);
+    return TmaKernel<TYv, true>::launch(lats, tiles, tile_offset, n_tiles, parity, maps, err, wait_cycles, drop_tile, s);
+}
 
 }  // namespace
 
 cudaError_t prepare_fused_tma()
 {
-    cudaError_t e = TmaKernel<2>::prepare();
-    if (e == cudaSuccess) e = TmaKernel<4>::prepare();
-    if (e == cudaSuccess) e = TmaKernel<8>::prepare();
+    cudaError_t e = prepare_height_tma<2>();
+    if (e == cudaSuccess) e = prepare_height_tma<4>();
+    if (e == cudaSuccess) e = prepare_height_tma<8>();
     return e;
 }
 
-cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
+cudaError_t launch_fused_tma(const Lat<float> *lats, const int4 *tiles, int tile_offset, int n_tiles, int n_box, int parity,
                              const TmaMaps *maps, int *err, long long wait_cycles, int drop_tile, int ty, cudaStream_t s)
 {
     if (n_tiles <= 0) return cudaSuccess;
+    if (n_box <= 0) return Launch<float>::fused(lats, tiles, tile_offset, n_tiles, parity, ty, s);
     switch (ty) {
-    case 2: return TmaKernel<2>::launch(lats, tiles, tile_offset, n_tiles, parity, maps, err, wait_cycles, drop_tile, s);
-    case 4: return TmaKernel<4>::launch(lats, tiles, tile_offset, n_tiles, parity, maps, err, wait_cycles, drop_tile, s);
-    case 8: return TmaKernel<8>::launch(lats, tiles, tile_offset, n_tiles, parity, maps, err, wait_cycles, drop_tile, s);
+    case 2: return launch_height_tma<2>(lats, tiles, tile_offset, n_tiles, n_box, parity, maps, err, wait_cycles, drop_tile, s);
+    case 4: return launch_height_tma<4>(lats, tiles, tile_offset, n_tiles, n_box, parity, maps, err, wait_cycles, drop_tile, s);
+    case 8: return launch_height_tma<8>(lats, tiles, tile_offset, n_tiles, n_box, parity, maps, err, wait_cycles, drop_tile, s);
     default: return cudaErrorInvalidValue;
     }
 }

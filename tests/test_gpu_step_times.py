@@ -1,0 +1,65 @@
+"""Configurations that do the same work take about the same time.  Each bound is
+the geometric middle between the time with and without the fault it guards
+against, on the shortest of several runs taken in turn; a run in which the
+device was busy otherwise is taken again, three times at most."""
+import time
+
+import pytest
+
+from paper_1806_06943_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+C6 = dict(G_AB=3.0, G1=-7.4, G2=6.4)
+STEPS = 512
+
+
+@pytest.fixture(scope="module")
+def lbmod():
+    from paper_1806_06943_gb300 import build
+    build.build()
+    from paper_1806_06943_gb300 import lb
+    return lb
+
+
+def batch(lbmod, nx, ny, n):
+    b = lbmod.Batch([dict(nx=nx, ny=ny, tau=(1.0, 1.0))] * n, precision=lbmod.LB_FP32, **C6)
+    for i in range(n):
+        b.set_fields(i, W.droplet(nx, ny, min(nx, ny) / 4, seed=i))
+    return b
+
+
+def step_times(b, configs, runs=7):
+    """Microseconds per step of each configuration, the shortest of `runs`."""
+    best = [float("inf")] * len(configs)
+    for _ in range(runs):
+        for k, cfg in enumerate(configs):
+            b.set_config(*cfg)
+            b.step(64)
+            b.synchronize()
+            t0 = time.perf_counter()
+            b.step(STEPS)
+            b.synchronize()
+            best[k] = min(best[k], (time.perf_counter() - t0) * 1e6 / STEPS)
+    return best
+
+
+def holds(b, configs, bound):
+    """The first configuration's time is at most `bound` times the second's."""
+    for _ in range(3):
+        t = step_times(b, configs)
+        if t[0] <= bound * t[1]:
+            return True
+        print("us a step", t)
+    return False
+
+
+@pytest.mark.parametrize("height", [2, 4, 8])
+def test_tma_mode_without_boxes_is_the_fused_mode(lbmod, height):
+    """Lattices narrower than a box have nothing to stage by TMA: both modes are
+    one kernel (1.12 to 1.15 times the time as plain tiles of the TMA kernel)."""
+    b = batch(lbmod, 32, 32, 9)
+    try:
+        assert holds(b, [(lbmod.LB_MODE_TMA, height), (lbmod.LB_MODE_FUSED, height)], 1.07)
+    finally:
+        b.close()
