@@ -346,8 +346,14 @@ struct lb_engine {
         cudaError_t e = cudaMemsetAsync(d_ctl, 0, ctl_bytes(), stream);
         if (e != cudaSuccess) return e;
         unsigned *dens = (unsigned *)((char *)d_ctl + 8), *coll = dens + n;
+        // No more blocks than tiles: only that many work items are ever ready, and
+        // blocks that wait poll the counters of those that work (24 lattices of
+        // 37 x 50 in FP32 tiles of 2: 27 us a step with every resident block, 12 so).
+        // At least one per SM, which claim items ahead (128 x 5 in tiles of 8: 8.1
+        // us with a block per tile, 7.3 so).
         int blocks = persist_bps[ti] * sm_count;
         if (blocks <= 0) blocks = sm_count > 0 ? sm_count : 1;
+        blocks = std::min(blocks, std::max(nt, sm_count));
         if (precision == LB_FP64)
             return lbk::Launch<double>::persistent((const lbk::Lat<double> *)d_lats, d_stiles[ti], d_sntiles[ti], nt,
                                                    nsteps, par, d_ctl, dens, coll, d_err, wait_cycles, drop_tile, ty,

@@ -516,17 +516,25 @@ __device__ __forceinline__ void collide_tile(const Lat<float> *__restrict__ lats
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (float)0;
-    constexpr int SHv = TYv + 2 * HALO;
+    constexpr int SHv = TYv + 2 * HALO, kSlots = (SW * SHv + TX * TYv - 1) / (TX * TYv);
     const float *__restrict__ rho = G.rho[parity ^ 1];
-    for (int idx = tid; idx < SW * SHv; idx += TX * TYv) {
-        const int sx = idx % SW, sy = idx / SW;
+    // all of the thread's slots loaded before the first is staged
+    float2 r[kSlots];
+#pragma unroll
+    for (int q = 0; q < kSlots; ++q) {
+        const int idx = tid + q * TX * TYv;
+        if (idx >= SW * SHv) break;
         int gx, gy;
-        if (!slot_node(G, t, sx, sy, gx, gy)) {
-            sm.put(sy, sx, G.wall_rho[0], G.wall_rho[1]);
-            continue;
+        r[q] = make_float2(G.wall_rho[0], G.wall_rho[1]);
+        if (slot_node(G, t, idx % SW, idx / SW, gx, gy)) {
+            const size_t cc = (size_t)gy * G.pitch + gx;
+            r[q] = make_float2(ldg_state<kCG>(&rho[cc]), ldg_state<kCG>(&rho[G.plane + cc]));
         }
-        const size_t cc = (size_t)gy * G.pitch + gx;
-        sm.put(sy, sx, ldg_state<kCG>(&rho[cc]), ldg_state<kCG>(&rho[G.plane + cc]));
+    }
+#pragma unroll
+    for (int q = 0; q < kSlots; ++q) {
+        const int idx = tid + q * TX * TYv;
+        if (idx < SW * SHv) sm.put(idx / SW, idx % SW, r[q].x, r[q].y);
     }
     __syncthreads();
     if (!valid) return;

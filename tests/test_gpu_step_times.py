@@ -63,3 +63,13 @@ def test_tma_mode_without_boxes_is_the_fused_mode(lbmod, height):
         assert holds(b, [(lbmod.LB_MODE_TMA, height), (lbmod.LB_MODE_FUSED, height)], 1.07)
     finally:
         b.close()
+
+
+def test_persistent_mode_of_many_small_tiles(lbmod):
+    """24 lattices of 37 x 50: tiles of 2 rows, 1200 of them, take 1.1 times as
+    long as tiles of 8 (2.4 times with more blocks polling than tiles)."""
+    b = batch(lbmod, 37, 50, 24)
+    try:
+        assert holds(b, [(lbmod.LB_MODE_PERSISTENT, 2), (lbmod.LB_MODE_PERSISTENT, 8)], 1.6)
+    finally:
+        b.close()
