@@ -106,9 +106,10 @@ struct lb3_handle {
         tmp_elems = elems;
         return LB_OK;
     }
-    cudaError_t density(int par)
+    cudaError_t density(int par, bool step)
     {
-        return f64() ? lbk3::Launch3<double>::density(L64, par, stream) : lbk3::Launch3<float>::density(L32, par, stream);
+        return f64() ? lbk3::Launch3<double>::density(L64, par, step, stream)
+                     : lbk3::Launch3<float>::density(L32, par, step, stream);
     }
     cudaError_t collide(int par)
     {
@@ -252,7 +253,7 @@ int lb3_observables(lb3_handle *h, lb3_obs *o)
 {
     CHECK3(h);
     if (!o) return fail3(LB_EINVAL, "o is NULL");
-    LB3_CUDA(h->density(h->parity));
+    LB3_CUDA(h->density(h->parity, false));
     LB3_CUDA(h->observe(h->partials, nullptr, nullptr));
     LB3_CUDA(lbk3::reduce3(h->partials, h->n_tiles, h->obs, h->stream));
     double s[lbk3::kNumAcc];
@@ -287,7 +288,7 @@ int lb3_get_fields(lb3_handle *h, double *rho, double *ubar)
     const size_t n = h->cells();
     int rc = h->ensure_tmp(5 * n);
     if (rc) return rc;
-    LB3_CUDA(h->density(h->parity));
+    LB3_CUDA(h->density(h->parity, false));
     LB3_CUDA(h->observe(nullptr, h->tmp, h->tmp + 2 * n));
     if (rho) LB3_CUDA(cudaMemcpyAsync(rho, h->tmp, 2 * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     if (ubar) LB3_CUDA(cudaMemcpyAsync(ubar, h->tmp + 2 * n, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -330,7 +331,7 @@ int lb3_profile(lb3_handle *h, int32_t nsteps, void *flush_buf, size_t flush_byt
         if (flush_bytes) ce = cudaMemsetAsync(flush_buf, s & 0xff, flush_bytes, h->stream);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s], h->stream);
         // FP32: the whole step is one kernel
-        if (ce == cudaSuccess && h->f64()) ce = h->density(h->parity);
+        if (ce == cudaSuccess && h->f64()) ce = h->density(h->parity, true);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], h->stream);
         if (ce == cudaSuccess) ce = h->f64() ? h->collide(h->parity) : h->step(h->parity);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 2], h->stream);

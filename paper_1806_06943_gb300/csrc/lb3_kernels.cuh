@@ -313,7 +313,8 @@ __device__ __forceinline__ void force3(const Lat3<real> &L, const Stage3<real> &
     for (int a = 0; a < 3; ++a) F[a] = -L.G1 * psi * s1[a] - L.G2 * psi * s2[a] - L.GAB * rho * s3[a] + rho * L.g[a];
 }
 
-template <typename real>
+// kPsi: psi of the step (FP64) as well.
+template <typename real, bool kPsi>
 __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int parity)
 {
     int x0, y0, z0;
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) k3_density(const Lat3<real> L, int p
         L.rho[parity ^ 1][(size_t)k * L.plane + c] = r;
         // FP64 keeps no reference densities: copy parity holds psi for the
         // collide kernel, so that exp() runs once per node
-        if constexpr (!kOffset3<real>) L.rho[parity][(size_t)k * L.plane + c] = lbk::psi64(r, lbk::opaque_one(), L.exp_table);
+        if constexpr (kPsi) L.rho[parity][(size_t)k * L.plane + c] = lbk::psi64(r, lbk::opaque_one(), L.exp_table);
     }
 }
 

@@ -12,7 +12,8 @@ template <typename real>
 struct Launch3 {
     // one time step: FP32 in one pass (k3_march), FP64 density pass + collide
     static cudaError_t step(const Lat3<real> &L, int parity, int sms, cudaStream_t s);
-    static cudaError_t density(const Lat3<real> &L, int parity, cudaStream_t s);
+    // step: the density pass of a step (FP64: leaves psi as well), else of the observables
+    static cudaError_t density(const Lat3<real> &L, int parity, bool step, cudaStream_t s);
     static cudaError_t collide(const Lat3<real> &L, int parity, cudaStream_t s);
     static cudaError_t observe(const Lat3<real> &L, int parity, double *partials, double *rho, double *u,
                                cudaStream_t s);

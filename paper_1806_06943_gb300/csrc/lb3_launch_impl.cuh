@@ -7,10 +7,15 @@
 namespace lbk3 {
 
 template <typename real>
-cudaError_t Launch3<real>::density(const Lat3<real> &L, int parity, cudaStream_t s)
+cudaError_t Launch3<real>::density(const Lat3<real> &L, int parity, bool step, cudaStream_t s)
 {
     const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
-    k3_density<real><<<n, dim3(TX, TY, TZ), 0, s>>>(L, parity);
+    if constexpr (!kOffset3<real>)
+        if (step) {
+            k3_density<real, true><<<n, dim3(TX, TY, TZ), 0, s>>>(L, parity);
+            return cudaGetLastError();
+        }
+    k3_density<real, false><<<n, dim3(TX, TY, TZ), 0, s>>>(L, parity);
     return cudaGetLastError();
 }
 
@@ -66,7 +71,7 @@ cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, int sms, cudaSt
         k3_march<kMarchBlocks><<<n, dim3(TX, RY), sizeof(March3), s>>>(L, parity, tiles_y, lz);
         return cudaGetLastError();
     } else {
-        cudaError_t e = density(L, parity, s);
+        cudaError_t e = density(L, parity, true, s);
         if (e == cudaSuccess) e = collide(L, parity, s);
         return e;
     }

@@ -288,8 +288,8 @@ struct lb_engine {
     cudaError_t launch_density_obs(int par, int off, int cnt)
     {
         if (precision == LB_FP64)
-            return lbk::Launch<double>::density((const lbk::Lat<double> *)d_lats, d_tiles, off, cnt, par, 4, stream);
-        return lbk::Launch<float>::density((const lbk::Lat<float> *)d_lats, d_tiles, off, cnt, par, 4, stream);
+            return lbk::Launch<double>::density_obs((const lbk::Lat<double> *)d_lats, d_tiles, off, cnt, par, stream);
+        return lbk::Launch<float>::density_obs((const lbk::Lat<float> *)d_lats, d_tiles, off, cnt, par, stream);
     }
     // The kernels of a step for the current configuration.  The two passes of
     // LB_MODE_LAUNCH are slower than one in FP32 at every size (64^2 6.2 us a step

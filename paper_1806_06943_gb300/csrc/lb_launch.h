@@ -20,6 +20,9 @@ struct Launch {
     // height ty (2, 4 or 8)
     static cudaError_t density(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                                int ty, cudaStream_t s);
+    // the densities alone (FP64: no psi), over tiles of height 4, for the observables
+    static cudaError_t density_obs(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
+                                   cudaStream_t s);
     static cudaError_t collide(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
                                int ty, cudaStream_t s);
     // one time step in one pass (densities formed in the kernel)

@@ -38,11 +38,20 @@ cudaError_t Launch<real>::density(const Lat<real> *lats, const int4 *tiles, int 
 {
     if (n_tiles <= 0) return cudaSuccess;
     switch (ty) {
-    case 2: k_density<real, 2><<<n_tiles, dim3(TX, 2), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 4: k_density<real, 4><<<n_tiles, dim3(TX, 4), 0, s>>>(lats, tiles, tile_offset, parity); break;
-    case 8: k_density<real, 8><<<n_tiles, dim3(TX, 8), 0, s>>>(lats, tiles, tile_offset, parity); break;
+    case 2: k_density<real, 2, !kOffset<real>><<<n_tiles, dim3(TX, 2), 0, s>>>(lats, tiles, tile_offset, parity); break;
+    case 4: k_density<real, 4, !kOffset<real>><<<n_tiles, dim3(TX, 4), 0, s>>>(lats, tiles, tile_offset, parity); break;
+    case 8: k_density<real, 8, !kOffset<real>><<<n_tiles, dim3(TX, 8), 0, s>>>(lats, tiles, tile_offset, parity); break;
     default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+template <typename real>
+cudaError_t Launch<real>::density_obs(const Lat<real> *lats, const int4 *tiles, int tile_offset, int n_tiles, int parity,
+                                      cudaStream_t s)
+{
+    if (n_tiles <= 0) return cudaSuccess;
+    k_density<real, TY, false><<<n_tiles, dim3(TX, TY), 0, s>>>(lats, tiles, tile_offset, parity);
     return cudaGetLastError();
 }
 
