@@ -53,8 +53,11 @@ constexpr int kTileHeights[3] = {2, 4, 8};
 // (512^2, 1024 tiles: 12.7 us a step plain, 13.5 by TMA; 1000^2, 4000 tiles: 45.3
 // and 40.4).
 constexpr int kTmaTilesPerSm = 12;
-// rows of 32 nodes per SM up to which an FP64 step runs as k_small64
-constexpr int kSmallRowsPerSm = 3;
+// Rows of 32 nodes per SM up to which an FP64 step runs as k_small64: its blocks of
+// one row are resident four to an SM, so one wave.  Microseconds a step by rows
+// and by the fastest tiles, lattices 64 wide: 152 rows 11.2 and 25.3, 456 18.9 and
+// 25.6, 608 23.5 and 25.6, 684 33.5 and 31.6.
+constexpr int kSmallRowsPerSm = 4;
 
 int ty_index(int ty) { return ty == 2 ? 0 : (ty == 4 ? 1 : (ty == 8 ? 2 : -1)); }
 constexpr size_t kAlign = 256;
@@ -300,10 +303,12 @@ struct lb_engine {
     {
         smode = mode;
         sti = ty_index(ty);
-        // The two passes in FP64 stage fewer slots per node in tiles of 32 x 8, as
-        // long as these leave no SM idle (128^2, 64 tiles: 31.0 us a step against
-        // 25.6 in tiles of 32 x 4; 144^2, 90 tiles: 31.0 and 32.5; 1024^2 641, 655).
-        if (precision == LB_FP64 && mode == LB_MODE_LAUNCH) sti = 2 * (int64_t)stiles[2].size() >= sm_count ? 2 : 1;
+        // The two passes in FP64 stage fewer slots per node in tiles of 32 x 8, but
+        // a step of at most one tile of 32 x 4 per SM takes one such tile's time
+        // (64 x 304, 152 tiles of 4: 25.6 us a step and 31.3 in tiles of 8; 64 x 342,
+        // 172 tiles, 32.8 and 31.6; 1024^2 655 and 641).  Without rows only: the
+        // velocity-shift model.
+        if (precision == LB_FP64 && mode == LB_MODE_LAUNCH) sti = (int64_t)stiles[1].size() > sm_count ? 2 : 1;
         if (precision == LB_FP32 && mode == LB_MODE_LAUNCH) {
             sti = 2;
             smode = tma_ok && (int64_t)stiles[sti].size() >= (int64_t)kTmaTilesPerSm * sm_count ? LB_MODE_TMA : LB_MODE_FUSED;
@@ -496,9 +501,8 @@ struct lb_engine {
     }
 
     // Row tiles of k_small64 where the FP64 step of all lattices is short of
-    // nodes: up to kSmallRowsPerSm rows of 32 nodes per SM (a wave of one row
-    // per SM takes 15 k clocks, the tile kernels 40 k for their first wave of
-    // four).  The velocity-shift model stays on the tile kernels.
+    // nodes: up to kSmallRowsPerSm rows of 32 nodes per SM.  The velocity-shift
+    // model stays on the tile kernels.
     int build_rows(const std::vector<int> &chain)
     {
         if (precision != LB_FP64) return LB_OK;

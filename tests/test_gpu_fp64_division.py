@@ -58,7 +58,7 @@ def planned(nx, ny, seed, fast):
     return f.reshape(2, 9, ny, nx)
 
 
-@pytest.mark.parametrize("nx,ny", [(70, 37), (230, 75)])   # row by row (k_small64), and in tiles
+@pytest.mark.parametrize("nx,ny", [(70, 37), (300, 90)])   # row by row (k_small64), and in tiles
 @pytest.mark.parametrize("mode", [0, 1, 2])
 @pytest.mark.parametrize("fast", [False, True])
 def test_velocity_is_the_rounded_quotient(oracle_mod, nx, ny, mode, fast):
