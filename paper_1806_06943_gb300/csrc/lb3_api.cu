@@ -184,6 +184,7 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
     }
     if (h->f64()) {
         const cudaError_t e = lbk::make_exp_table(&h->exp_table, h->stream);
+        if (e == cudaErrorMemoryAllocation) return bail(fail3(LB_ENOMEM, "lb3: cudaMalloc of the exp table failed"));
         if (e != cudaSuccess) return bail(cuda_fail3(e, "exp table"));
         h->L64.exp_table = h->exp_table;
     }

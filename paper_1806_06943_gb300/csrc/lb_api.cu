@@ -558,6 +558,14 @@ struct lb_engine {
         return lbk::Launch<float>::finalize((const lbk::Lat<float> *)d_lats, n, d_partials, d_fold, d_obs, stream);
     }
 
+    int ensure_exp_table()
+    {
+        if (d_exp) return LB_OK;
+        const cudaError_t e = lbk::make_exp_table(&d_exp, stream);
+        if (e == cudaErrorMemoryAllocation) return fail(LB_ENOMEM, "cudaMalloc of the exp table failed");
+        return e == cudaSuccess ? LB_OK : cuda_fail(e, "exp table");
+    }
+
     int ensure_tmp(size_t elems)
     {
         if (elems <= tmp_elems) return LB_OK;
@@ -822,7 +830,6 @@ struct lb_engine {
             L = L64[0];
         } else {
             fill_lat(L, p);
-            L.exp_table = d_exp;
             L.pitch = L32[0].pitch;
             L.plane = L32[0].plane;
             L.has_probe = L32[0].has_probe;
@@ -837,6 +844,8 @@ struct lb_engine {
         }
         int rc = begin();
         if (rc) return rc;
+        if ((rc = ensure_exp_table())) return rc;
+        L.exp_table = d_exp;
         // pop64: one FP64 state, the adjoint's unit; state: one state of the
         // forward precision (FP32: offsets + reference densities)
         const size_t plane_b = plane(0) * sizeof(double), pop64 = 18 * plane_b;
@@ -1241,7 +1250,9 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
     }
     if ((ce = cudaMemsetAsync(e->d_pool, 0, total, e->stream)) != cudaSuccess) return bail(cuda_fail(ce, "cudaMemsetAsync"));
 
-    if ((ce = lbk::make_exp_table(&e->d_exp, e->stream)) != cudaSuccess) return bail(cuda_fail(ce, "exp table"));
+    // (an FP32 lattice's adjoint makes it when it first runs)
+    if (e->precision == LB_FP64)
+        if (int rc = e->ensure_exp_table()) return bail(rc);
     // tiles in raster order, lattice by lattice
     for (int l = 0; l < n; ++l) {
         const int begin = (int)e->tiles.size();

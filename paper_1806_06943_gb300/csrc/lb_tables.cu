@@ -1,9 +1,8 @@
 // lb_tables.cu -- the table of exp(-j/512) the FP64 kernels read (lb_f64.cuh),
 // formed once per process in extended precision and kept by each handle on its
 // device.
+#include <array>
 #include <cmath>
-#include <mutex>
-#include <vector>
 
 #include "lb_f64.cuh"
 #include "lb_launch.h"
@@ -12,19 +11,25 @@ namespace lbk {
 
 cudaError_t make_exp_table(double2 **out, cudaStream_t s)
 {
-    static std::vector<double2> host;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        host.resize(kExpSize);
+    static const std::array<double2, kExpSize> host = [] {
+        std::array<double2, kExpSize> t{};
         for (int j = 0; j < kExpSize; ++j) {
             const long double e = expl(-(long double)j / kExpSteps);
-            host[j].x = (double)e;
-            host[j].y = (double)(e - (long double)host[j].x);
+            t[j].x = (double)e;
+            t[j].y = (double)(e - (long double)t[j].x);
         }
-    });
-    cudaError_t e = cudaMalloc((void **)out, kExpSize * sizeof(double2));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(*out, host.data(), kExpSize * sizeof(double2), cudaMemcpyHostToDevice, s);
+        return t;
+    }();
+    double2 *table = nullptr;
+    cudaError_t e = cudaMalloc((void **)&table, kExpSize * sizeof(double2));
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // not left for the next launch's check to find
+        return e;
+    }
+    e = cudaMemcpyAsync(table, host.data(), kExpSize * sizeof(double2), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) *out = table;
+    else cudaFree(table);
     return e;
 }
 
