@@ -62,8 +62,9 @@ extern "C" {
  * LB_MODE_LAUNCH: each time step is launched by itself, replayed 32 steps per
  *   CUDA graph: a density-pass launch and a fused-kernel launch over the tiles
  *   of all lattices, or the one launch of the fastest one-pass form where that
- *   takes less time (LB_FP32; LB_FP64 lattices of a few thousand nodes, in
- *   LB_MODE_FUSED too).  lb_profile always times the two launches.
+ *   takes less time (LB_FP32; LB_FP64 lattices of up to some 20,000 nodes, in
+ *   LB_MODE_FUSED too, whatever the tile height).  lb_profile times the two
+ *   launches in this mode.
  * LB_MODE_PERSISTENT: one launch advances 64 time steps of all lattices; its
  *   blocks take (step, phase, tile) work items from an atomic queue and wait,
  *   with a bounded spin, only for the tiles of their own lattice that an item
@@ -273,11 +274,14 @@ int lb_load(lb_handle *h, const void *buf, size_t len);
 
 /* Time nsteps time steps kernel by kernel with CUDA events on the handle's
  * stream (direct launches, no graph):
- *   ms[0]  mean duration of one density-pass launch (0 in LB_MODE_FUSED)
+ *   ms[0]  mean duration of one density-pass launch (0 in LB_MODE_FUSED and
+ *          LB_MODE_TMA)
  *   ms[1]  mean duration of one fused force/collide/stream launch (in
- *          LB_MODE_FUSED the one-pass kernel; LB_MODE_PERSISTENT is timed as
- *          LB_MODE_LAUNCH)
+ *          LB_MODE_FUSED and LB_MODE_TMA the one-pass kernel lb_step launches;
+ *          in LB_MODE_LAUNCH and LB_MODE_PERSISTENT the two passes at the tile
+ *          height set, whatever kernels lb_step takes)
  *   ms[2]  mean duration of one whole time step (both launches)
+ * The populations are those of nsteps steps of lb_step.
  * If flush_bytes > 0, the caller's device buffer flush_buf of that size is
  * overwritten before every step, outside the timed intervals, so that each
  * step starts with no population data in L2.  The lattice advances by

@@ -666,8 +666,9 @@ struct lb_engine {
                 if (ce == cudaSuccess && !one) ce = lbk::Launch<double>::density(L, d_stiles[ti], 0, nt, parity, ty, stream);
                 if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], stream);
                 if (ce == cudaSuccess)
-                    ce = one ? lbk::Launch<double>::fused(L, d_stiles[ti], 0, nt, parity, ty, stream)
-                             : lbk::Launch<double>::collide(L, d_stiles[ti], 0, nt, parity, ty, stream);
+                    ce = one && n_rows ? lbk::Launch<double>::small(L, d_rows, 0, n_rows, parity, stream)
+                         : one         ? lbk::Launch<double>::fused(L, d_stiles[ti], 0, nt, parity, ty, stream)
+                                       : lbk::Launch<double>::collide(L, d_stiles[ti], 0, nt, parity, ty, stream);
             } else {
                 const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
                 if (ce == cudaSuccess && !one) ce = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, parity, ty, stream);

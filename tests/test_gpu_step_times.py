@@ -73,3 +73,19 @@ def test_persistent_mode_of_many_small_tiles(lbmod):
         assert holds(b, [(lbmod.LB_MODE_PERSISTENT, 2), (lbmod.LB_MODE_PERSISTENT, 8)], 1.6)
     finally:
         b.close()
+
+
+def test_profile_of_the_fused_mode_times_the_step(lbmod):
+    """A small FP64 lattice steps row by row in LB_MODE_FUSED whatever its tile
+    height, and lb_profile times that kernel (timing the tiles instead, those of
+    8 rows took 1.2 times those of 4)."""
+    L = lbmod.Lattice(64, 64, tau=(1.0, 1.0), **C6)
+    L.set_fields(W.droplet(64, 64, 16.0, seed=1))
+    best = {4: float("inf"), 8: float("inf")}
+    for _ in range(20):
+        for height in best:
+            L.set_config(lbmod.LB_MODE_FUSED, height)
+            best[height] = min(best[height], L.profile(32)[1])
+    L.close()
+    print("ms a launch", best)
+    assert best[8] <= 1.1 * best[4]
