@@ -201,14 +201,15 @@ int lb_synchronize(lb_handle *h);
 /* Execution configuration: mode (LB_MODE_LAUNCH, LB_MODE_PERSISTENT,
  * LB_MODE_FUSED, or LB_MODE_TMA for LB_FP32 lattices) and tile height (2, 4
  * or 8 nodes; tiles are 32 nodes wide, one thread per node).  Default:
- * LB_MODE_LAUNCH, 4.  Results do not depend on it beyond the rounding order of
- * FP32 sums.  LB_EINVAL for an unknown mode or height, or LB_MODE_TMA on an
+ * LB_MODE_LAUNCH, 4.  LB_MODE_LAUNCH takes the tile height that is fastest for
+ * the lattice; the one set is that of lb_profile, and lb_get_config returns it.
+ * Results do not depend on either.  LB_EINVAL for an unknown mode or height, or LB_MODE_TMA on an
  * LB_FP64 handle or where the driver offers no tensor-map encoder. */
 int lb_set_config(lb_handle *h, int32_t mode, int32_t tile_height);
 int lb_get_config(const lb_handle *h, int32_t *mode, int32_t *tile_height);
 
-/* Autotuner: times every mode and tile height on trial_steps time steps of
- * the current state (the state is restored after each trial, so the lattice
+/* Autotuner: times every mode and tile height (once each step that several of
+ * them share) on trial_steps time steps of the current state (the state is restored after each trial, so the lattice
  * does not advance) and keeps the fastest.  With cache_path != NULL the
  * choice is read from / appended to that text file, keyed by device name,
  * precision and lattice shapes; a cached key skips the trials.  *best_ms

@@ -727,7 +727,9 @@ struct lb_engine {
     }
 
     // Time every (mode, tile height) on trial_steps steps of the current state
-    // (restored after each trial) and keep the fastest; results are cached in
+    // (restored after each trial) and keep the fastest; of those that launch the
+    // same kernel over the same tiles (plan_step) only the first, LB_MODE_LAUNCH
+    // under the height it takes.  Results are cached in
     // cache_path (one "key mode ty ms" line per configuration) when given.
     int autotune(int trial_steps, const char *cache_path, double *best_ms)
     {
@@ -766,9 +768,16 @@ struct lb_engine {
         int bm = mode, bty = ty;
         cudaError_t ce = cudaMemcpyAsync(snap, d_pool, pool_bytes, cudaMemcpyDeviceToDevice, stream);
         const int last_mode = tma_ok ? LB_MODE_TMA : LB_MODE_FUSED;
+        constexpr int kRowsKind = LB_MODE_TMA + 1;
+        bool seen[kRowsKind + 1][3] = {};   // by kernel and tile list
         for (int m = LB_MODE_LAUNCH; m <= last_mode && ce == cudaSuccess && rc == LB_OK; ++m)
             for (int tyv : kTileHeights) {
                 if ((rc = set_config(m, tyv))) break;
+                if (m == LB_MODE_LAUNCH && kTileHeights[sti] != tyv) continue;
+                const bool rows = n_rows && (m == LB_MODE_LAUNCH || m == LB_MODE_FUSED);
+                bool &timed = rows ? seen[kRowsKind][0] : seen[smode][sti];
+                if (timed) continue;
+                timed = true;
                 if ((rc = step(chunk_steps()))) break;            // warm-up, builds the graph
                 ce = cudaEventRecord(e0, stream);
                 if (ce == cudaSuccess && (rc = step(trial_steps))) break;
