@@ -81,8 +81,7 @@ extern "C" {
  *   reference-density planes), completed on an mbarrier; each block also
  *   prefetches into L2 the box of a tile about a wave of blocks later.  Nodes
  *   across a periodic edge or on wall ghost rows, and smaller lattices, load as
- *   in LB_MODE_FUSED, in the same launch.  Same arithmetic as LB_MODE_FUSED,
- *   same results.  A copy not complete within the wait limit (default 2 s) ends
+ *   in LB_MODE_FUSED.  Same arithmetic as LB_MODE_FUSED, same results.  A copy not complete within the wait limit (default 2 s) ends
  *   its block and the next synchronising call returns LB_ETIMEOUT. */
 #define LB_MODE_LAUNCH 0
 #define LB_MODE_PERSISTENT 1
@@ -190,12 +189,13 @@ int lb_set_fields_device(lb_handle *h, const double *rho, const double *u);
 
 /* Advance n >= 0 time steps.  Asynchronous: returns once the work is
  * enqueued; a failure detected on the device surfaces on the next
- * synchronising call (lb_observables, lb_get_fields, lb_synchronize). */
+ * synchronising call (lb_observables, lb_get_fields, lb_synchronize and the
+ * other calls that read the state). */
 int lb_step(lb_handle *h, int64_t n);
 
 /* Block until the handle's queued work has finished.  Returns LB_ETIMEOUT
- * (once) if a bounded device-side wait of a persistent launch, or of a TMA
- * copy in LB_MODE_TMA, expired. */
+ * (once) if a bounded device-side wait expired: of a persistent launch, or of a
+ * TMA copy (LB_MODE_TMA, and LB_MODE_LAUNCH where it steps so). */
 int lb_synchronize(lb_handle *h);
 
 /* Execution configuration: mode (LB_MODE_LAUNCH, LB_MODE_PERSISTENT,
@@ -353,7 +353,8 @@ int lb_batch_set_config(lb_batch *b, int32_t mode, int32_t tile_height);
 int lb_batch_get_config(const lb_batch *b, int32_t *mode, int32_t *tile_height);
 int lb_batch_autotune(lb_batch *b, int32_t trial_steps, const char *cache_path, double *best_ms);
 /* Limit of every bounded wait of the persistent kernel and of the TMA copies
- * of LB_MODE_TMA, in seconds (default 2).  drop_tile >= 0 is a test hook:
+ * of LB_MODE_TMA, in seconds (default 2; the TMA copies of LB_MODE_LAUNCH keep
+ * the default).  drop_tile >= 0 is a test hook:
  * that tile of the batch's tile list (for the configured tile height) never
  * reports completion in LB_MODE_PERSISTENT, or never has its copy started in
  * LB_MODE_TMA, so the waits on it run out and the launch ends with

@@ -189,6 +189,7 @@ struct lb_engine {
     long long wait_cycles = 0;
     long long default_wait = 0;       // 2 s
     int drop_tile = -1;
+    bool waits = false;               // steps with bounded waits enqueued since the last check_timeout
     void *d_pool = nullptr;
     size_t pool_bytes = 0;
     // LB_MODE_TMA: one set of tensor maps per lattice (FP32 only), and per
@@ -536,6 +537,7 @@ struct lb_engine {
         int h = 0;
         LB_CUDA(cudaMemcpyAsync(&h, d_err, sizeof h, cudaMemcpyDeviceToHost, stream));
         LB_CUDA(cudaStreamSynchronize(stream));
+        waits = false;
         if (h) {
             LB_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
             LB_CUDA(cudaStreamSynchronize(stream));
@@ -609,6 +611,7 @@ struct lb_engine {
         int rc = begin();
         if (rc) return rc;
         const int chunk = chunk_steps();
+        if (nsteps > 0 && (smode == LB_MODE_PERSISTENT || smode == LB_MODE_TMA)) waits = true;
         while (nsteps > 0) {
             if (parity == 0 && nsteps >= chunk) {
                 if (!gexec && (rc = build_graph())) return rc;
@@ -656,6 +659,7 @@ struct lb_engine {
                 return fail(LB_ECUDA, "cudaEventCreate failed");
             }
         const int ti = ty_index(ty), nt = (int)stiles[ti].size();
+        if (mode == LB_MODE_TMA) waits = true;
         cudaError_t ce = cudaSuccess;
         for (int s = 0; s < nsteps && ce == cudaSuccess; ++s) {
             if (flush_bytes) ce = cudaMemsetAsync(flush, s & 0xff, flush_bytes, stream);
@@ -1111,6 +1115,7 @@ struct lb_engine {
         const size_t cells = (size_t)nx(l) * ny(l);
         int rc = begin();
         if (rc) return rc;
+        if (waits && (rc = check_timeout())) return rc;
         if ((rc = ensure_tmp(8 * cells))) return rc;
         LB_CUDA(launch_density_obs(parity, tile_begin(l), tile_end(l) - tile_begin(l)));
         LB_CUDA(launch_observe(parity, tile_begin(l), tile_end(l) - tile_begin(l), nullptr, d_tmp, d_tmp + 2 * cells,
@@ -1156,6 +1161,7 @@ struct lb_engine {
         const size_t cells = (size_t)nx(l) * ny(l);
         int rc = begin();
         if (rc) return rc;
+        if (waits && (rc = check_timeout())) return rc;
         if ((rc = ensure_tmp(18 * cells))) return rc;
         if (precision == LB_FP64)
             LB_CUDA(lbk::Launch<double>::get_pops((const lbk::Lat<double> *)d_lats, l, nx(l), ny(l), parity, d_tmp, stream));
@@ -1584,6 +1590,7 @@ int lb_save(lb_handle *h, void *buf, size_t *len)
     std::memcpy(buf, &hd, sizeof hd);
     int rc = e->begin();
     if (rc) return rc;
+    if (e->waits && (rc = e->check_timeout())) return rc;
     LB_CUDA(cudaMemcpyAsync((char *)buf + sizeof hd, e->fbuf(0, e->parity), e->pop_bytes(0), cudaMemcpyDeviceToHost,
                             e->stream));
     if (e->ref_bytes(0))
