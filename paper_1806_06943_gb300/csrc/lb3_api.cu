@@ -74,7 +74,7 @@ struct lb3_handle {
     double *partials = nullptr, *obs = nullptr, *tmp = nullptr;
     size_t tmp_elems = 0;
     int n_tiles = 0;
-    int sm_count = 0;
+    int march = 0;                    // planes a block of the FP32 step marches
     int parity = 0;
     int64_t t = 0;
 
@@ -117,8 +117,8 @@ struct lb3_handle {
     }
     cudaError_t step(int par)
     {
-        return f64() ? lbk3::Launch3<double>::step(L64, par, sm_count, stream)
-                     : lbk3::Launch3<float>::step(L32, par, sm_count, stream);
+        return f64() ? lbk3::Launch3<double>::step(L64, par, march, stream)
+                     : lbk3::Launch3<float>::step(L32, par, march, stream);
     }
     cudaError_t observe(double *part, double *rho, double *u)
     {
@@ -153,7 +153,8 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
         cudaGetLastError();
         return bail(fail3(LB_ECUDA, "no CUDA device"));
     }
-    if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail3(LB_ECUDA, "cudaDeviceGetAttribute failed"));
     }
@@ -198,6 +199,9 @@ int lb3_create(const lb3_params *p, lb3_handle **out)
     h->L32.f[1] = (float *)f1;
     h->L32.rho[0] = (float *)r0;
     h->L32.rho[1] = (float *)r1;
+    const cudaError_t e = h->f64() ? lbk3::Launch3<double>::prepare(h->L64, sms, h->march)
+                                   : lbk3::Launch3<float>::prepare(h->L32, sms, h->march);
+    if (e != cudaSuccess) return bail(cuda_fail3(e, "shared memory of the step kernel"));
     *out = h;
     return LB_OK;
 }

@@ -10,8 +10,11 @@ namespace lbk3 {
 
 template <typename real>
 struct Launch3 {
+    // shared memory of the step's kernel on the current device, and the planes
+    // a block marches (FP32); call before the first step
+    static cudaError_t prepare(const Lat3<real> &L, int sms, int &march);
     // one time step: FP32 in one pass (k3_march), FP64 density pass + collide
-    static cudaError_t step(const Lat3<real> &L, int parity, int sms, cudaStream_t s);
+    static cudaError_t step(const Lat3<real> &L, int parity, int march, cudaStream_t s);
     // step: the density pass of a step (FP64: leaves psi as well), else of the observables
     static cudaError_t density(const Lat3<real> &L, int parity, bool step, cudaStream_t s);
     static cudaError_t collide(const Lat3<real> &L, int parity, cudaStream_t s);

@@ -26,15 +26,12 @@ cudaError_t Launch3<real>::collide(const Lat3<real> &L, int parity, cudaStream_t
         return cudaErrorInvalidValue;   // FP32 steps in one pass
     } else {
         const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
-        cudaError_t e = cudaFuncSetAttribute(k3_collide<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kCollideSmem3<real>);
-        if (e != cudaSuccess) return e;
         k3_collide<real><<<n, dim3(TX, TY, TZ), kCollideSmem3<real>, s>>>(L, parity);
         return cudaGetLastError();
     }
 }
 
-// Resident blocks per SM of the marching kernels.
+// Resident blocks per SM of the marching kernel.
 constexpr int kMarchBlocks = 2;
 
 // Planes a block marches along z: the whole column, or segments of it where
@@ -58,17 +55,25 @@ inline int march_planes(int64_t columns, int nz, int slots, double rim)
 }
 
 template <typename real>
-cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, int sms, cudaStream_t s)
+cudaError_t Launch3<real>::prepare(const Lat3<real> &L, int sms, int &march)
+{
+    if constexpr (kOffset3<real>) {
+        march = march_planes((int64_t)L.tiles_x * ((L.ny + RY - 1) / RY), L.nz, kMarchBlocks * sms, 0.4);
+        return cudaFuncSetAttribute(k3_march<kMarchBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March3));
+    } else {
+        march = 0;
+        return cudaFuncSetAttribute(k3_collide<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kCollideSmem3<real>);
+    }
+}
+
+template <typename real>
+cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, int march, cudaStream_t s)
 {
     if constexpr (kOffset3<real>) {
         const int tiles_y = (L.ny + RY - 1) / RY;
-        const int64_t columns = (int64_t)L.tiles_x * tiles_y;
-        const int lz = march_planes(columns, L.nz, kMarchBlocks * sms, 0.4);
-        cudaError_t e = cudaFuncSetAttribute(k3_march<kMarchBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(March3));
-        if (e != cudaSuccess) return e;
-        const unsigned n = (unsigned)(columns * ((L.nz + lz - 1) / lz));
-        k3_march<kMarchBlocks><<<n, dim3(TX, RY), sizeof(March3), s>>>(L, parity, tiles_y, lz);
+        const unsigned n = (unsigned)((int64_t)L.tiles_x * tiles_y * ((L.nz + march - 1) / march));
+        k3_march<kMarchBlocks><<<n, dim3(TX, RY), sizeof(March3), s>>>(L, parity, tiles_y, march);
         return cudaGetLastError();
     } else {
         cudaError_t e = density(L, parity, true, s);

@@ -89,3 +89,23 @@ def test_profile_of_the_fused_mode_times_the_step(lbmod):
     L.close()
     print("ms a launch", best)
     assert best[8] <= 1.1 * best[4]
+
+
+def test_enqueueing_a_3d_step_does_not_grow_with_the_lattice(lbmod):
+    """lb3_step returns once its launch is enqueued: the host's time for it is the
+    same for 100 planes and for 40,000 (the search for the planes a block marches,
+    made at every step, took 200 us there)."""
+    best = {}
+    for nz in (100, 40000):
+        L = lbmod.Lattice3(5, 5, nz, precision=lbmod.LB_FP32, **C6)
+        L.step(4)
+        L.observables(check=False)
+        best[nz] = float("inf")
+        for _ in range(7):
+            t0 = time.perf_counter()
+            L.step(20)
+            best[nz] = min(best[nz], (time.perf_counter() - t0) / 20)
+            L.observables(check=False)
+        L.close()
+    print("host seconds a step", best)
+    assert best[40000] <= 4.0 * best[100]
