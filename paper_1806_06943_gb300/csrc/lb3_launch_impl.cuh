@@ -35,17 +35,23 @@ cudaError_t Launch3<real>::collide(const Lat3<real> &L, int parity, cudaStream_t
 constexpr int kMarchBlocks = 2;
 
 // Planes a block marches along z: the whole column, or segments of it where
-// columns alone do not fill the device evenly.  A segment forms the densities
-// of 4 more planes than it steps, `rim` of a plane's work each.
-inline int march_planes(int64_t columns, int nz, int slots, double rim)
+// columns alone do not fill the device evenly.  A segment forms the densities of
+// 4 more planes than it steps, 0.4 of a plane's work each, and a wave of two
+// blocks per SM takes 1.45 times as long as one of a single block.  Microseconds
+// a step by planes (blocks): 33 x 33 x 32 3 (110) 21.0, 2 (160) 24.8, 1 (320) 24.8;
+// 75 x 38 x 32 2 (240) 24.8, 4 (120) 26.8; 64^3 4 (256) 36.9, 8 (128) 42.2; 160^3
+// 54 (300) 422, 27 (600) 417, 20 (800) 455.
+inline int march_planes(int64_t columns, int nz, int sms)
 {
+    constexpr double kRim = 4 * 0.4, kPair = 1.45;
+    static_assert(kMarchBlocks == 2, "the cost of a wave counts one or two blocks per SM");
     int best = nz;
     double cost = 1e300;
     for (int segs = 1; segs <= nz; ++segs) {
         const int lz = (nz + segs - 1) / segs;
         if ((nz + lz - 1) / lz != segs) continue;
-        const int64_t waves = (columns * segs + slots - 1) / slots;
-        const double c = (double)waves * (lz + 4.0 * rim);
+        const int64_t blocks = columns * segs, waves = blocks / (2 * sms), rest = blocks % (2 * sms);
+        const double c = (kPair * (double)waves + (rest == 0 ? 0.0 : rest <= sms ? 1.0 : kPair)) * (lz + kRim);
         if (c < cost * 0.999) {
             cost = c;
             best = lz;
@@ -58,7 +64,7 @@ template <typename real>
 cudaError_t Launch3<real>::prepare(const Lat3<real> &L, int sms, int &march)
 {
     if constexpr (kOffset3<real>) {
-        march = march_planes((int64_t)L.tiles_x * ((L.ny + RY - 1) / RY), L.nz, kMarchBlocks * sms, 0.4);
+        march = march_planes((int64_t)L.tiles_x * ((L.ny + RY - 1) / RY), L.nz, sms);
         return cudaFuncSetAttribute(k3_march<kMarchBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March3));
     } else {
         march = 0;
