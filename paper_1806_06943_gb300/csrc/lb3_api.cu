@@ -111,10 +111,6 @@ struct lb3_handle {
         return f64() ? lbk3::Launch3<double>::density(L64, par, step, stream)
                      : lbk3::Launch3<float>::density(L32, par, step, stream);
     }
-    cudaError_t collide(int par)
-    {
-        return f64() ? lbk3::Launch3<double>::collide(L64, par, stream) : lbk3::Launch3<float>::collide(L32, par, stream);
-    }
     cudaError_t step(int par)
     {
         return f64() ? lbk3::Launch3<double>::step(L64, par, march, stream)
@@ -338,7 +334,7 @@ int lb3_profile(lb3_handle *h, int32_t nsteps, void *flush_buf, size_t flush_byt
         // FP32: the whole step is one kernel
         if (ce == cudaSuccess && h->f64()) ce = h->density(h->parity, true);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 1], h->stream);
-        if (ce == cudaSuccess) ce = h->f64() ? h->collide(h->parity) : h->step(h->parity);
+        if (ce == cudaSuccess) ce = h->f64() ? lbk3::collide3(h->L64, h->parity, h->stream) : h->step(h->parity);
         if (ce == cudaSuccess) ce = cudaEventRecord(ev[3 * s + 2], h->stream);
         if (ce == cudaSuccess) {
             h->parity ^= 1;

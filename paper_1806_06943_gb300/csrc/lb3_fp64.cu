@@ -5,6 +5,13 @@
 namespace lbk3 {
 template struct Launch3<double>;
 
+cudaError_t collide3(const Lat3<double> &L, int parity, cudaStream_t s)
+{
+    const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
+    k3_collide<double><<<n, dim3(TX, TY, TZ), kCollideSmem3<double>, s>>>(L, parity);
+    return cudaGetLastError();
+}
+
 cudaError_t reduce3(double *partials, int n_tiles, double *out, cudaStream_t s)
 {
     // one block took 1.5 ms over a 160^3 lattice's 16000 tiles: fold them first

@@ -17,7 +17,6 @@ struct Launch3 {
     static cudaError_t step(const Lat3<real> &L, int parity, int march, cudaStream_t s);
     // step: the density pass of a step (FP64: leaves psi as well), else of the observables
     static cudaError_t density(const Lat3<real> &L, int parity, bool step, cudaStream_t s);
-    static cudaError_t collide(const Lat3<real> &L, int parity, cudaStream_t s);
     static cudaError_t observe(const Lat3<real> &L, int parity, double *partials, double *rho, double *u,
                                cudaStream_t s);
     static cudaError_t init(const Lat3<real> &L, const double *rho, const double *u, int parity, cudaStream_t s);
@@ -28,6 +27,9 @@ struct Launch3 {
 // behind the n_tiles.
 constexpr int kFold3 = 64;
 cudaError_t reduce3(double *partials, int n_tiles, double *out, cudaStream_t s);
+
+// the FP64 step after its density pass
+cudaError_t collide3(const Lat3<double> &L, int parity, cudaStream_t s);
 
 extern template struct Launch3<double>;
 extern template struct Launch3<float>;

@@ -19,18 +19,6 @@ cudaError_t Launch3<real>::density(const Lat3<real> &L, int parity, bool step, c
     return cudaGetLastError();
 }
 
-template <typename real>
-cudaError_t Launch3<real>::collide(const Lat3<real> &L, int parity, cudaStream_t s)
-{
-    if constexpr (kOffset3<real>) {
-        return cudaErrorInvalidValue;   // FP32 steps in one pass
-    } else {
-        const unsigned n = (unsigned)L.tiles_x * L.tiles_y * L.tiles_z;
-        k3_collide<real><<<n, dim3(TX, TY, TZ), kCollideSmem3<real>, s>>>(L, parity);
-        return cudaGetLastError();
-    }
-}
-
 // Resident blocks per SM of the marching kernel.
 constexpr int kMarchBlocks = 2;
 
@@ -83,7 +71,7 @@ cudaError_t Launch3<real>::step(const Lat3<real> &L, int parity, int march, cuda
         return cudaGetLastError();
     } else {
         cudaError_t e = density(L, parity, true, s);
-        if (e == cudaSuccess) e = collide(L, parity, s);
+        if (e == cudaSuccess) e = collide3(L, parity, s);
         return e;
     }
 }

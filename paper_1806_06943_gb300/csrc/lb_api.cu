@@ -330,6 +330,7 @@ struct lb_engine {
             const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
             if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, d_stiles[ti], 0, nt, par, h, stream);
             if (smode == LB_MODE_TMA) return launch_tma(L, d_btiles[ti], 0, nt, n_box[ti], par, h, stream);
+            // LB_MODE_PERSISTENT: the steps lb_grad recomputes
             e = lbk::Launch<float>::density(L, d_stiles[ti], 0, nt, par, h, stream);
             if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, d_stiles[ti], 0, nt, par, h, stream);
         }
@@ -384,11 +385,8 @@ struct lb_engine {
             return e;
         }
         const lbk::Lat<float> *L = (const lbk::Lat<float> *)d_lats;
-        if (smode == LB_MODE_FUSED) return lbk::Launch<float>::fused(L, T, off, cnt, par, h, s);
         if (smode == LB_MODE_TMA) return launch_tma(L, T, off, cnt, c_box[ti][g], par, h, s);
-        e = lbk::Launch<float>::density(L, T, off, cnt, par, h, s);
-        if (e == cudaSuccess) e = lbk::Launch<float>::collide(L, T, off, cnt, par, h, s);
-        return e;
+        return lbk::Launch<float>::fused(L, T, off, cnt, par, h, s);   // one pass (plan_step)
     }
     // time steps in the current mode, as captured into one graph: with
     // chains, chains 1.. fork onto their auxiliary streams and join the
