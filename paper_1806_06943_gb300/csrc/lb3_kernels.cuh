@@ -89,7 +89,7 @@ struct Lat3 {
     real omega[2];       // 1 / tau_k
     real aw3[2][3];      // 3 (1 - omega_k / 2) w(|e|^2) for |e|^2 = 0, 1, 2
     const double2 *exp_table;   // exp(-j/512) for the FP64 density pass (lb_f64.cuh)
-    real cw[9];          // -(G1 w + G2 q) for |e|^2 = 0 .. 8 (FP32: the two psi sums of Eq. 8 as one)
+    real cw[9];          // -(G1 w + G2 q) for |e|^2 = 0 .. 8 (the two psi sums of Eq. 8 as one)
     real G1, G2, GAB;
     real g[3];
     double probe[4];     // cx, cy, cz, R

@@ -104,9 +104,9 @@ __device__ __forceinline__ void adj_sums(const Arith64<false> &A, const double (
 //   rho_bar = omega P,  P = M0 + 3 M1.u + 4.5 u.M2 u - 1.5 u.u M0,
 //   omega_bar = rho P - sum_i lam*_i f_i - V.F / 2,
 // which takes a third of the FP64 instructions (they bound the kernel) of the
-// sums written per direction: 397 a node instead of 1414, 214 -> 64 us on a
+// sums written per direction: 415 a node instead of 1414, 214 -> 67 us on a
 // 512 x 128 lattice; k_adj_gather, with one combined stencil, 158 instead of
-// 559, 90 -> 31 us.
+// 559, 90 -> 30 us.
 __global__ void __launch_bounds__(kThreads, 4) k_adj_local(const Lat<double> L, const double *__restrict__ f,
                                                            const double *__restrict__ rho, const double *__restrict__ lam_next,
                                                            double *__restrict__ abuf, double *__restrict__ gpart, int seed_kind,

@@ -15,8 +15,8 @@
 // has the bits of the IEEE operation it stands for, so the step still rounds
 // as a plain evaluation of the equations, operation by operation.  With the
 // products shared between neighbours (Stage64) a node of the one-pass step
-// costs 380 FP64 instructions instead of 641; a 1024^2 step 0.73 ms instead
-// of 1.30, its FP64 pipe 89 % busy.
+// costs 369 FP64 instructions instead of 641; a 1024^2 step 0.67 ms instead
+// of 1.30, its FP64 pipe 86 % busy.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -81,7 +81,8 @@ __device__ __forceinline__ double factor_mul(const Factor &a, const Factor &b)
 //   the populations, densities and psi it reads are zero or in
 //     [2^-179, 2^77) (base_outside() is 0),
 //   the couplings, relaxation rates and body forces are zero or in
-//     [2^-64, 2^64) (checked on the host: Lat::products), and
+//     [2^-58, 2^64) (checked on the host: Lat::products), so that times a weight
+//     of at least 1/36 they are above 2^-64, and
 //   the velocity's components are zero or in [2^-255, 2^256)
 //     (velocity_outside() is 0).
 // A nonzero sum is at least 2^-53 times its smallest term, so stencil sums
@@ -131,8 +132,8 @@ struct Arith64 {
 // with j the nearest integer to 512 r and t = r - j/512 (exact),
 //   exp(-r) = T_j exp(-t) = T_j + T_j p,   p = -t + t^2 (1/2 - t/6 + t^2/24 - t^3/120)
 // to 2^-69 for |t| <= 2^-10, T_j as a double and its remainder.  10 FP64
-// instructions, where exp() takes 15 (1024^2 step 0.73 -> 0.69 ms, 333 x 97 36.7
-// -> 34.5 us).  Largest error seen on 2e7 arguments 0.5015 ulp.  Outside the
+// instructions, where exp() takes 15 (1024^2 one-pass step 704 -> 674 us, 333 x 97
+// 34.1 -> 33.0, 64^2 11.4 -> 10.9).  Largest error seen on 2e7 arguments 0.5015 ulp.  Outside the
 // table (densities below 0 or from 2 on) exp().
 constexpr int kExpSteps = 512, kExpSize = 2 * kExpSteps + 1;
 

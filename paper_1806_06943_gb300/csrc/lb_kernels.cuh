@@ -1192,7 +1192,7 @@ __global__ void __launch_bounds__(TX *TYv, kCollideMinBlocks<real, TYv>)
 // in two launches, 13.4 here with the products on the FP64 pipe, 12.0 with
 // them in integers, which fill the 64 clocks between FP64 instructions
 // (unrolling the staging loop: 14.1, its code outgrows the instruction cache),
-// 11.4 with exp() by table.
+// 10.9 with exp() by table.
 constexpr int kSmallWarps = 4;
 
 struct Small64 {
