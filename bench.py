@@ -20,7 +20,7 @@ written once: 144 B per node in FP32, 288 B in FP64) per launch over its
 CUDA-event time, against the measured copy bandwidth; the design's own
 byte count (160 B per node in FP32, with the reference densities) beside
 it.  The FP64 kernel is bound by the FP64 pipe and is reported against the
-device's measured FP64 FMA rate.
+device's measured rate of FP64 FMA instructions.
 
 Side legs (skipped with --quick): the Laplace fit of the sweep after 20000
 steps, the same batch in FP64, the 4096x4096 dense emulsion in FP32 and
@@ -57,14 +57,13 @@ FLOOR_BYTES = {1: 144, 0: 288}
 BYTES_FUSED = {1: 160, 0: 288}     # one-pass: 18 pops read + 18 written (+ 2 reference rho read, 2 written)
 BYTES_COLLIDE = {1: 160, 0: 304}   # two-pass fused kernel: 18 pops read + 18 written + 2 rho read (+ 2 reference rho read)
 BYTES_DENSITY = {1: 88, 0: 160}    # density pass: 18 pops read + 2 rho written (+ 2 reference rho read)
-# FP64 operations per node of the plain evaluation of the FP64 one-pass step
-# (sums, products and 2 per fma of exp and the divisions: 344 + 236 + 2 x 61.25,
-# counted by ncu on the 512^2 dense emulsion when every one of them ran on the
-# FP64 pipe), and the FP64 pipe instructions per node that k_fused<double, 8>
-# issues for them now that its products are formed in integer instructions
-# (profiles/k_fused_fp64_dense_emulsion_512.md).
+# FP64 pipe instructions per node that the one-pass kernel and the second of two
+# passes issue at tile height 8 (profiles/k_fused_fp64_dense_emulsion_512.md; most
+# of their products are formed in integer instructions), and the FP64 operations of the plain evaluation of the
+# same step (sums, products and 2 per fma of exp and the divisions: 344 + 236 +
+# 2 x 61.25, counted by ncu when every one of them ran on the FP64 pipe).
+FP64_PIPE_OPS_PER_NODE = {"k_fused": 369.1, "k_collide": 290.0}
 FP64_FLOPS_PER_NODE = 702.6
-FP64_PIPE_OPS_PER_NODE = 365.1
 
 
 def parse():
@@ -259,16 +258,20 @@ def hbm_roofline(kname, units, ms, peak, peak_kind, floor_b, design_b, traffic):
 
 
 def alu_roofline(kname, units, ms, peak_tflops, hbm_peak):
-    """Roofline of the FP64 step kernel, bound by the FP64 pipe: FP64
-    operations per node (ncu count) x nodes / launch time against the
-    measured FP64 FMA rate of the device."""
-    ach = FP64_FLOPS_PER_NODE * units / (ms * 1e-3) / 1e12 if FP64_FLOPS_PER_NODE else None
-    return {"bound": "alu", "kernel": kname, "achieved": ach, "peak": peak_tflops, "unit": "TFLOP/s",
-            "frac": (ach / peak_tflops) if (ach and peak_tflops) else None, "traffic": None,
-            "peak_source": "measured FP64 FMA throughput of this device (lb_device_fp64_peak)",
-            "flops_per_site": FP64_FLOPS_PER_NODE, "units_per_launch": units, "ms_per_launch": ms,
-            "fp64_pipe_frac": FP64_PIPE_OPS_PER_NODE * units / (ms * 1e-3) / (peak_tflops * 1e12 / 2),
-            "hbm_frac_floor": FLOOR_BYTES[0] * units / (ms * 1e-3) / 1e9 / hbm_peak}
+    """Roofline of the FP64 step kernel, bound by the FP64 pipe: the FP64
+    instructions the kernel issues (ncu count) x nodes / launch time against the
+    measured rate of the device's FP64 FMA instructions (two operations each).
+    The plain evaluation's operations over the same time stand beside it: part
+    of them run on other pipes, so they have no fraction of this peak."""
+    per_s = units / (ms * 1e-3)
+    ops = FP64_PIPE_OPS_PER_NODE[kname.split("<")[0]]
+    ach, peak = ops * per_s / 1e12, peak_tflops / 2
+    return {"bound": "alu", "kernel": kname, "achieved": ach, "peak": peak, "unit": "T FP64 instructions/s",
+            "frac": ach / peak, "traffic": None,
+            "peak_source": "measured FP64 FMA throughput of this device (lb_device_fp64_peak), an instruction a fma",
+            "fp64_instructions_per_site": ops, "units_per_launch": units, "ms_per_launch": ms,
+            "plain_evaluation_tflops": FP64_FLOPS_PER_NODE * per_s / 1e12,
+            "hbm_frac_floor": FLOOR_BYTES[0] * per_s / 1e9 / hbm_peak}
 
 
 # ---- CPU oracle timing -------------------------------------------------------------
