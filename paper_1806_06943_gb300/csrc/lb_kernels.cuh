@@ -520,7 +520,8 @@ __device__ __forceinline__ void collide_tile(const Lat<float> *__restrict__ lats
         for (int i = 0; i < 9; ++i) fk[k][i] = valid ? ldg_state<kCG>(&fc[(size_t)(k * 9 + i) * G.plane + c]) : (float)0;
     constexpr int SHv = TYv + 2 * HALO, kSlots = (SW * SHv + TX * TYv - 1) / (TX * TYv);
     const float *__restrict__ rho = G.rho[parity ^ 1];
-    // all of the thread's slots loaded before the first is staged
+    // all of the thread's slots loaded before the first is staged (128 x 5 in tiles of
+    // 4, LB_MODE_PERSISTENT: 9.2 us a step one after the other, 8.8 so)
     float2 r[kSlots];
 #pragma unroll
     for (int q = 0; q < kSlots; ++q) {
