@@ -207,7 +207,7 @@ struct lb_engine {
     std::string tma_why = "LB_MODE_TMA needs LB_FP32 populations";
     double2 *d_exp = nullptr;         // table of the FP64 kernels (also the adjoint of FP32 lattices)
     double *d_partials = nullptr;
-    double *d_fold = nullptr;         // kFold records per lattice, where one has more than kFoldTiles tiles
+    double *d_fold = nullptr;         // kFold records per lattice behind the partials, where one has more than kFoldTiles tiles
     double *d_obs = nullptr;
     double *d_psum = nullptr;         // pressure-tensor sums, kPStride doubles per lattice
     double *d_tmp = nullptr;
@@ -246,7 +246,6 @@ struct lb_engine {
         cudaFree(d_tmaps);
         cudaFree(d_partials);
         cudaFree(d_exp);
-        cudaFree(d_fold);
         cudaFree(d_obs);
         cudaFree(d_psum);
         cudaFree(d_tmp);
@@ -463,7 +462,11 @@ struct lb_engine {
                 }
             }
         }
-        if (lbk::prepare_fused_tma() != cudaSuccess) {
+        bool mixed = false;
+        for (int tyv : kTileHeights)
+            for (const lb_params &p : P)
+                mixed = mixed || lbk::tma_box_tile(p.nx, p.ny, tyv) != lbk::tma_box_tile(P[0].nx, P[0].ny, tyv);
+        if (lbk::prepare_fused_tma(mixed) != cudaSuccess) {
             cudaGetLastError();
             tma_why = "LB_MODE_TMA: the TMA kernels cannot get their shared memory on this device";
             return LB_OK;
@@ -1299,19 +1302,20 @@ int engine_create(const lb_params *p, int n, lb_engine **out)
     }
     const size_t lat_bytes = e->precision == LB_FP64 ? n * sizeof(lbk::Lat<double>) : n * sizeof(lbk::Lat<float>);
     const void *lat_src = e->precision == LB_FP64 ? (const void *)e->L64.data() : (const void *)e->L32.data();
+    size_t n_rec = e->tiles.size(), fold_at = 0;
+    for (int l = 0; l < n && !fold_at; ++l)
+        if (e->tile_end(l) - e->tile_begin(l) > lbk::kFoldTiles) {
+            fold_at = n_rec;
+            n_rec += (size_t)n * lbk::kFold;
+        }
     if (cudaMalloc(&e->d_lats, lat_bytes) != cudaSuccess ||
         cudaMalloc((void **)&e->d_tiles, e->tiles.size() * sizeof(int4)) != cudaSuccess ||
-        cudaMalloc((void **)&e->d_partials, e->tiles.size() * lbk::kAccStride * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void **)&e->d_partials, n_rec * lbk::kAccStride * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void **)&e->d_obs, (size_t)n * lbk::kObsStride * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(LB_ENOMEM, "cudaMalloc of the descriptors failed"));
     }
-    for (int l = 0; l < n; ++l)
-        if (e->tile_end(l) - e->tile_begin(l) > lbk::kFoldTiles && !e->d_fold &&
-            cudaMalloc((void **)&e->d_fold, (size_t)n * lbk::kFold * lbk::kAccStride * sizeof(double)) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(fail(LB_ENOMEM, "cudaMalloc of the folded partials failed"));
-        }
+    if (fold_at) e->d_fold = e->d_partials + fold_at * lbk::kAccStride;
     // time-step tiles for every supported tile height, and the persistent
     // launch's control block and error word
     if ((ce = e->precision == LB_FP64 ? lbk::Launch<double>::prepare() : lbk::Launch<float>::prepare()) != cudaSuccess)

@@ -82,8 +82,9 @@ __host__ __device__ inline bool tma_box_tile(int nx, int ny, int ty) { return nx
 // that the TMA kernel checks its tile without loading its lattice first.
 constexpr int kTmaBoxMark = 1;
 // Shared-memory opt-in of the TMA kernels on the current device; call once
-// before the first launch_fused_tma, outside stream capture.
-cudaError_t prepare_fused_tma();
+// before the first launch_fused_tma, outside stream capture.  mixed: some list
+// may hold tiles of both kinds.
+cudaError_t prepare_fused_tma(bool mixed);
 // One time step of the FP32 tiles [tile_offset, tile_offset + n_tiles) in
 // one pass, one block per tile, each tile staged by one TMA copy of its
 // population box and one of its reference-density box.  The first n_box tiles

@@ -295,11 +295,11 @@ template <int TYv, bool kMixed>
 int TmaKernel<TYv, kMixed>::grid_wave = 0;
 
 template <int TYv>
-cudaError_t prepare_height_tma()
+cudaError_t prepare_height_tma(bool mixed)
 {
     if constexpr (TYv < 8) {
         const cudaError_t e = TmaKernel<TYv, false>::prepare();
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || !mixed) return e;
     }
     return TmaKernel<TYv, true>::prepare();
 }
@@ -316,11 +316,11 @@ cudaError_t launch_height_tma(const Lat<float> *lats, const int4 *tiles, int til
 
 }  // namespace
 
-cudaError_t prepare_fused_tma()
+cudaError_t prepare_fused_tma(bool mixed)
 {
-    cudaError_t e = prepare_height_tma<2>();
-    if (e == cudaSuccess) e = prepare_height_tma<4>();
-    if (e == cudaSuccess) e = prepare_height_tma<8>();
+    cudaError_t e = prepare_height_tma<2>(mixed);
+    if (e == cudaSuccess) e = prepare_height_tma<4>(mixed);
+    if (e == cudaSuccess) e = prepare_height_tma<8>(mixed);
     return e;
 }
 
