@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 2) k3_collide(const Lat3<real> L, in
 // the pushes of its own plane, whose populations it reads a second time out
 // of L2.  A step is one launch; the density pass and collide kernel before it
 // moved 160 bytes a node more and formed the stencils once per species and as
-// two sums each, 3021 instructions a node against 1606 here.  160^3: 660 us a
+// two sums each, 3021 instructions a node against 1592 here.  160^3: 660 us a
 // step before, 421 now; 64^3: 50 and 37.  What bounds it is latency at 16 warps
 // per SM (39 % of the issue slots, 42 % of HBM): three blocks of 80 registers
 // spill (566 us); the populations by cp.async into shared memory a plane ahead
