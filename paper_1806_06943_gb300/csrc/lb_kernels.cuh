@@ -99,6 +99,16 @@ __device__ __forceinline__ int wrap_index(int a, int n)
     return a < 0 ? a + n : a;
 }
 
+// The same for a column of the FP64 step's slots, most of which lie inside: the
+// row kernel takes the shorter code (films of 186 x 8 11.8 us a step, 12.0 with
+// wrap_index).
+__device__ __forceinline__ int wrap_column64(int a, int n)
+{
+    if ((unsigned)a < (unsigned)n) return a;
+    a %= n;
+    return a < 0 ? a + n : a;
+}
+
 // Stage rho_k and psi_k of the tile plus its halo into shared memory from the
 // density copy `rho`.  Periodic copies in x (and in y without walls); beyond a
 // wall the ghost rows are either mirrored from the fluid or set to the fixed
@@ -880,7 +890,8 @@ __device__ __forceinline__ real node_density(const Lat<real> &L, int k, int gx, 
 template <typename real>
 __device__ __forceinline__ bool slot_node(const Lat<real> &G, int4 t, int sx, int sy, int &gx, int &gy)
 {
-    gx = wrap_index(t.y + sx - HALO, G.nx);
+    gx = t.y + sx - HALO;
+    gx = kOffset<real> ? wrap_index(gx, G.nx) : wrap_column64(gx, G.nx);
     gy = t.z + sy - HALO;
     if (gy < 0 || gy >= G.ny) {
         if (!G.walls) {
